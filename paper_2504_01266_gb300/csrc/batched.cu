@@ -116,6 +116,7 @@ giga_status_t build_plan(const giga_image_t* images, int32_t n, int32_t ops, int
     r.x = g.x; r.y = g.y; r.dy = g.dy; r.dx = g.dx; r.w = g.w; r.dw = g.dw;
     r.H = g.H; r.W = g.W; r.C = g.C; r.K = g.K;
     r.vec = vec_image(g, dtype);
+    r.odd_rows = has_odd_rows(dtype == GIGA_BF16 ? 2 : 4, g.W, g.x ? g.x : g.dy, g.x ? g.dy : nullptr);
     const int64_t px = (int64_t)g.H * g.W;
     if (px == 0 || g.C == 0) {
       if ((ops & GIGA_OP_BWD_FILTER) && g.C > 0) plan->empty_filter_grads.push_back(i);

@@ -17,9 +17,11 @@
 //    16-byte aligned, one thread issues a TMA tensor load per tile (the
 //    out-of-image part arrives as zeros: the zero border; under the clamp
 //    border the edge tiles are then fixed in shared memory by clamp_fix);
-//    other inputs are staged by every thread's cp.async copies with the border
-//    rule applied while copying.  Either way the compute loops never branch on
-//    coordinates.  BF16 is widened to FP32 once per staged tile (forward and
+//    other inputs are staged by every thread's cp.async copies (stage_any) to
+//    the same layout.  The kernels are compiled once for each: the aligned one
+//    keeps the registers and instructions that the other spends on staging and
+//    on rows that cannot be stored in whole chunks.  Either way the compute
+//    loops never branch on coordinates.  BF16 is widened to FP32 once per staged tile (forward and
 //    fused backward) or when a row enters registers.  The column halo is
 //    rounded up to 16 bytes of elements so every staged row stays 16-byte
 //    aligned (TMA's rule for the x coordinate).
@@ -48,12 +50,20 @@ __host__ __device__ constexpr int geo_rp(int K, int ES) {
   return ES == 2 ? ((K - 1) / 2 + 7) / 8 * 8 : ((K - 1) / 2 + 3) / 4 * 4;
 }
 
+// Row pitch (elements) of a staged tile.  Tiles staged by stage_any (RAW) may
+// hold a BF16 row one element to the right until shift_odd_rows moves it: the
+// halo's rounding has room for that, or the pitch grows by 16 bytes.
+__host__ __device__ constexpr int geo_pitch(int K, int ES, bool raw) {
+  const int rp = geo_rp(K, ES);
+  return kTileW + 2 * rp + (raw && ES == 2 && rp == (K - 1) / 2 ? 8 : 0);
+}
+
 // Tile geometry of a K x K filter for elements of ES bytes.
-template <int K, int ES = 4>
+template <int K, int ES = 4, bool RAW = false>
 struct Geo {
   static constexpr int R = (K - 1) / 2;
   static constexpr int RP = geo_rp(K, ES);
-  static constexpr int SP = kTileW + 2 * RP;        // staged row pitch (elements)
+  static constexpr int SP = geo_pitch(K, ES, RAW);  // staged row pitch (elements)
   static constexpr int OFF = RP - R;                // first column a lane needs
   static constexpr int OFF4 = OFF / 4 * 4;          // whole 4-element chunks skipped
   static constexpr int OFFR = OFF - OFF4;           // offset inside the first chunk
@@ -108,12 +118,6 @@ __device__ __forceinline__ void cp_async_wait_group() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// Wait for this thread's staging copies, then for the whole CTA.
-__device__ __forceinline__ void stage_wait() {
-  cp_async_wait_all();
-  cta_barrier();
-}
-
 // A 16-byte shared load the compiler may not re-issue: the value must stay
 // in registers (used for filter taps and dy blocks that feed many FMAs).
 __device__ __forceinline__ float4 lds128_pinned(const float* p) {
@@ -131,9 +135,6 @@ template <> struct Tile<float> {
     return *reinterpret_cast<const float4*>(p);
   }
   static __device__ __forceinline__ float4 load4_pinned(const float* p) { return lds128_pinned(p); }
-  static __device__ __forceinline__ void store4(float* p, float4 v) {
-    *reinterpret_cast<float4*>(p) = v;
-  }
 };
 __device__ __forceinline__ float4 bf16x4_to_float4(uint32_t lo, uint32_t hi) {
   return make_float4(__uint_as_float(lo << 16), __uint_as_float(lo & 0xffff0000u),
@@ -150,195 +151,156 @@ template <> struct Tile<__nv_bfloat16> {
                  : "r"(smem_addr(p)));
     return bf16x4_to_float4(lo, hi);
   }
-  // values come from BF16 storage, so the round trip is exact
-  static __device__ __forceinline__ void store4(__nv_bfloat16* p, float4 v) {
-    __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y);
-    __nv_bfloat162 b = __floats2bfloat162_rn(v.z, v.w);
-    uint2 u;
-    u.x = *reinterpret_cast<uint32_t*>(&a);
-    u.y = *reinterpret_cast<uint32_t*>(&b);
-    *reinterpret_cast<uint2*>(p) = u;
-  }
 };
 
-// One staged chunk of 4 consecutive columns at (gi, gj..gj+3), border applied.
-template <typename T>
-__device__ __forceinline__ float4 load_chunk(const T* __restrict__ plane, int H, int W, int gi,
-                                             int gj, bool clamp, bool vec) {
-  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-  bool row_ok = gi >= 0 && gi < H;
-  if (!row_ok && clamp) {
-    gi = gi < 0 ? 0 : H - 1;
-    row_ok = true;
+// ------------------------------------------------ staging of any plane
+// Planes that TMA cannot address (a base or a row stride that is not a
+// multiple of 16 bytes: three of four image widths in FP32, seven of eight in
+// BF16).  A warp takes whole rows of the tile, and consecutive lanes copy
+// consecutive pieces with cp.async, the widest the row's address allows (the
+// same for the whole warp): 16, 8 or 4 bytes.  Every copy instruction reads
+// contiguous bytes and writes different banks, and a row of 128 columns takes
+// one, two or four copies (FP32) and about ten integer instructions; the few
+// columns right of them are copied for all rows together.  What bounds the
+// unaligned passes at small K is the instructions and the load/store slots
+// they take: a lane per 4-element chunk with four 4-byte copies (the former
+// scheme) took about 40 instructions a chunk and touched 16 sectors and a
+// quarter of the banks per copy; 16-byte copies of the row's aligned chunks
+// followed by a shift inside shared memory took about 65 instructions a row.
+// Pixels outside the image arrive as zeros; the clamp border is clamp_fix's.
+// With store_rows, 4 x 3 x 1801 x 2399, zero border, former scheme -> this one
+// (W = 2400, staged by TMA, beside it), us:
+//   FP32 K = 3 forward 112 -> 79 (65), both gradients 204 -> 166 (124),
+//        separable 115 -> 89 (65); K = 7 165 -> 136 (112), 369 -> 304 (243)
+//   BF16 K = 3 forward 135 -> 101 (58), both gradients 293 -> 252 (121),
+//        separable 124 -> 107 (63); K = 7 203 -> 163 (112), 501 -> 447 (274)
+
+// `odd_rows` of the general kernels: some BF16 row of one of the planes starts
+// off a 4-byte boundary, so shift_odd_rows has work.
+inline int has_odd_rows(int es, int64_t W, const void* p, const void* q = nullptr) {
+  const uintptr_t b = reinterpret_cast<uintptr_t>(p) | reinterpret_cast<uintptr_t>(q);
+  return es == 2 && (W % 2 != 0 || b % 4 != 0);
+}
+
+// One 4-byte word of a BF16 row, columns j and j + 1; zeros outside the image.
+__device__ __forceinline__ void stage_bf16_word(uint32_t* dst, const __nv_bfloat16* row, int j,
+                                                int W, bool row_ok) {
+  if (row_ok && j >= 0 && j + 1 < W) {
+    cp_async4(reinterpret_cast<float*>(dst), row + j, true);
+  } else {  // the word crosses an image edge, or is outside
+    const uint16_t* r = reinterpret_cast<const uint16_t*>(row);
+    const uint32_t v0 = row_ok && j >= 0 && j < W ? (uint32_t)r[j] : 0u;
+    const uint32_t v1 = row_ok && j + 1 >= 0 && j + 1 < W ? (uint32_t)r[j + 1] : 0u;
+    *dst = v0 | (v1 << 16);
   }
-  if (row_ok) {
-    const T* src = plane + (int64_t)gi * W;
-    if (vec && gj >= 0 && gj + 3 < W) {
-      v = Elem<T>::load4(src + gj);
-    } else {
-      float e[4];
+}
+
+template <typename T>
+__device__ __forceinline__ int row_is_odd(const T* row) {
+  return sizeof(T) == 2 ? (int)((reinterpret_cast<uintptr_t>(row) >> 1) & 1) : 0;
+}
+
+// rows x pitch elements at `sm`: row sr is image row ty0 - R + sr, element c
+// image column tx0 - RP + c, for c < kTileW + RP + R.  BF16 rows that start off
+// a 4-byte boundary land one element to the right (shift_odd_rows).  Nothing
+// outside the rows is read.  Issues the copies, no commit.
+template <typename T, int NT>
+__device__ __forceinline__ void stage_any(T* __restrict__ sm, const T* plane, int H, int W,
+                                          int ty0, int tx0, int rows, int R, int RP, int pitch,
+                                          int odd_rows) {
+  constexpr int ES = (int)sizeof(T);
+  const int lane = threadIdx.x & 31, w0 = threadIdx.x >> 5;
+  const int j0 = tx0 - RP;  // a multiple of 16 bytes of elements
+  const bool inside = j0 >= 1 && j0 + kTileW <= W;
+  const T* row = plane + (int64_t)(ty0 - R + w0) * W;
+  T* dst = sm + w0 * pitch;
+  for (int sr = w0; sr < rows; sr += NT / 32) {
+    const int gi = ty0 - R + sr;
+    const bool row_ok = gi >= 0 && gi < H;
+    if (inside && row_ok) {
+      const uint32_t a = (uint32_t)reinterpret_cast<uintptr_t>(row) & 15u;
+      if constexpr (ES == 4) {
+        if (a == 0) {
+          cp_async16(dst + 4 * lane, row + j0 + 4 * lane, true);
+        } else if (a == 8) {
+#pragma unroll
+          for (int q = 0; q < 2; ++q)
+            cp_async8(dst + 2 * lane + 64 * q, row + j0 + 2 * lane + 64 * q, true);
+        } else {
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            cp_async4(dst + lane + 32 * q, row + j0 + lane + 32 * q, true);
+        }
+      } else {
+        if ((a & 7) == 0) {
+          cp_async8(dst + 4 * lane, row + j0 + 4 * lane, true);
+        } else {
+          const int p = row_is_odd(row);
+#pragma unroll
+          for (int q = 0; q < 2; ++q)
+            cp_async4(reinterpret_cast<float*>(dst + 2 * lane + 64 * q),
+                      row + j0 - p + 2 * lane + 64 * q, true);
+        }
+      }
+    } else if constexpr (ES == 4) {
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        int j = gj + q;
-        bool ok = j >= 0 && j < W;
-        if (!ok && clamp) {
-          j = j < 0 ? 0 : W - 1;
-          ok = true;
-        }
-        e[q] = ok ? Elem<T>::load(src + j) : 0.f;
-      }
-      v = make_float4(e[0], e[1], e[2], e[3]);
-    }
-  }
-  return v;
-}
-
-// Four consecutive FP32 elements inside an image row whose start is not
-// 16-byte aligned (W not a multiple of 4, or a view): the widest copies the
-// source address allows -- one 16-byte copy on the rows that happen to be
-// aligned, two 8-byte copies on 8-byte boundaries (every row when W = 2 mod 4,
-// half of them when W is odd), else four 4-byte copies.  `dst` is 16-byte
-// aligned.
-__device__ __forceinline__ void stage_chunk_unaligned(float* dst, const float* src) {
-  const uintptr_t a = reinterpret_cast<uintptr_t>(src);
-  if ((a & 15) == 0) {
-    cp_async16(dst, src, true);
-  } else if ((a & 7) == 0) {
-    cp_async8(dst, src, true);
-    cp_async8(dst + 2, src + 2, true);
-  } else {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) cp_async4(dst + q, src + q, true);
-  }
-}
-
-// Stage rows [ty0 - HR, ty0 - HR + rows) x cols [tx0 - HC, tx0 - HC + pitch)
-// of one image plane into shared memory (same element type as the tensor).
-// Outside the image: zero, or (clamp) the nearest edge pixel, row and column
-// clamped independently.  Chunks of 4 elements that lie inside the image on
-// an aligned row are asynchronous cp.async copies (16 bytes FP32, 8 bytes
-// BF16); rows outside a zero border are zero-filled by cp.async; the rest
-// (edges, clamped columns, unaligned rows) go element by element (FP32:
-// 4-byte cp.async; BF16: a plain load and store).  Completion: stage_wait().
-template <typename T, int HR, int HC, int PITCH, int NT = kThreads, bool COMMIT = true>
-__device__ __forceinline__ void stage_tile(T* __restrict__ sm, const T* __restrict__ plane,
-                                           int H, int W, int ty0, int tx0, int rows,
-                                           bool clamp, bool vec) {
-  constexpr int CPR = PITCH / 4;
-  const int total = rows * CPR;
-  for (int k = threadIdx.x; k < total; k += NT) {
-    const int sr = k / CPR;
-    const int sc = (k - sr * CPR) * 4;
-    int gi = ty0 - HR + sr;
-    const int gj = tx0 - HC + sc;
-    T* dst = sm + sr * PITCH + sc;
-    bool row_ok = gi >= 0 && gi < H;
-    if (!row_ok && clamp) {
-      gi = gi < 0 ? 0 : H - 1;
-      row_ok = true;
-    }
-    if constexpr (sizeof(T) == 4) {
-      if (!row_ok) {
-        cp_async16(reinterpret_cast<float*>(dst), plane, false);
-        continue;
-      }
-      const T* src = plane + (int64_t)gi * W;
-      if (vec && gj >= 0 && gj + 3 < W) {
-        cp_async16(reinterpret_cast<float*>(dst), src + gj, true);
-      } else if (gj >= 0 && gj + 3 < W) {
-        stage_chunk_unaligned(reinterpret_cast<float*>(dst), src + gj);
-      } else {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          int j = gj + q;
-          bool ok = j >= 0 && j < W;
-          if (!ok && clamp) {
-            j = j < 0 ? 0 : W - 1;
-            ok = true;
-          }
-          cp_async4(reinterpret_cast<float*>(dst) + q, ok ? src + j : plane, ok);
-        }
+        const int j = j0 + lane + 32 * q;
+        const bool in = row_ok && j >= 0 && j < W;
+        cp_async4(dst + lane + 32 * q, in ? row + j : plane, in);
       }
     } else {
-      if (!row_ok) {
-        cp_async8(dst, plane, false);
-        continue;
-      }
-      const T* src = plane + (int64_t)gi * W;
-      if (vec && gj >= 0 && gj + 3 < W) {
-        cp_async8(dst, src + gj, true);
-      } else if (gj >= 0 && gj + 3 < W &&
-                 (reinterpret_cast<uintptr_t>(src + gj) & 3) == 0) {
-        // interior chunk of a row that is not 8-byte aligned, at a 4-byte
-        // boundary: two 4-byte copies of two elements each
-        cp_async4(reinterpret_cast<float*>(dst), src + gj, true);
-        cp_async4(reinterpret_cast<float*>(dst) + 1, src + gj + 2, true);
-      } else {
-        Tile<T>::store4(dst, load_chunk<T>(plane, H, W, gi, gj, clamp, vec));
-      }
+      const int p = row_is_odd(row);
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+        stage_bf16_word(reinterpret_cast<uint32_t*>(dst) + lane + 32 * q, row,
+                        j0 - p + 2 * (lane + 32 * q), W, row_ok);
+    }
+    row += (int64_t)(NT / 32) * W;
+    dst += NT / 32 * pitch;
+  }
+  // columns kTileW .. kTileW + RP + R - 1 of every row (BF16: whole words, one
+  // more column where rows are to be shifted)
+  const int tail = ES == 4 ? RP + R : (RP + R + (odd_rows ? 2 : 1)) / 2;
+  for (int t = threadIdx.x; t < rows * tail; t += NT) {
+    const int sr = t / tail, k = t - sr * tail;
+    const int gi = ty0 - R + sr;
+    const bool row_ok = gi >= 0 && gi < H;
+    const T* r = plane + (int64_t)(row_ok ? gi : 0) * W;
+    if constexpr (ES == 4) {
+      const int j = j0 + kTileW + k;
+      const bool in = row_ok && j >= 0 && j < W;
+      cp_async4(sm + sr * pitch + kTileW + k, in ? r + j : plane, in);
+    } else {
+      stage_bf16_word(reinterpret_cast<uint32_t*>(sm + sr * pitch + kTileW) + k, r,
+                      j0 + kTileW + 2 * k - row_is_odd(r), W, row_ok);
     }
   }
-  if (COMMIT) cp_async_commit();
 }
 
-// stage_tile with the halo and pitch known only at run time (used where the
-// next tile's filter size is data-dependent); issues the copies, no commit.
+// BF16 rows that stage_any left one element to the right (row addresses that
+// are not multiples of 4: every second row when W is odd) move into place.
+// Every thread calls it once its own copies have landed; it begins with a CTA
+// barrier, and another must follow before the tile is read.
 template <typename T, int NT>
-__device__ __forceinline__ void stage_tile_rt(T* __restrict__ sm, const T* __restrict__ plane,
-                                              int H, int W, int ty0, int tx0, int rows, int HR,
-                                              int HC, int pitch, bool clamp, bool vec) {
-  const int cpr = pitch / 4;
-  const int total = rows * cpr;
-  for (int k = threadIdx.x; k < total; k += NT) {
-    const int sr = k / cpr;
-    const int sc = (k - sr * cpr) * 4;
-    int gi = ty0 - HR + sr;
-    const int gj = tx0 - HC + sc;
-    T* dst = sm + sr * pitch + sc;
-    bool row_ok = gi >= 0 && gi < H;
-    if (!row_ok && clamp) {
-      gi = gi < 0 ? 0 : H - 1;
-      row_ok = true;
-    }
-    if constexpr (sizeof(T) == 4) {
-      if (!row_ok) {
-        cp_async16(reinterpret_cast<float*>(dst), plane, false);
-        continue;
-      }
-      const T* src = plane + (int64_t)gi * W;
-      if (vec && gj >= 0 && gj + 3 < W) {
-        cp_async16(reinterpret_cast<float*>(dst), src + gj, true);
-      } else if (gj >= 0 && gj + 3 < W) {
-        stage_chunk_unaligned(reinterpret_cast<float*>(dst), src + gj);
-      } else {
+__device__ __forceinline__ void shift_odd_rows(T* __restrict__ sm, const T* plane, int H, int W,
+                                               int ty0, int rows, int R, int RP, int pitch) {
+  if constexpr (sizeof(T) == 2) {
+    const int lane = threadIdx.x & 31;
+    const int words = (kTileW + RP + R + 1) / 2;  // at most 80
+    cta_barrier();
+    for (int sr = threadIdx.x >> 5; sr < rows; sr += NT / 32) {
+      const int gi = ty0 - R + sr;
+      if (gi < 0 || gi >= H || !row_is_odd(plane + (int64_t)gi * W)) continue;
+      uint32_t* d = reinterpret_cast<uint32_t*>(sm + sr * pitch) + lane;
+      uint32_t v[3];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          int j = gj + q;
-          bool ok = j >= 0 && j < W;
-          if (!ok && clamp) {
-            j = j < 0 ? 0 : W - 1;
-            ok = true;
-          }
-          cp_async4(reinterpret_cast<float*>(dst) + q, ok ? src + j : plane, ok);
-        }
-      }
-    } else {
-      if (!row_ok) {
-        cp_async8(dst, plane, false);
-        continue;
-      }
-      const T* src = plane + (int64_t)gi * W;
-      if (vec && gj >= 0 && gj + 3 < W) {
-        cp_async8(dst, src + gj, true);
-      } else if (gj >= 0 && gj + 3 < W &&
-                 (reinterpret_cast<uintptr_t>(src + gj) & 3) == 0) {
-        // interior chunk of a row that is not 8-byte aligned, at a 4-byte
-        // boundary: two 4-byte copies of two elements each
-        cp_async4(reinterpret_cast<float*>(dst), src + gj, true);
-        cp_async4(reinterpret_cast<float*>(dst) + 1, src + gj + 2, true);
-      } else {
-        Tile<T>::store4(dst, load_chunk<T>(plane, H, W, gi, gj, clamp, vec));
-      }
+      for (int q = 0; q < 3; ++q)
+        if (lane + 32 * q < words) v[q] = __funnelshift_r(d[32 * q], d[32 * q + 1], 16);
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+        if (lane + 32 * q < words) d[32 * q] = v[q];
     }
   }
 }
@@ -411,13 +373,19 @@ __device__ __forceinline__ void widen_tile(float* __restrict__ dst,
   cta_barrier();
 }
 
-// The halo tile of filter size K (ROWS rows) staged as T, widened if BF16.
-template <int K, typename T, int ROWS>
-using HaloTile = StagedTile<T, ROWS, Geo<K, 4>::SP, Geo<K, sizeof(T)>::SP>;
+// Geometry of the FP32 tile the kernels compute on: the staged one for FP32,
+// the widened one for BF16.
+template <int K, typename T, bool RAW>
+using GeoC = Geo<K, 4, RAW && sizeof(T) == 4>;
 
-template <int K, int ROWS, int NT>
+// The halo tile of filter size K (ROWS rows) staged as T, widened if BF16.
+template <int K, typename T, int ROWS, bool RAW>
+using HaloTile = StagedTile<T, ROWS, GeoC<K, T, RAW>::SP, Geo<K, sizeof(T), RAW>::SP>;
+
+template <int K, int ROWS, int NT, bool RAW>
 __device__ __forceinline__ void widen_halo_tile(float* dst, const __nv_bfloat16* src) {
-  widen_tile<ROWS, Geo<K, 4>::SP, Geo<K, 2>::SP, Geo<K, 2>::RP - Geo<K, 4>::RP, NT>(dst, src);
+  widen_tile<ROWS, Geo<K, 4>::SP, Geo<K, 2, RAW>::SP, Geo<K, 2>::RP - Geo<K, 4>::RP, NT>(dst,
+                                                                                        src);
 }
 
 // Clamp border on a tile that TMA staged with zeros outside the image: tile
@@ -471,35 +439,76 @@ __device__ __forceinline__ void stage_filter_async(float* __restrict__ sm,
   }
 }
 
-// Stage a K x K filter with rows padded to KP (zeros), optionally rotated by
-// 180 degrees (the input gradient's flipped filter).
-template <int K>
-__device__ __forceinline__ void stage_filter(float* __restrict__ sm, const float* __restrict__ w,
-                                             bool flip, int NT) {
-  constexpr int KP = Geo<K>::KP;
-  for (int k = threadIdx.x; k < K * KP; k += NT) {
-    const int a = k / KP, b = k - (k / KP) * KP;
-    sm[k] = b < K ? w[flip ? (K - 1 - a) * K + (K - 1 - b) : a * K + b] : 0.f;
-  }
-}
-
-// Write a lane's PY x 4 block (rows gi0.., columns gj..gj+3) with bounds checks.
+// Write a lane's PY x 4 block (rows gi0.., columns gj..gj+3) of a plane whose
+// rows start on a chunk boundary (16 bytes FP32, 8 BF16; W % 4 == 0).
 template <typename T, int PY>
 __device__ __forceinline__ void store_block(T* __restrict__ plane, int H, int W, int gi0, int gj,
-                                            bool vec, const float (&acc)[PY][4]) {
+                                            const float (&acc)[PY][4]) {
 #pragma unroll
   for (int py = 0; py < PY; ++py) {
     const int gi = gi0 + py;
     if (gi >= H) break;
-    T* dst = plane + (int64_t)gi * W + gj;
-    if (vec && gj + 3 < W) {
-      Elem<T>::store4(dst, make_float4(acc[py][0], acc[py][1], acc[py][2], acc[py][3]));
-    } else {
+    if (gj < W)
+      Elem<T>::store4(plane + (int64_t)gi * W + gj,
+                      make_float4(acc[py][0], acc[py][1], acc[py][2], acc[py][3]));
+  }
+}
+
+// Shared memory of store_rows: one row of kTileW floats per warp.
+constexpr int kRowBuf = kTileW * 4;
+
+// The same for any row alignment; every lane of the warp calls it with the
+// warp's first column tx0 and the warp's own row buffer.  Each row goes
+// through the buffer so that consecutive lanes store consecutive elements
+// (four scalar stores 16 bytes apart between lanes wrote every L2 sector in
+// four pieces; shifting the values between lanes to keep 16-byte stores took
+// about 55 instructions a row, this takes about 15).
+template <typename T, int PY>
+__device__ __forceinline__ void store_rows(T* __restrict__ plane, int H, int W, int gi0, int tx0,
+                                           float* __restrict__ buf, const float (&acc)[PY][4]) {
+  const int lane = threadIdx.x & 31;
+  const int left = W - tx0;  // columns of this tile row inside the image
+#pragma unroll
+  for (int py = 0; py < PY; ++py) {
+    const int gi = gi0 + py;
+    if (gi >= H) break;
+    __syncwarp();  // the previous row has been read
+    *reinterpret_cast<float4*>(buf + 4 * lane) =
+        make_float4(acc[py][0], acc[py][1], acc[py][2], acc[py][3]);
+    __syncwarp();
+    T* row = plane + (int64_t)gi * W + tx0;
+    if constexpr (sizeof(T) == 4) {
 #pragma unroll
       for (int q = 0; q < 4; ++q)
-        if (gj + q < W) Elem<T>::store(dst + q, acc[py][q]);
+        if (lane + 32 * q < left) row[lane + 32 * q] = buf[lane + 32 * q];
+    } else {
+      // pairs on 4-byte boundaries: (0, 1), (2, 3), ... or, when the row starts
+      // off one, 0 alone, then (1, 2), (3, 4), ...
+      const int p = (int)((reinterpret_cast<uintptr_t>(row) >> 1) & 1);
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int c = 2 * (lane + 32 * q) + p;
+        if (c + 1 < kTileW && c + 1 < left)
+          *reinterpret_cast<__nv_bfloat162*>(row + c) =
+              __floats2bfloat162_rn(buf[c], buf[c + 1]);
+        else if (c < kTileW && c < left)
+          Elem<T>::store(row + c, buf[c]);
+      }
+      if (p && lane == 0) Elem<T>::store(row, buf[0]);
     }
   }
+}
+
+// Kernels compiled for aligned planes (AL) always store whole chunks; the
+// others choose per launch.  gj = tx0 + 4 * lane.
+template <typename T, int PY, bool AL>
+__device__ __forceinline__ void store_tile(T* __restrict__ plane, int H, int W, int gi0, int tx0,
+                                           bool vec, float* __restrict__ buf,
+                                           const float (&acc)[PY][4]) {
+  if (AL || vec)
+    store_block<T, PY>(plane, H, W, gi0, tx0 + 4 * (int)(threadIdx.x & 31), acc);
+  else
+    store_rows<T, PY>(plane, H, W, gi0, tx0, buf, acc);
 }
 
 // The window of a lane's 4 output columns: staged columns from the lane's
@@ -521,10 +530,10 @@ __device__ __forceinline__ void load_window_row(const TS* __restrict__ row,
 // acc[py][px] += sum_{s < A, b < K} f[s*KP + b] * win[(py + s) * SP + OFF + px + b]
 // `win` points at the staged row of output row 0 plus filter row 0 of this
 // group, at the lane's first column; `f` at filter row 0 of this group.
-template <int K, int PY, int A, typename TS>
+template <int K, int PY, int A, typename TS, bool RAW>
 __device__ __forceinline__ void fwd_group(const TS* __restrict__ win,
                                           const float* __restrict__ f, float (&acc)[PY][4]) {
-  using G = Geo<K, sizeof(TS)>;
+  using G = Geo<K, sizeof(TS), RAW>;
   float wr[A][G::KP];
 #pragma unroll
   for (int s = 0; s < A; ++s)
@@ -554,21 +563,22 @@ __device__ __forceinline__ void fwd_group(const TS* __restrict__ win,
   }
 }
 
-template <int K, int PY, typename TS>
+template <int K, int PY, typename TS, bool RAW>
 __device__ __forceinline__ void fwd_block(const TS* __restrict__ win,
                                           const float* __restrict__ f, float (&acc)[PY][4]) {
   constexpr int A = fwd_group_rows<K>();
   constexpr int NG = K / A;
   constexpr int REM = K % A;
+  constexpr int SP = Geo<K, sizeof(TS), RAW>::SP;
 #pragma unroll
   for (int py = 0; py < PY; ++py)
 #pragma unroll
     for (int px = 0; px < 4; ++px) acc[py][px] = 0.f;
 #pragma unroll 1
   for (int g = 0; g < NG; ++g)
-    fwd_group<K, PY, A, TS>(win + g * A * Geo<K, sizeof(TS)>::SP, f + g * A * Geo<K>::KP, acc);
+    fwd_group<K, PY, A, TS, RAW>(win + g * A * SP, f + g * A * Geo<K>::KP, acc);
   if constexpr (REM > 0)
-    fwd_group<K, PY, REM, TS>(win + NG * A * Geo<K, sizeof(TS)>::SP, f + NG * A * Geo<K>::KP, acc);
+    fwd_group<K, PY, REM, TS, RAW>(win + NG * A * SP, f + NG * A * Geo<K>::KP, acc);
 }
 
 // Filter gradient of one DR-row dy block for the NR filter rows [a_lo, a_lo + NR):
@@ -578,11 +588,11 @@ __device__ __forceinline__ void fwd_block(const TS* __restrict__ win,
 // compile-time constant: the unrolled body has no data-dependent control flow
 // (with a run-time row count the accumulators live across guarded paths and
 // are copied where those paths merge).
-template <int K, int NR, int AT, int DYP, int DR, typename TS>
+template <int K, int NR, int AT, int DYP, int DR, typename TS, bool RAW>
 __device__ __forceinline__ void dw_block(const TS* __restrict__ dyb,
                                          const TS* __restrict__ xw, float (&acc)[AT][K]) {
   static_assert(NR >= 1 && NR <= AT, "row count");
-  using G = Geo<K, sizeof(TS)>;
+  using G = Geo<K, sizeof(TS), RAW>;
   float d[DR][4];
 #pragma unroll
   for (int py = 0; py < DR; ++py) {
@@ -614,23 +624,23 @@ __device__ __forceinline__ void dw_block(const TS* __restrict__ dyb,
 // `nrows` rows.  Splitting K rows into GT groups gives groups of AT or
 // AT - 1 rows; the branch on the (warp-uniform, fixed) row count is taken
 // once, outside the unrolled bodies.
-template <int K, int AT, int GT, int DYP, int DR, typename TS>
+template <int K, int AT, int GT, int DYP, int DR, typename TS, bool RAW>
 __device__ __forceinline__ void dw_rows(const TS* __restrict__ dyb, const TS* __restrict__ xw,
                                         int nblocks, int nrows, float (&acc)[AT][K]) {
-  constexpr int SP = Geo<K, sizeof(TS)>::SP;
+  constexpr int SP = Geo<K, sizeof(TS), RAW>::SP;
   if constexpr (K % GT == 0) {
 #pragma unroll 1
     for (int i = 0; i < nblocks; ++i)
-      dw_block<K, AT, AT, DYP, DR, TS>(dyb + i * DR * DYP, xw + i * DR * SP, acc);
+      dw_block<K, AT, AT, DYP, DR, TS, RAW>(dyb + i * DR * DYP, xw + i * DR * SP, acc);
   } else {
     if (nrows == AT) {
 #pragma unroll 1
       for (int i = 0; i < nblocks; ++i)
-        dw_block<K, AT, AT, DYP, DR, TS>(dyb + i * DR * DYP, xw + i * DR * SP, acc);
+        dw_block<K, AT, AT, DYP, DR, TS, RAW>(dyb + i * DR * DYP, xw + i * DR * SP, acc);
     } else {
 #pragma unroll 1
       for (int i = 0; i < nblocks; ++i)
-        dw_block<K, AT - 1, AT, DYP, DR, TS>(dyb + i * DR * DYP, xw + i * DR * SP, acc);
+        dw_block<K, AT - 1, AT, DYP, DR, TS, RAW>(dyb + i * DR * DYP, xw + i * DR * SP, acc);
     }
   }
 }
@@ -651,33 +661,39 @@ constexpr int bwd_block_rows() {
 // shared memory: while a tile is computed, the cp.async copies of the next
 // tile and of its plane's filter are in flight.  With flip = 1 the filter is
 // rotated by 180 degrees: that computes g (input gradient, zero border) from dy.
-template <int K, int PY, typename T>
+// AL: input planes a TMA load can address and output rows that start on a
+// chunk boundary; the other compilation stages any plane (stage_any)
+// and stores any row (store_rows).  Apart, the aligned kernel carries neither
+// the code nor the registers of the general one.
+template <int K, int PY, typename T, bool AL>
 struct FwdShape {
-  using G = Geo<K>;  // FP32 compute geometry
+  using G = GeoC<K, T, !AL>;  // FP32 compute geometry
   static constexpr int TH = kWarps * PY;
   static constexpr int ROWS = TH + 2 * G::R;
-  using ST = HaloTile<K, T, ROWS>;
+  using ST = HaloTile<K, T, ROWS, !AL>;
   static constexpr int W_OFF = ST::BYTES;  // FP32 tile (128-aligned), then the filter
   static constexpr int STAGE_BYTES = round_up(W_OFF + G::WPAD * 4, 128);
-  static constexpr int HEAD = 128;  // two mbarriers and the abort flag
+  // two mbarriers and the abort flag, then the row buffers of store_rows
+  static constexpr int HEAD = 128 + (AL ? 0 : kWarps * kRowBuf);
   static constexpr int SM_BYTES = HEAD + 2 * STAGE_BYTES;
   static constexpr int SM_BYTES_1 = HEAD + STAGE_BYTES;  // one tile per CTA
 };
 
-template <typename T, int K, int PY>
+template <typename T, int K, int PY, bool AL>
 __device__ __forceinline__ void dw_fwd_body(
     const CUtensorMap& tmx, const T* __restrict__ x, const float* __restrict__ w,
     T* __restrict__ y, FastDiv fc, int H, int W, FastDiv ftx, FastDiv fty, int64_t num_tiles,
-    int clamp, int vec, int flip, int use_tma, int64_t pf, int* err) {
-  using G = Geo<K>;
-  using GS = Geo<K, sizeof(T)>;
-  using S = FwdShape<K, PY, T>;
+    int clamp, int vec, int odd_rows, int flip, int64_t pf, int* err) {
+  using S = FwdShape<K, PY, T, AL>;
+  using G = typename S::G;
+  using GS = Geo<K, sizeof(T), !AL>;
   using ST = typename S::ST;
   constexpr int TH = S::TH;
   extern __shared__ __align__(128) float smem[];
   char* sm = reinterpret_cast<char*>(smem);
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm);
   volatile int* s_abort = reinterpret_cast<volatile int*>(sm + 16);
+  float* row_buf = reinterpret_cast<float*>(sm + 128 + (threadIdx.x >> 5) * kRowBuf);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   // tile t (< 2^31) -> column and row of the tile, plane (n * C + c)
@@ -697,7 +713,7 @@ __device__ __forceinline__ void dw_fwd_body(
     float* sw = reinterpret_cast<float*>(buf + S::W_OFF);
     const int c = plane - (int)(fdiv((uint32_t)plane, fc) * fc.d);
     stage_filter_async<K>(sw, w + (int64_t)c * K * K, flip != 0, kThreads);
-    if (use_tma) {
+    if constexpr (AL) {
       cp_async_commit();
       if (threadIdx.x == 0) {
         fence_proxy_async();
@@ -705,8 +721,9 @@ __device__ __forceinline__ void dw_fwd_body(
         tma_load_3d(staged, &tmx, tx0 - GS::RP, ty0 - G::R, plane, bars + sb);
       }
     } else {
-      stage_tile<T, G::R, GS::RP, GS::SP>(staged, x + (int64_t)plane * H * W, H, W, ty0, tx0,
-                                          S::ROWS, clamp != 0, vec != 0);
+      stage_any<T, kThreads>(staged, x + (int64_t)plane * H * W, H, W, ty0, tx0, S::ROWS, G::R,
+                             GS::RP, GS::SP, odd_rows);
+      cp_async_commit();
     }
   };
 
@@ -725,7 +742,7 @@ __device__ __forceinline__ void dw_fwd_body(
   for (; t < num_tiles; t += gridDim.x, sb ^= 1) {
     // L2 prefetch of the tile this CTA's successor (one tile per CTA) or this
     // CTA two tiles on (persistent) will load: its TMA load then hits L2
-    if (use_tma && pf > 0 && threadIdx.x == 0 && t + pf < num_tiles) {
+    if (AL && pf > 0 && threadIdx.x == 0 && t + pf < num_tiles) {
       int py0, px0, pplane;
       coords(t + pf, py0, px0, pplane);
       tma_prefetch_3d(&tmx, px0 - GS::RP, py0 - G::R, pplane);
@@ -737,45 +754,49 @@ __device__ __forceinline__ void dw_fwd_body(
     } else {
       cp_async_wait_group<0>();
     }
-    if (use_tma) {
+    int ty0, tx0, plane;
+    coords(t, ty0, tx0, plane);
+    char* buf = sm + S::HEAD + sb * S::STAGE_BYTES;
+    if constexpr (AL) {
       if (!mbar_wait(bars + sb, (phase >> sb) & 1u)) {
         record_error(err, kDevErrTimeout);
         *s_abort = 1;
       }
       phase ^= 1u << sb;
+    } else if (odd_rows) {
+      shift_odd_rows<T, kThreads>(reinterpret_cast<T*>(buf + ST::STAGE_OFF),
+                                  x + (int64_t)plane * H * W, H, W, ty0, S::ROWS, G::R, GS::RP,
+                                  GS::SP);
     }
     cta_barrier();
-    if (*s_abort) break;
-    int ty0, tx0, plane;
-    coords(t, ty0, tx0, plane);
-    char* buf = sm + S::HEAD + sb * S::STAGE_BYTES;
+    if (AL && *s_abort) break;
     float* sx = reinterpret_cast<float*>(buf);
     const float* sw = reinterpret_cast<const float*>(buf + S::W_OFF);
     if constexpr (sizeof(T) == 2)
-      widen_halo_tile<K, S::ROWS, kThreads>(
+      widen_halo_tile<K, S::ROWS, kThreads, !AL>(
           sx, reinterpret_cast<const __nv_bfloat16*>(buf + ST::STAGE_OFF));
-    if (use_tma && clamp &&
+    if (clamp &&
         (ty0 - G::R < 0 || ty0 + TH + G::R > H || tx0 - G::RP < 0 || tx0 + kTileW + G::RP > W))
       clamp_fix<float, G::SP, kThreads>(sx, H, W, ty0, tx0, G::R, G::RP, S::ROWS);
     float acc[PY][4];
-    fwd_block<K, PY, float>(sx + warp * PY * G::SP + 4 * lane, sw, acc);
-    store_block<T, PY>(y + (int64_t)plane * H * W, H, W, ty0 + warp * PY, tx0 + 4 * lane,
-                       vec != 0, acc);
+    fwd_block<K, PY, float, !AL && sizeof(T) == 4>(sx + warp * PY * G::SP + 4 * lane, sw, acc);
+    store_tile<T, PY, AL>(y + (int64_t)plane * H * W, H, W, ty0 + warp * PY, tx0, vec != 0,
+                          row_buf, acc);
     cta_barrier();  // every warp is done with stage sb before it is refilled
   }
   cp_async_wait_group<0>();
   // after an abort: let a TMA load still in flight land (bounded) before exiting
-  if (*s_abort && use_tma && t + gridDim.x < num_tiles)
+  if (AL && *s_abort && t + gridDim.x < num_tiles)
     mbar_wait(bars + (sb ^ 1), (phase >> (sb ^ 1)) & 1u);
 }
 
-template <typename T, int K, int PY>
+template <typename T, int K, int PY, bool AL>
 __global__ void __launch_bounds__(kThreads) dw_fwd_kernel(
     const __grid_constant__ CUtensorMap tmx, const T* __restrict__ x, const float* __restrict__ w,
     T* __restrict__ y, FastDiv fc, int H, int W, FastDiv ftx, FastDiv fty, int64_t num_tiles,
-    int clamp, int vec, int flip, int use_tma, int64_t pf, int* err) {
-  dw_fwd_body<T, K, PY>(tmx, x, w, y, fc, H, W, ftx, fty, num_tiles, clamp, vec, flip, use_tma,
-                        pf, err);
+    int clamp, int vec, int odd_rows, int flip, int64_t pf, int* err) {
+  dw_fwd_body<T, K, PY, AL>(tmx, x, w, y, fc, H, W, ftx, fty, num_tiles, clamp, vec, odd_rows, flip,
+                            pf, err);
 }
 
 // The same pass compiled for five CTAs per SM (at most 51 registers).  Used
@@ -783,13 +804,13 @@ __global__ void __launch_bounds__(kThreads) dw_fwd_kernel(
 // of shared memory and the extra CTA per SM hides more of each CTA's tile
 // load; other sizes keep the default allocation (with this bound K = 3 and 15
 // lose registers they need).
-template <typename T, int K, int PY>
+template <typename T, int K, int PY, bool AL>
 __global__ void __launch_bounds__(kThreads, 5) dw_fwd_kernel_hi_occ(
     const __grid_constant__ CUtensorMap tmx, const T* __restrict__ x, const float* __restrict__ w,
     T* __restrict__ y, FastDiv fc, int H, int W, FastDiv ftx, FastDiv fty, int64_t num_tiles,
-    int clamp, int vec, int flip, int use_tma, int64_t pf, int* err) {
-  dw_fwd_body<T, K, PY>(tmx, x, w, y, fc, H, W, ftx, fty, num_tiles, clamp, vec, flip, use_tma,
-                        pf, err);
+    int clamp, int vec, int odd_rows, int flip, int64_t pf, int* err) {
+  dw_fwd_body<T, K, PY, AL>(tmx, x, w, y, fc, H, W, ftx, fty, num_tiles, clamp, vec, odd_rows, flip,
+                            pf, err);
 }
 
 // ------------------------------------------------------ separable filter
@@ -801,25 +822,25 @@ __global__ void __launch_bounds__(kThreads, 5) dw_fwd_kernel_hi_occ(
 // widened); the row pass writes t over the first 128 columns of the same
 // staged row (a warp owns whole rows and reads a row completely before it
 // writes it), then the column pass runs down t in 8-row register blocks.
-template <int K, typename T>
+template <int K, typename T, bool AL>
 struct SepShape {
-  using G = Geo<K>;
+  using G = GeoC<K, T, !AL>;
   static constexpr int TH = 64;
   static constexpr int ROWS = TH + 2 * G::R;
-  using ST = HaloTile<K, T, ROWS>;
-  static constexpr int HEAD = 128;  // mbarrier, abort flag
+  using ST = HaloTile<K, T, ROWS, !AL>;
+  static constexpr int HEAD = 128 + (AL ? 0 : kWarps * kRowBuf);  // mbarrier, abort flag; row buffers
   static constexpr int W_OFF = HEAD + ST::BYTES;  // wrow then wcol, K floats each (padded)
   static constexpr int SM_BYTES = W_OFF + 2 * round_up(K, 4) * 4;
 };
 
-template <typename T, int K>
+template <typename T, int K, bool AL>
 __device__ __forceinline__ void dw_sep_body(
     const CUtensorMap& tmx, const T* __restrict__ x, const float* __restrict__ wcol,
     const float* __restrict__ wrow, T* __restrict__ y, FastDiv fc, int H, int W, FastDiv ftx,
-    FastDiv fty, int clamp, int vec, int use_tma, int pf, int* err) {
-  using G = Geo<K>;
-  using GS = Geo<K, sizeof(T)>;
-  using S = SepShape<K, T>;
+    FastDiv fty, int clamp, int vec, int odd_rows, int pf, int* err) {
+  using S = SepShape<K, T, AL>;
+  using G = typename S::G;
+  using GS = Geo<K, sizeof(T), !AL>;
   using ST = typename S::ST;
   constexpr int KP = round_up(K, 4);
   extern __shared__ __align__(128) float smem[];
@@ -850,7 +871,7 @@ __device__ __forceinline__ void dw_sep_body(
   }
   cta_barrier();
   T* staged = reinterpret_cast<T*>(sm + S::HEAD + ST::STAGE_OFF);
-  if (use_tma) {
+  if constexpr (AL) {
     cp_async_commit();
     if (threadIdx.x == 0) {
       fence_proxy_async();
@@ -870,18 +891,20 @@ __device__ __forceinline__ void dw_sep_body(
       *s_abort = 1;
     }
   } else {
-    stage_tile<T, G::R, GS::RP, GS::SP>(staged, x + (int64_t)plane * H * W, H, W, ty0, tx0,
-                                        S::ROWS, clamp != 0, vec != 0);
+    const T* xp = x + (int64_t)plane * H * W;
+    stage_any<T, kThreads>(staged, xp, H, W, ty0, tx0, S::ROWS, G::R, GS::RP, GS::SP, odd_rows);
     cp_async_wait_all();
+    if (odd_rows)
+      shift_odd_rows<T, kThreads>(staged, xp, H, W, ty0, S::ROWS, G::R, GS::RP, GS::SP);
   }
   cta_barrier();
-  if (*s_abort) {
+  if (AL && *s_abort) {
     mbar_wait(bar, 0);  // let a late copy land (bounded) before the CTA exits
     return;
   }
   if constexpr (sizeof(T) == 2)
-    widen_halo_tile<K, S::ROWS, kThreads>(st, reinterpret_cast<const __nv_bfloat16*>(staged));
-  if (use_tma && clamp &&
+    widen_halo_tile<K, S::ROWS, kThreads, !AL>(st, reinterpret_cast<const __nv_bfloat16*>(staged));
+  if (clamp &&
       (ty0 - G::R < 0 || ty0 + S::TH + G::R > H || tx0 - G::RP < 0 || tx0 + kTileW + G::RP > W))
     clamp_fix<float, G::SP, kThreads>(st, H, W, ty0, tx0, G::R, G::RP, S::ROWS);
 
@@ -923,28 +946,28 @@ __device__ __forceinline__ void dw_sep_body(
       }
     }
   }
-  store_block<T, PY>(y + (int64_t)plane * H * W, H, W, ty0 + warp * PY, tx0 + 4 * lane,
-                     vec != 0, acc);
+  store_tile<T, PY, AL>(y + (int64_t)plane * H * W, H, W, ty0 + warp * PY, tx0, vec != 0,
+                        reinterpret_cast<float*>(sm + 128 + warp * kRowBuf), acc);
 }
 
-template <typename T, int K>
+template <typename T, int K, bool AL>
 __global__ void __launch_bounds__(kThreads) dw_sep_kernel(
     const __grid_constant__ CUtensorMap tmx, const T* __restrict__ x,
     const float* __restrict__ wcol, const float* __restrict__ wrow, T* __restrict__ y, FastDiv fc,
-    int H, int W, FastDiv ftx, FastDiv fty, int clamp, int vec, int use_tma, int pf, int* err) {
-  dw_sep_body<T, K>(tmx, x, wcol, wrow, y, fc, H, W, ftx, fty, clamp, vec, use_tma, pf, err);
+    int H, int W, FastDiv ftx, FastDiv fty, int clamp, int vec, int odd_rows, int pf, int* err) {
+  dw_sep_body<T, K, AL>(tmx, x, wcol, wrow, y, fc, H, W, ftx, fty, clamp, vec, odd_rows, pf, err);
 }
 
 // The same pass compiled for five CTAs per SM (48 registers): used for FP32
 // K = 13 and 15, whose tiles (44 KB) still fit five times in shared memory and
 // whose pass waits on its tile loads (K = 15: 0.701 -> 0.689 ms on
 // 8 x 3 x 4096^2); smaller K run near the HBM rate with the default allocation.
-template <typename T, int K>
+template <typename T, int K, bool AL>
 __global__ void __launch_bounds__(kThreads, 5) dw_sep_kernel_hi_occ(
     const __grid_constant__ CUtensorMap tmx, const T* __restrict__ x,
     const float* __restrict__ wcol, const float* __restrict__ wrow, T* __restrict__ y, FastDiv fc,
-    int H, int W, FastDiv ftx, FastDiv fty, int clamp, int vec, int use_tma, int pf, int* err) {
-  dw_sep_body<T, K>(tmx, x, wcol, wrow, y, fc, H, W, ftx, fty, clamp, vec, use_tma, pf, err);
+    int H, int W, FastDiv ftx, FastDiv fty, int clamp, int vec, int odd_rows, int pf, int* err) {
+  dw_sep_body<T, K, AL>(tmx, x, wcol, wrow, y, fc, H, W, ftx, fty, clamp, vec, odd_rows, pf, err);
 }
 
 // -------------------------------------------------------------- backward
@@ -955,9 +978,9 @@ __global__ void __launch_bounds__(kThreads, 5) dw_sep_kernel_hi_occ(
 // stride are staged by two TMA loads per tile (zeros outside the image; under
 // the clamp border the x tile of an edge tile then gets clamp_fix), others by
 // cp.async with the border applied.
-template <int K, typename T>
+template <int K, typename T, bool AL>
 struct BwdShape {
-  using G = Geo<K>;  // FP32 compute geometry
+  using G = GeoC<K, T, !AL>;  // FP32 compute geometry
   static constexpr int NDX = 4;
   static constexpr int NDW = kWarps - NDX;
   static constexpr int GT = dw_groups<K>();
@@ -965,11 +988,11 @@ struct BwdShape {
   static constexpr int AT = (K + GT - 1) / GT;      // max filter rows per group
   static constexpr int DW_ROWS = kBwdTileH / WPG;   // tile rows per dw warp
   static constexpr int ROWS = kBwdTileH + 2 * G::R;  // x and dy tiles, both with the halo
-  using ST = HaloTile<K, T, ROWS>;
+  using ST = HaloTile<K, T, ROWS, !AL>;
   // byte offsets: mbarrier and abort flag, the FP32 x and dy tiles (staged
   // tiles at ST::STAGE_OFF inside them, 128-byte aligned for TMA), flipped
   // filter and reduction
-  static constexpr int SM_X = 128;
+  static constexpr int SM_X = 128 + (AL ? 0 : NDX * kRowBuf);  // row buffers of the dx warps
   static constexpr int SM_DY = SM_X + ST::BYTES;
   static constexpr int SM_W = SM_DY + ST::BYTES;
   // the warps' filter-gradient sums are written after every warp has left the
@@ -986,22 +1009,23 @@ __device__ __forceinline__ int group_lo(int g, int K, int GT) { return g * K / G
 
 // CTAs per SM the backward kernel is compiled for: the small-K instances are
 // memory-bound and need fewer registers, so a third CTA adds loads in flight.
-template <typename T, int K>
+// (The general FP32 K = 7 kernel's row buffers leave room for two.)
+template <typename T, int K, bool AL>
 constexpr int bwd_min_ctas() {
-  return (K <= 5 || (K == 7 && sizeof(T) == 4)) ? 3 : 2;
+  return (K <= 5 || (AL && K == 7 && sizeof(T) == 4)) ? 3 : 2;
 }
 
-template <typename T, int K>
-__global__ void __launch_bounds__(kThreads, bwd_min_ctas<T, K>())
+template <typename T, int K, bool AL>
+__global__ void __launch_bounds__(kThreads, bwd_min_ctas<T, K, AL>())
     dw_bwd_kernel(const __grid_constant__ CUtensorMap tmx,
                   const __grid_constant__ CUtensorMap tmdy, const T* __restrict__ x,
                   const T* __restrict__ dy, const float* __restrict__ w, T* __restrict__ dx,
                   float* __restrict__ partials, int C, int H, int W, int tiles_x,
                   int tiles_per_plane, int chunks_per_plane, int tpc, int clamp, int vec,
-                  int use_tma, int* err) {
-  using G = Geo<K>;
-  using GS = Geo<K, sizeof(T)>;
-  using S = BwdShape<K, T>;
+                  int odd_rows, int* err) {
+  using S = BwdShape<K, T, AL>;
+  using G = typename S::G;
+  using GS = Geo<K, sizeof(T), !AL>;
   using ST = typename S::ST;
   extern __shared__ __align__(128) float smem[];
   char* sm = reinterpret_cast<char*>(smem);
@@ -1035,7 +1059,7 @@ __global__ void __launch_bounds__(kThreads, bwd_min_ctas<T, K>())
   // false if a TMA wait gave up (every thread then leaves its tile loop).
   auto stage = [&](int ty0, int tx0) -> bool {
     cta_barrier();
-    if (use_tma) {
+    if constexpr (AL) {
       cp_async_commit();
       if (threadIdx.x == 0) {
         fence_proxy_async();
@@ -1053,17 +1077,20 @@ __global__ void __launch_bounds__(kThreads, bwd_min_ctas<T, K>())
       cta_barrier();
       if (*s_abort) return false;
     } else {
-      stage_tile<T, G::R, GS::RP, GS::SP>(st_x, xp, H, W, ty0, tx0, S::ROWS, clamp != 0,
-                                          vec != 0);
-      stage_tile<T, G::R, GS::RP, GS::SP>(st_dy, dyp, H, W, ty0, tx0, S::ROWS, false,
-                                          vec != 0);
-      stage_wait();
+      stage_any<T, kThreads>(st_x, xp, H, W, ty0, tx0, S::ROWS, G::R, GS::RP, GS::SP, odd_rows);
+      stage_any<T, kThreads>(st_dy, dyp, H, W, ty0, tx0, S::ROWS, G::R, GS::RP, GS::SP, odd_rows);
+      cp_async_wait_all();
+      if (odd_rows) {
+        shift_odd_rows<T, kThreads>(st_x, xp, H, W, ty0, S::ROWS, G::R, GS::RP, GS::SP);
+        shift_odd_rows<T, kThreads>(st_dy, dyp, H, W, ty0, S::ROWS, G::R, GS::RP, GS::SP);
+      }
+      cta_barrier();
     }
     if constexpr (sizeof(T) == 2) {
-      widen_halo_tile<K, S::ROWS, kThreads>(sm_x, reinterpret_cast<const __nv_bfloat16*>(st_x));
-      widen_halo_tile<K, S::ROWS, kThreads>(sm_dy, reinterpret_cast<const __nv_bfloat16*>(st_dy));
+      widen_halo_tile<K, S::ROWS, kThreads, !AL>(sm_x, reinterpret_cast<const __nv_bfloat16*>(st_x));
+      widen_halo_tile<K, S::ROWS, kThreads, !AL>(sm_dy, reinterpret_cast<const __nv_bfloat16*>(st_dy));
     }
-    if (use_tma && clamp &&
+    if (clamp &&
         (ty0 - G::R < 0 || ty0 + kBwdTileH + G::R > H || tx0 - G::RP < 0 ||
          tx0 + kTileW + G::RP > W))
       clamp_fix<float, G::SP, kThreads>(sm_x, H, W, ty0, tx0, G::R, G::RP, S::ROWS);
@@ -1082,8 +1109,9 @@ __global__ void __launch_bounds__(kThreads, bwd_min_ctas<T, K>())
       for (int pass = 0; pass < 16 / BR; ++pass) {
         const int r0 = warp * 16 + pass * BR;
         float acc[BR][4];
-        fwd_block<K, BR, float>(sm_dy + r0 * G::SP + 4 * lane, sm_w, acc);
-        store_block<T, BR>(dx + plane_off, H, W, ty0 + r0, tx0 + 4 * lane, vec != 0, acc);
+        fwd_block<K, BR, float, !AL && sizeof(T) == 4>(sm_dy + r0 * G::SP + 4 * lane, sm_w, acc);
+        store_tile<T, BR, AL>(dx + plane_off, H, W, ty0 + r0, tx0, vec != 0,
+                              reinterpret_cast<float*>(sm + 128 + warp * kRowBuf), acc);
       }
     }
     cta_barrier();
@@ -1105,9 +1133,9 @@ __global__ void __launch_bounds__(kThreads, bwd_min_ctas<T, K>())
       if (!stage(ty0, tx0)) break;
       constexpr int BR = bwd_block_rows<K>();
       const int r0 = part * S::DW_ROWS;
-      dw_rows<K, S::AT, S::GT, G::SP, BR, float>(sm_dy + (r0 + G::R) * G::SP + G::RP + 4 * lane,
-                                             sm_x + (r0 + a_lo) * G::SP + 4 * lane,
-                                             S::DW_ROWS / BR, nrows, acc);
+      dw_rows<K, S::AT, S::GT, G::SP, BR, float, !AL && sizeof(T) == 4>(
+          sm_dy + (r0 + G::R) * G::SP + G::RP + 4 * lane, sm_x + (r0 + a_lo) * G::SP + 4 * lane,
+          S::DW_ROWS / BR, nrows, acc);
     }
     // warp reduction (fixed butterfly order), one row of sm_red per warp
     cta_barrier();
@@ -1133,7 +1161,7 @@ __global__ void __launch_bounds__(kThreads, bwd_min_ctas<T, K>())
     partials[(int64_t)blockIdx.x * K * K + k] = sum;
   }
   cp_async_wait_all();
-  if (*s_abort && use_tma) mbar_wait(bar, phase);  // let a late TMA load land (bounded)
+  if (AL && *s_abort) mbar_wait(bar, phase);  // let a late TMA load land (bounded)
 }
 
 // ------------------------------------------------------- filter gradient
@@ -1168,9 +1196,10 @@ constexpr int filter_groups() {
   return (K == 9 || K == 15) ? 3 : dw_groups<K>();
 }
 
-template <int K, typename T>
+template <int K, typename T, bool AL>
 struct FilterShape {
-  using G = Geo<K, sizeof(T)>;  // tiles stay in the storage type (no widening pass)
+  using G = Geo<K, sizeof(T), !AL>;  // tiles stay in the storage type (no widening pass)
+  static constexpr int DYP = geo_pitch(1, sizeof(T), !AL);  // dy tile pitch (no halo)
   static constexpr int NW = filter_warps<K>();
   static constexpr int NT = NW * 32;
   static constexpr int GT = filter_groups<K>();
@@ -1180,7 +1209,7 @@ struct FilterShape {
   static constexpr int DR = 4;                     // dy rows per unrolled block
   static constexpr int X_ROWS = kFilterTileH + 2 * G::R;
   static constexpr int X_BYTES = X_ROWS * G::SP * (int)sizeof(T);
-  static constexpr int DY_BYTES = kFilterTileH * kTileW * (int)sizeof(T);
+  static constexpr int DY_BYTES = kFilterTileH * DYP * (int)sizeof(T);
   static constexpr int DY_OFF = round_up(X_BYTES, 128);  // TMA destinations: 128-byte aligned
   static constexpr int STAGE_BYTES = round_up(DY_OFF + DY_BYTES, 128);
   static constexpr int NS = K <= 9 ? 3 : 2;
@@ -1191,15 +1220,15 @@ struct FilterShape {
   static_assert(SM_BYTES <= 227 * 1024, "shared memory");
 };
 
-template <typename T, int K>
-__global__ void __launch_bounds__(FilterShape<K, T>::NT, 1)
+template <typename T, int K, bool AL>
+__global__ void __launch_bounds__(FilterShape<K, T, AL>::NT, 1)
     dw_filter_kernel(const __grid_constant__ CUtensorMap tmx,
                      const __grid_constant__ CUtensorMap tmdy, const T* __restrict__ x,
                      const T* __restrict__ dy, float* __restrict__ partials, int H, int W,
                      FastDiv ftx, int tiles_per_plane, FastDiv fcpp, int tpc, int num_chunks,
-                     int clamp, int vec, int use_tma, int* err) {
-  using G = Geo<K, sizeof(T)>;
-  using S = FilterShape<K, T>;
+                     int clamp, int odd_rows, int* err) {
+  using S = FilterShape<K, T, AL>;
+  using G = typename S::G;
   extern __shared__ __align__(128) float smem[];
   char* sm = reinterpret_cast<char*>(smem);
   float* sm_red = reinterpret_cast<float*>(sm + S::SM_RED);
@@ -1246,7 +1275,7 @@ __global__ void __launch_bounds__(FilterShape<K, T>::NT, 1)
     tile_origin(it.t, ty0, tx0);
     T* sx = reinterpret_cast<T*>(sm + sb * S::STAGE_BYTES);
     T* sdy = reinterpret_cast<T*>(sm + sb * S::STAGE_BYTES + S::DY_OFF);
-    if (use_tma) {
+    if constexpr (AL) {
       if (threadIdx.x == 0) {
         fence_proxy_async();
         mbar_expect_tx(bars + sb, (uint32_t)(S::X_BYTES + S::DY_BYTES));
@@ -1255,10 +1284,8 @@ __global__ void __launch_bounds__(FilterShape<K, T>::NT, 1)
       }
     } else {
       const int64_t off = (int64_t)plane * H * W;
-      stage_tile<T, G::R, G::RP, G::SP, S::NT, false>(sx, x + off, H, W, ty0, tx0, S::X_ROWS,
-                                                      clamp != 0, vec != 0);
-      stage_tile<T, 0, 0, kTileW, S::NT, false>(sdy, dy + off, H, W, ty0, tx0, kFilterTileH,
-                                                false, vec != 0);
+      stage_any<T, S::NT>(sx, x + off, H, W, ty0, tx0, S::X_ROWS, G::R, G::RP, G::SP, odd_rows);
+      stage_any<T, S::NT>(sdy, dy + off, H, W, ty0, tx0, kFilterTileH, 0, 0, S::DYP, odd_rows);
     }
   };
 
@@ -1279,7 +1306,7 @@ __global__ void __launch_bounds__(FilterShape<K, T>::NT, 1)
 #pragma unroll
   for (int i = 0; i < S::NS - 1; ++i) {
     if (pf.q < num_chunks) {
-      if (use_tma) pending |= 1u << i;
+      if (AL) pending |= 1u << i;
       stage(pf, i);
       advance(pf);
     }
@@ -1296,7 +1323,7 @@ __global__ void __launch_bounds__(FilterShape<K, T>::NT, 1)
     // refill the stage released at the end of the previous item
     if (pf.q < num_chunks) {
       const int ps = sb == 0 ? S::NS - 1 : sb - 1;
-      if (use_tma) pending |= 1u << ps;
+      if (AL) pending |= 1u << ps;
       stage(pf, ps);
       advance(pf);
     }
@@ -1310,18 +1337,25 @@ __global__ void __launch_bounds__(FilterShape<K, T>::NT, 1)
       phase ^= 1u << sb;
       pending &= ~(1u << sb);
     }
-    cta_barrier();
-    if (*s_abort) break;
     T* sx = reinterpret_cast<T*>(sm + sb * S::STAGE_BYTES);
-    const T* sdy = reinterpret_cast<const T*>(sm + sb * S::STAGE_BYTES + S::DY_OFF);
-    if (use_tma && clamp && at_edge(cs)) {
+    T* sdy = reinterpret_cast<T*>(sm + sb * S::STAGE_BYTES + S::DY_OFF);
+    if (!AL && odd_rows) {
+      const int64_t off = (int64_t)fdiv((uint32_t)cs.q, fcpp) * H * W;
+      int ty0, tx0;
+      tile_origin(cs.t, ty0, tx0);
+      shift_odd_rows<T, S::NT>(sx, x + off, H, W, ty0, S::X_ROWS, G::R, G::RP, G::SP);
+      shift_odd_rows<T, S::NT>(sdy, dy + off, H, W, ty0, kFilterTileH, 0, 0, S::DYP);
+    }
+    cta_barrier();
+    if (AL && *s_abort) break;
+    if (clamp && at_edge(cs)) {
       int ty0, tx0;
       tile_origin(cs.t, ty0, tx0);
       clamp_fix<T, G::SP, S::NT>(sx, H, W, ty0, tx0, G::R, G::RP, S::X_ROWS);
     }
-    dw_rows<K, S::AT, S::GT, kTileW, S::DR, T>(sdy + part * S::ROWS * kTileW + 4 * lane,
-                                               sx + (part * S::ROWS + a_lo) * G::SP + 4 * lane,
-                                               S::ROWS / S::DR, nrows, acc);
+    dw_rows<K, S::AT, S::GT, S::DYP, S::DR, T, !AL>(
+        sdy + part * S::ROWS * S::DYP + 4 * lane, sx + (part * S::ROWS + a_lo) * G::SP + 4 * lane,
+        S::ROWS / S::DR, nrows, acc);
     const bool chunk_end = cs.t + 1 == cs.t_end;
     if (chunk_end) {
 #pragma unroll
@@ -1352,7 +1386,7 @@ __global__ void __launch_bounds__(FilterShape<K, T>::NT, 1)
   }
   cp_async_wait_group<0>();
   // after an abort: let the TMA loads still in flight land (bounded) before exiting
-  for (int s = 0; s < S::NS; ++s)
+  for (int s = 0; AL && s < S::NS; ++s)
     if (pending & (1u << s)) mbar_wait(bars + s, (phase >> s) & 1u);
 }
 
@@ -1368,9 +1402,9 @@ __global__ void __launch_bounds__(FilterShape<K, T>::NT, 1)
 // tuning candidate for every K.  Tiles stay in the storage type (BF16 rows
 // are widened as they enter registers).  The rotated filter of a chunk's
 // channel goes to one of two buffers (chunk parity), written by the g warps.
-template <int K, typename T>
+template <int K, typename T, bool AL>
 struct RingShape {
-  using G = Geo<K, sizeof(T)>;
+  using G = Geo<K, sizeof(T), !AL>;
   static constexpr int NT = kThreads;
   static constexpr int GT = dw_groups<K>();
   static constexpr int WPG = 4 / GT;
@@ -1381,11 +1415,13 @@ struct RingShape {
   static constexpr int T_BYTES = round_up(ROWS * G::SP * (int)sizeof(T), 128);
   static constexpr int STAGE_BYTES = 2 * T_BYTES;  // x, then dy (both with the halo)
   // three stages where they fit (two tiles in flight while one is computed)
-  static constexpr int NS = 3 * STAGE_BYTES + 2 * Geo<K>::WPAD * 4 + 4 * AT * K * 4 + 64 <=
+  static constexpr int BUFS = AL ? 0 : 4 * kRowBuf;  // row buffers of the dx warps
+  static constexpr int NS = 3 * STAGE_BYTES + 2 * Geo<K>::WPAD * 4 + 4 * AT * K * 4 + BUFS + 64 <=
                                     227 * 1024
                                 ? 3
                                 : 2;
-  static constexpr int SM_W = NS * STAGE_BYTES;
+  static constexpr int SM_BUF = NS * STAGE_BYTES;
+  static constexpr int SM_W = SM_BUF + BUFS;
   static constexpr int SM_RED = SM_W + 2 * Geo<K>::WPAD * 4;
   static constexpr int SM_BAR = round_up(SM_RED + 4 * AT * K * 4, 8);
   static constexpr int SM_BYTES = SM_BAR + NS * 8 + 8;
@@ -1393,16 +1429,16 @@ struct RingShape {
   static_assert(SM_BYTES <= 227 * 1024, "shared memory");
 };
 
-template <typename T, int K>
+template <typename T, int K, bool AL>
 __global__ void __launch_bounds__(kThreads, 1)
     dw_bwd_ring_kernel(const __grid_constant__ CUtensorMap tmx,
                        const __grid_constant__ CUtensorMap tmdy, const T* __restrict__ x,
                        const T* __restrict__ dy, const float* __restrict__ w, T* __restrict__ dx,
                        float* __restrict__ partials, int C, int H, int W, FastDiv ftx,
                        int tiles_per_plane, FastDiv fcpp, int tpc, int num_chunks, int clamp,
-                       int vec, int use_tma, int* err) {
-  using G = Geo<K, sizeof(T)>;
-  using S = RingShape<K, T>;
+                       int vec, int odd_rows, int* err) {
+  using S = RingShape<K, T, AL>;
+  using G = typename S::G;
   constexpr int KP = Geo<K>::KP;
   extern __shared__ __align__(128) float smem[];
   char* sm = reinterpret_cast<char*>(smem);
@@ -1442,7 +1478,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tile_origin(it.t, ty0, tx0);
     T* sx = reinterpret_cast<T*>(sm + sb * S::STAGE_BYTES);
     T* sdy = reinterpret_cast<T*>(sm + sb * S::STAGE_BYTES + S::T_BYTES);
-    if (use_tma) {
+    if constexpr (AL) {
       if (threadIdx.x == 0) {
         fence_proxy_async();
         mbar_expect_tx(bars + sb, (uint32_t)(2 * S::ROWS * G::SP * (int)sizeof(T)));
@@ -1451,10 +1487,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     } else {
       const int64_t off = (int64_t)plane * H * W;
-      stage_tile<T, G::R, G::RP, G::SP, S::NT, false>(sx, x + off, H, W, ty0, tx0, S::ROWS,
-                                                      clamp != 0, vec != 0);
-      stage_tile<T, G::R, G::RP, G::SP, S::NT, false>(sdy, dy + off, H, W, ty0, tx0, S::ROWS,
-                                                      false, vec != 0);
+      stage_any<T, S::NT>(sx, x + off, H, W, ty0, tx0, S::ROWS, G::R, G::RP, G::SP, odd_rows);
+      stage_any<T, S::NT>(sdy, dy + off, H, W, ty0, tx0, S::ROWS, G::R, G::RP, G::SP, odd_rows);
     }
   };
 
@@ -1474,7 +1508,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
   for (int i = 0; i < S::NS - 1; ++i) {
     if (pf.q < num_chunks) {
-      if (use_tma) pending |= 1u << i;
+      if (AL) pending |= 1u << i;
       stage(pf, i);
       advance(pf);
     }
@@ -1493,7 +1527,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // refill the stage released at the end of the previous item
     if (pf.q < num_chunks) {
       const int ps = sb == 0 ? S::NS - 1 : sb - 1;
-      if (use_tma) pending |= 1u << ps;
+      if (AL) pending |= 1u << ps;
       stage(pf, ps);
       advance(pf);
     }
@@ -1518,13 +1552,18 @@ __global__ void __launch_bounds__(kThreads, 1)
       phase ^= 1u << sb;
       pending &= ~(1u << sb);
     }
-    cta_barrier();
-    if (*s_abort) break;
     T* sx = reinterpret_cast<T*>(sm + sb * S::STAGE_BYTES);
-    const T* sdy = reinterpret_cast<const T*>(sm + sb * S::STAGE_BYTES + S::T_BYTES);
+    T* sdy = reinterpret_cast<T*>(sm + sb * S::STAGE_BYTES + S::T_BYTES);
     int ty0, tx0;
     tile_origin(cs.t, ty0, tx0);
-    if (use_tma && clamp &&
+    if (!AL && odd_rows) {
+      const int64_t off = (int64_t)plane * H * W;
+      shift_odd_rows<T, S::NT>(sx, x + off, H, W, ty0, S::ROWS, G::R, G::RP, G::SP);
+      shift_odd_rows<T, S::NT>(sdy, dy + off, H, W, ty0, S::ROWS, G::R, G::RP, G::SP);
+    }
+    cta_barrier();
+    if (AL && *s_abort) break;
+    if (clamp &&
         (ty0 - G::R < 0 || ty0 + kBwdTileH + G::R > H || tx0 - G::RP < 0 ||
          tx0 + kTileW + G::RP > W))
       clamp_fix<T, G::SP, S::NT>(sx, H, W, ty0, tx0, G::R, G::RP, S::ROWS);
@@ -1533,15 +1572,15 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int pass = 0; pass < 16 / S::BR; ++pass) {
         const int r0 = wl * 16 + pass * S::BR;
         float o[S::BR][4];
-        fwd_block<K, S::BR, T>(sdy + r0 * G::SP + 4 * lane, swf, o);
-        store_block<T, S::BR>(dx + (int64_t)plane * H * W, H, W, ty0 + r0, tx0 + 4 * lane,
-                              vec != 0, o);
+        fwd_block<K, S::BR, T, !AL>(sdy + r0 * G::SP + 4 * lane, swf, o);
+        store_tile<T, S::BR, AL>(dx + (int64_t)plane * H * W, H, W, ty0 + r0, tx0, vec != 0,
+                                 reinterpret_cast<float*>(sm + S::SM_BUF + wl * kRowBuf), o);
       }
     } else {
       const int r0 = part * S::DW_ROWS;
-      dw_rows<K, S::AT, S::GT, G::SP, S::BR, T>(sdy + (r0 + G::R) * G::SP + G::RP + 4 * lane,
-                                                sx + (r0 + a_lo) * G::SP + 4 * lane,
-                                                S::DW_ROWS / S::BR, nrows, acc);
+      dw_rows<K, S::AT, S::GT, G::SP, S::BR, T, !AL>(
+          sdy + (r0 + G::R) * G::SP + G::RP + 4 * lane, sx + (r0 + a_lo) * G::SP + 4 * lane,
+          S::DW_ROWS / S::BR, nrows, acc);
     }
     const bool chunk_end = cs.t + 1 == cs.t_end;
     if (chunk_end && dw_warp) {
@@ -1575,7 +1614,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   cp_async_wait_group<0>();
   // after an abort: let the TMA loads still in flight land (bounded) before exiting
-  for (int s = 0; s < S::NS; ++s)
+  for (int s = 0; AL && s < S::NS; ++s)
     if (pending & (1u << s)) mbar_wait(bars + s, (phase >> s) & 1u);
 }
 

@@ -10,32 +10,33 @@
 
 namespace giga {
 
-// persistent = 0 (the default, fastest on the measured workloads): one tile
-// per CTA and a single shared-memory stage (the kernel's prefetch branch never
-// runs because gridDim.x >= tiles); 1: as many CTAs as fit on the GPU, each
-// with two stages -- an autotuning candidate.
 // The forward kernel of a launch: for FP32 K = 7 with one tile per CTA the
 // five-CTA-per-SM compilation (instantiated for that case only), else the
 // default one.  Raises the kernel's shared-memory limit first.
-template <typename T, int K, int PY>
+template <typename T, int K, int PY, bool AL>
 static cudaError_t fwd_kernel_for(bool persistent, size_t smem,
-                                  decltype(&dw_fwd_kernel<T, K, PY>)* kern) {
+                                  decltype(&dw_fwd_kernel<T, K, PY, AL>)* kern) {
   if constexpr (sizeof(T) == 4 && K == 7 && PY == 8) {
     if (!persistent) {
-      *kern = dw_fwd_kernel_hi_occ<T, K, PY>;
-      return set_smem_once<dw_fwd_kernel_hi_occ<T, K, PY>>(smem);
+      *kern = dw_fwd_kernel_hi_occ<T, K, PY, AL>;
+      return set_smem_once<dw_fwd_kernel_hi_occ<T, K, PY, AL>>(smem);
     }
   }
-  *kern = dw_fwd_kernel<T, K, PY>;
-  return set_smem_once<dw_fwd_kernel<T, K, PY>>(smem);
+  *kern = dw_fwd_kernel<T, K, PY, AL>;
+  return set_smem_once<dw_fwd_kernel<T, K, PY, AL>>(smem);
 }
 
-template <typename T, int K, int PY>
-static cudaError_t fwd_impl(const DwArgs& a, bool input_grad, bool persistent, bool prefetch,
-                            cudaStream_t st) {
-  using S = FwdShape<K, PY, T>;
-  decltype(&dw_fwd_kernel<T, K, PY>) kern = nullptr;
-  cudaError_t e = fwd_kernel_for<T, K, PY>(persistent, (size_t)S::SM_BYTES, &kern);
+// persistent = 0 (the default, fastest on the measured workloads): one tile
+// per CTA and a single shared-memory stage (the kernel's prefetch branch never
+// runs because gridDim.x >= tiles); 1: as many CTAs as fit on the GPU, each
+// with two stages -- an autotuning candidate.  AL: the compilation for planes
+// that TMA loads and whole-chunk stores can address (`tm` is their map).
+template <typename T, int K, int PY, bool AL>
+static cudaError_t fwd_run(const DwArgs& a, const CUtensorMap& tm, bool input_grad,
+                           bool persistent, bool prefetch, cudaStream_t st) {
+  using S = FwdShape<K, PY, T, AL>;
+  decltype(&dw_fwd_kernel<T, K, PY, AL>) kern = nullptr;
+  cudaError_t e = fwd_kernel_for<T, K, PY, AL>(persistent, (size_t)S::SM_BYTES, &kern);
   if (e != cudaSuccess) return e;
   const int64_t tiles_x = (a.W + kTileW - 1) / kTileW;
   const int64_t tiles_y = (a.H + S::TH - 1) / S::TH;
@@ -66,19 +67,26 @@ static cudaError_t fwd_impl(const DwArgs& a, bool input_grad, bool persistent, b
   if (tiles > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   const T* in = static_cast<const T*>(input_grad ? a.dy : a.x);
   T* out = static_cast<T*>(input_grad ? a.dx : a.y);
-  // TMA staging for rows with a 16-byte stride from a 16-byte aligned base
-  CUtensorMap tm;
-  std::memset(&tm, 0, sizeof(tm));
-  int use_tma = 0;
-  if (plane_tma_ok(in, sizeof(T), a.W))
-    use_tma = make_plane_map(&tm, in, sizeof(T), a.W, a.H, a.N * a.C, Geo<K, sizeof(T)>::SP,
-                             S::ROWS);
   kern<<<(unsigned)grid, kThreads, smem, st>>>(
       tm, in, a.w, out, make_fastdiv((uint32_t)a.C), (int)a.H, (int)a.W,
       make_fastdiv((uint32_t)tiles_x), make_fastdiv((uint32_t)tiles_y), tiles,
-      input_grad ? 0 : a.border, a.vec, input_grad ? 1 : 0, use_tma, pf, dw_error_word());
+      input_grad ? 0 : a.border, a.vec, has_odd_rows(sizeof(T), a.W, in), input_grad ? 1 : 0,
+      pf, dw_error_word());
   note_launch();
   return cudaGetLastError();
+}
+
+template <typename T, int K, int PY>
+static cudaError_t fwd_impl(const DwArgs& a, bool input_grad, bool persistent, bool prefetch,
+                            cudaStream_t st) {
+  const void* in = input_grad ? a.dy : a.x;
+  CUtensorMap tm;
+  std::memset(&tm, 0, sizeof(tm));
+  if (a.vec && plane_tma_ok(in, sizeof(T), a.W) &&
+      make_plane_map(&tm, in, sizeof(T), a.W, a.H, a.N * a.C, Geo<K, sizeof(T)>::SP,
+                     FwdShape<K, PY, T, true>::ROWS))
+    return fwd_run<T, K, PY, true>(a, tm, input_grad, persistent, prefetch, st);
+  return fwd_run<T, K, PY, false>(a, tm, input_grad, persistent, prefetch, st);
 }
 
 template <int K>
@@ -93,32 +101,49 @@ cudaError_t dw_fwd_launch(const DwArgs& a, const DwConfig& cfg, bool input_grad,
              : fwd_impl<__nv_bfloat16, K, 8>(a, input_grad, pers, pf, st);
 }
 
+// Tensor maps of x and dy for the aligned kernels, boxes of ROWS x SP (dy: of
+// rows_dy x pitch_dy); false: the general kernels run (`vec`: every tensor's
+// rows start on a chunk boundary).
 template <typename T, int K>
-static cudaError_t bwd_impl(const DwArgs& a, const DwConfig& cfg, cudaStream_t st) {
-  using S = BwdShape<K, T>;
+static bool xdy_maps(const DwArgs& a, int rows, int rows_dy, int pitch_dy, CUtensorMap* tmx,
+                     CUtensorMap* tmdy) {
+  constexpr int es = sizeof(T);
+  std::memset(tmx, 0, sizeof(*tmx));
+  std::memset(tmdy, 0, sizeof(*tmdy));
+  return a.vec && plane_tma_ok(a.x, es, a.W) && plane_tma_ok(a.dy, es, a.W) &&
+         make_plane_map(tmx, a.x, es, a.W, a.H, a.N * a.C, Geo<K, es>::SP, rows) &&
+         make_plane_map(tmdy, a.dy, es, a.W, a.H, a.N * a.C, pitch_dy, rows_dy);
+}
+
+template <typename T, int K, bool AL>
+static cudaError_t bwd_run(const DwArgs& a, const CUtensorMap& tmx, const CUtensorMap& tmdy,
+                           const DwConfig& cfg, cudaStream_t st) {
+  using S = BwdShape<K, T, AL>;
   const size_t smem = (size_t)S::SM_BYTES;
-  auto kern = dw_bwd_kernel<T, K>;
-  cudaError_t e = set_smem_once<dw_bwd_kernel<T, K>>(smem);
+  auto kern = dw_bwd_kernel<T, K, AL>;
+  cudaError_t e = set_smem_once<dw_bwd_kernel<T, K, AL>>(smem);
   if (e != cudaSuccess) return e;
   const int64_t tiles_x = (a.W + kTileW - 1) / kTileW;
   const int64_t tiles_y = (a.H + kBwdTileH - 1) / kBwdTileH;
   const int64_t tpp = tiles_x * tiles_y;
   const int64_t chunks = dw_bwd_chunks_per_plane(a.H, a.W, cfg.tiles_per_cta);
   const int64_t grid = a.N * a.C * chunks;
-  CUtensorMap tmx, tmdy;
-  std::memset(&tmx, 0, sizeof(tmx));
-  std::memset(&tmdy, 0, sizeof(tmdy));
-  int use_tma = 0;
-  constexpr int es = sizeof(T);
-  if (plane_tma_ok(a.x, es, a.W) && plane_tma_ok(a.dy, es, a.W))
-    use_tma = make_plane_map(&tmx, a.x, es, a.W, a.H, a.N * a.C, Geo<K, es>::SP, S::ROWS) &&
-              make_plane_map(&tmdy, a.dy, es, a.W, a.H, a.N * a.C, Geo<K, es>::SP, S::ROWS);
+  const int odd_rows = has_odd_rows(sizeof(T), a.W, a.x, a.dy);
   kern<<<(unsigned)grid, kThreads, smem, st>>>(
       tmx, tmdy, static_cast<const T*>(a.x), static_cast<const T*>(a.dy), a.w,
       static_cast<T*>(a.dx), a.partials, (int)a.C, (int)a.H, (int)a.W, (int)tiles_x, (int)tpp,
-      (int)chunks, cfg.tiles_per_cta, a.border, a.vec, use_tma, dw_error_word());
+      (int)chunks, cfg.tiles_per_cta, a.border, a.vec, odd_rows, dw_error_word());
   note_launch();
   return cudaGetLastError();
+}
+
+template <typename T, int K>
+static cudaError_t bwd_impl(const DwArgs& a, const DwConfig& cfg, cudaStream_t st) {
+  constexpr int rows = BwdShape<K, T, true>::ROWS;
+  CUtensorMap tmx, tmdy;
+  return xdy_maps<T, K>(a, rows, rows, Geo<K, sizeof(T)>::SP, &tmx, &tmdy)
+             ? bwd_run<T, K, true>(a, tmx, tmdy, cfg, st)
+             : bwd_run<T, K, false>(a, tmx, tmdy, cfg, st);
 }
 
 template <int K>
@@ -130,12 +155,13 @@ cudaError_t dw_bwd_launch(const DwArgs& a, const DwConfig& cfg, cudaStream_t st)
   }
 }
 
-template <typename T, int K>
-static cudaError_t bwd_ring_impl(const DwArgs& a, const DwConfig& cfg, cudaStream_t st) {
-  using S = RingShape<K, T>;
+template <typename T, int K, bool AL>
+static cudaError_t bwd_ring_run(const DwArgs& a, const CUtensorMap& tmx, const CUtensorMap& tmdy,
+                                const DwConfig& cfg, cudaStream_t st) {
+  using S = RingShape<K, T, AL>;
   const size_t smem = (size_t)S::SM_BYTES;
-  auto kern = dw_bwd_ring_kernel<T, K>;
-  cudaError_t e = set_smem_once<dw_bwd_ring_kernel<T, K>>(smem);
+  auto kern = dw_bwd_ring_kernel<T, K, AL>;
+  cudaError_t e = set_smem_once<dw_bwd_ring_kernel<T, K, AL>>(smem);
   if (e != cudaSuccess) return e;
   static int ctas_per_sm[64] = {};
   int dev = 0;
@@ -154,21 +180,23 @@ static cudaError_t bwd_ring_impl(const DwArgs& a, const DwConfig& cfg, cudaStrea
   const int64_t num_chunks = a.N * a.C * chunks;
   const int64_t grid = std::min<int64_t>(num_chunks, (int64_t)per_sm * sm_count());
   if (num_chunks + grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  CUtensorMap tmx, tmdy;
-  std::memset(&tmx, 0, sizeof(tmx));
-  std::memset(&tmdy, 0, sizeof(tmdy));
-  int use_tma = 0;
-  constexpr int es = sizeof(T);
-  if (plane_tma_ok(a.x, es, a.W) && plane_tma_ok(a.dy, es, a.W))
-    use_tma = make_plane_map(&tmx, a.x, es, a.W, a.H, a.N * a.C, Geo<K, es>::SP, S::ROWS) &&
-              make_plane_map(&tmdy, a.dy, es, a.W, a.H, a.N * a.C, Geo<K, es>::SP, S::ROWS);
+  const int odd_rows = has_odd_rows(sizeof(T), a.W, a.x, a.dy);
   kern<<<(unsigned)grid, S::NT, smem, st>>>(
       tmx, tmdy, static_cast<const T*>(a.x), static_cast<const T*>(a.dy), a.w,
       static_cast<T*>(a.dx), a.partials, (int)a.C, (int)a.H, (int)a.W,
       make_fastdiv((uint32_t)tiles_x), (int)(tiles_x * tiles_y), make_fastdiv((uint32_t)chunks),
-      cfg.tiles_per_cta, (int)num_chunks, a.border, a.vec, use_tma, dw_error_word());
+      cfg.tiles_per_cta, (int)num_chunks, a.border, a.vec, odd_rows, dw_error_word());
   note_launch();
   return cudaGetLastError();
+}
+
+template <typename T, int K>
+static cudaError_t bwd_ring_impl(const DwArgs& a, const DwConfig& cfg, cudaStream_t st) {
+  constexpr int rows = RingShape<K, T, true>::ROWS;
+  CUtensorMap tmx, tmdy;
+  return xdy_maps<T, K>(a, rows, rows, Geo<K, sizeof(T)>::SP, &tmx, &tmdy)
+             ? bwd_ring_run<T, K, true>(a, tmx, tmdy, cfg, st)
+             : bwd_ring_run<T, K, false>(a, tmx, tmdy, cfg, st);
 }
 
 template <int K>
@@ -181,12 +209,13 @@ cudaError_t dw_bwd_ring_launch(const DwArgs& a, const DwConfig& cfg, cudaStream_
   }
 }
 
-template <typename T, int K>
-static cudaError_t filter_impl(const DwArgs& a, const DwConfig& cfg, cudaStream_t st) {
-  using S = FilterShape<K, T>;
+template <typename T, int K, bool AL>
+static cudaError_t filter_run(const DwArgs& a, const CUtensorMap& tmx, const CUtensorMap& tmdy,
+                              const DwConfig& cfg, cudaStream_t st) {
+  using S = FilterShape<K, T, AL>;
   const size_t smem = (size_t)S::SM_BYTES;
-  auto kern = dw_filter_kernel<T, K>;
-  cudaError_t e = set_smem_once<dw_filter_kernel<T, K>>(smem);
+  auto kern = dw_filter_kernel<T, K, AL>;
+  cudaError_t e = set_smem_once<dw_filter_kernel<T, K, AL>>(smem);
   if (e != cudaSuccess) return e;
   static int ctas_per_sm[64] = {};
   int dev = 0;
@@ -206,25 +235,23 @@ static cudaError_t filter_impl(const DwArgs& a, const DwConfig& cfg, cudaStream_
   const int64_t num_chunks = a.N * a.C * chunks;
   const int64_t grid = std::min<int64_t>(num_chunks, (int64_t)per_sm * sm_count());
   if (num_chunks + grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  // TMA staging: rows with a 16-byte stride from 16-byte aligned bases;
-  // otherwise cp.async staging.
-  CUtensorMap tmx, tmdy;
-  std::memset(&tmx, 0, sizeof(tmx));
-  std::memset(&tmdy, 0, sizeof(tmdy));
-  int use_tma = 0;
-  constexpr int es = sizeof(T);
-  if (plane_tma_ok(a.x, es, a.W) && plane_tma_ok(a.dy, es, a.W)) {
-    use_tma = make_plane_map(&tmx, a.x, es, a.W, a.H, a.N * a.C, Geo<K, es>::SP, S::X_ROWS) &&
-              make_plane_map(&tmdy, a.dy, es, a.W, a.H, a.N * a.C, kTileW, kFilterTileH);
-  }
+  const int odd_rows = has_odd_rows(sizeof(T), a.W, a.x, a.dy);
   int* err = dw_error_word();
   kern<<<(unsigned)grid, S::NT, smem, st>>>(
       tmx, tmdy, static_cast<const T*>(a.x), static_cast<const T*>(a.dy), a.partials, (int)a.H,
       (int)a.W, make_fastdiv((uint32_t)tiles_x), (int)(tiles_x * tiles_y),
-      make_fastdiv((uint32_t)chunks), cfg.tiles_per_cta, (int)num_chunks, a.border, a.vec,
-      use_tma, err);
+      make_fastdiv((uint32_t)chunks), cfg.tiles_per_cta, (int)num_chunks, a.border, odd_rows,
+      err);
   note_launch();
   return cudaGetLastError();
+}
+
+template <typename T, int K>
+static cudaError_t filter_impl(const DwArgs& a, const DwConfig& cfg, cudaStream_t st) {
+  CUtensorMap tmx, tmdy;
+  return xdy_maps<T, K>(a, FilterShape<K, T, true>::X_ROWS, kFilterTileH, kTileW, &tmx, &tmdy)
+             ? filter_run<T, K, true>(a, tmx, tmdy, cfg, st)
+             : filter_run<T, K, false>(a, tmx, tmdy, cfg, st);
 }
 
 template <int K>
@@ -237,30 +264,24 @@ cudaError_t dw_filter_launch(const DwArgs& a, const DwConfig& cfg, cudaStream_t 
   }
 }
 
-template <typename T, int K>
-static cudaError_t sep_impl(const DwArgs& a, const float* wcol, const float* wrow,
-                            cudaStream_t st) {
-  using S = SepShape<K, T>;
+template <typename T, int K, bool AL>
+static cudaError_t sep_run(const DwArgs& a, const CUtensorMap& tm, const float* wcol,
+                           const float* wrow, cudaStream_t st) {
+  using S = SepShape<K, T, AL>;
   // FP32 K = 13, 15: the five-CTA compilation (instantiated for those only)
-  decltype(&dw_sep_kernel<T, K>) kern = dw_sep_kernel<T, K>;
+  decltype(&dw_sep_kernel<T, K, AL>) kern = dw_sep_kernel<T, K, AL>;
   cudaError_t e;
-  if constexpr (sizeof(T) == 4 && (K == 13 || K == 15)) {
-    kern = dw_sep_kernel_hi_occ<T, K>;
-    e = set_smem_once<dw_sep_kernel_hi_occ<T, K>>((size_t)S::SM_BYTES);
+  if constexpr (AL && sizeof(T) == 4 && (K == 13 || K == 15)) {
+    kern = dw_sep_kernel_hi_occ<T, K, AL>;
+    e = set_smem_once<dw_sep_kernel_hi_occ<T, K, AL>>((size_t)S::SM_BYTES);
   } else {
-    e = set_smem_once<dw_sep_kernel<T, K>>((size_t)S::SM_BYTES);
+    e = set_smem_once<dw_sep_kernel<T, K, AL>>((size_t)S::SM_BYTES);
   }
   if (e != cudaSuccess) return e;
   const int64_t tiles_x = (a.W + kTileW - 1) / kTileW;
   const int64_t tiles_y = (a.H + S::TH - 1) / S::TH;
   const int64_t grid = a.N * a.C * tiles_x * tiles_y;
   if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  CUtensorMap tm;
-  std::memset(&tm, 0, sizeof(tm));
-  int use_tma = 0;
-  if (plane_tma_ok(a.x, sizeof(T), a.W))
-    use_tma = make_plane_map(&tm, a.x, sizeof(T), a.W, a.H, a.N * a.C, Geo<K, sizeof(T)>::SP,
-                             S::ROWS);
   // L2 prefetch of the tile one wave of resident CTAs ahead: at K = 15 the
   // pass waits on its tile load (0.731 -> 0.700 ms on 8 x 3 x 4096^2); at
   // K = 3 and 7 it runs near the HBM rate and the prefetch costs 23 % / 15 %,
@@ -281,9 +302,22 @@ static cudaError_t sep_impl(const DwArgs& a, const float* wcol, const float* wro
   kern<<<(unsigned)grid, kThreads, (size_t)S::SM_BYTES, st>>>(
       tm, static_cast<const T*>(a.x), wcol, wrow, static_cast<T*>(a.y),
       make_fastdiv((uint32_t)a.C), (int)a.H, (int)a.W, make_fastdiv((uint32_t)tiles_x),
-      make_fastdiv((uint32_t)tiles_y), a.border, a.vec, use_tma, pf, dw_error_word());
+      make_fastdiv((uint32_t)tiles_y), a.border, a.vec,
+      has_odd_rows(sizeof(T), a.W, a.x), pf, dw_error_word());
   note_launch();
   return cudaGetLastError();
+}
+
+template <typename T, int K>
+static cudaError_t sep_impl(const DwArgs& a, const float* wcol, const float* wrow,
+                            cudaStream_t st) {
+  CUtensorMap tm;
+  std::memset(&tm, 0, sizeof(tm));
+  if (a.vec && plane_tma_ok(a.x, sizeof(T), a.W) &&
+      make_plane_map(&tm, a.x, sizeof(T), a.W, a.H, a.N * a.C, Geo<K, sizeof(T)>::SP,
+                     SepShape<K, T, true>::ROWS))
+    return sep_run<T, K, true>(a, tm, wcol, wrow, st);
+  return sep_run<T, K, false>(a, tm, wcol, wrow, st);
 }
 
 template <int K>

@@ -47,10 +47,10 @@ __global__ void __launch_bounds__(256) gray_kernel(const T* __restrict__ x, T* _
 // slices -- one TMA load with a box three planes deep, or cp.async -- then
 // every staged cell becomes its gray value (FP32: in place over the red
 // slice; BF16: into a separate FP32 tile in the compute geometry).
-template <int K, typename T>
+template <int K, typename T, bool AL>
 struct GrayShape {
-  using G = Geo<K>;
-  using GS = Geo<K, sizeof(T)>;
+  using G = GeoC<K, T, !AL>;
+  using GS = Geo<K, sizeof(T), !AL>;
   static constexpr int PY = 4;
   static constexpr int TH = kWarps * PY;
   static constexpr int ROWS = TH + 2 * G::R;
@@ -61,16 +61,21 @@ struct GrayShape {
   static constexpr int W_OFF =
       round_up(std::max(STAGED + 3 * SLICE, GRAY + ROWS * G::SP * 4), 16);
   static constexpr int SM_BYTES = W_OFF + G::WPAD * 4;
+  // row buffers of store_rows: staged pixels that are dead once the gray tile
+  // is formed (FP32: the green slice; BF16: the staged slices)
+  static constexpr int ROW_BUFS = STAGED + (sizeof(T) == 4 ? SLICE : 0);
+  static_assert(ROW_BUFS % 16 == 0 && kWarps * kRowBuf <= (sizeof(T) == 4 ? 2 : 3) * SLICE,
+                "row buffers fit the dead slices");
 };
 
-template <typename T, int K>
+template <typename T, int K, bool AL>
 __global__ void __launch_bounds__(kThreads) gray_fwd_kernel(
     const __grid_constant__ CUtensorMap tmx, const T* __restrict__ x, const float* __restrict__ w,
-    T* __restrict__ y, int H, int W, FastDiv ftx, FastDiv fty, int clamp, int vec, int use_tma,
+    T* __restrict__ y, int H, int W, FastDiv ftx, FastDiv fty, int clamp, int vec, int odd_rows,
     int* err) {
-  using G = Geo<K>;
-  using GS = Geo<K, sizeof(T)>;
-  using S = GrayShape<K, T>;
+  using S = GrayShape<K, T, AL>;
+  using G = typename S::G;
+  using GS = typename S::GS;
   extern __shared__ __align__(128) float smem[];
   char* sm = reinterpret_cast<char*>(smem);
   uint64_t* bar = reinterpret_cast<uint64_t*>(sm);
@@ -93,7 +98,7 @@ __global__ void __launch_bounds__(kThreads) gray_fwd_kernel(
     mbar_init_fence();
   }
   cta_barrier();
-  if (use_tma) {
+  if constexpr (AL) {
     cp_async_commit();
     if (threadIdx.x == 0) {
       fence_proxy_async();
@@ -109,14 +114,18 @@ __global__ void __launch_bounds__(kThreads) gray_fwd_kernel(
     constexpr int SLICE_ELEMS = S::ROWS * GS::SP;
 #pragma unroll 1
     for (int ch = 0; ch < 3; ++ch)
-      stage_tile<T, G::R, GS::RP, GS::SP, kThreads, false>(
-          staged + ch * SLICE_ELEMS, x + (3 * n + ch) * (int64_t)H * W, H, W, ty0, tx0, S::ROWS,
-          clamp != 0, vec != 0);
-    cp_async_commit();
+      stage_any<T, kThreads>(staged + ch * SLICE_ELEMS, x + (3 * n + ch) * (int64_t)H * W, H, W,
+                             ty0, tx0, S::ROWS, G::R, GS::RP, GS::SP, odd_rows);
     cp_async_wait_all();
+    if (odd_rows) {
+#pragma unroll 1
+      for (int ch = 0; ch < 3; ++ch)
+        shift_odd_rows<T, kThreads>(staged + ch * SLICE_ELEMS, x + (3 * n + ch) * (int64_t)H * W,
+                                    H, W, ty0, S::ROWS, G::R, GS::RP, GS::SP);
+    }
   }
   cta_barrier();
-  if (*s_abort) {
+  if (AL && *s_abort) {
     mbar_wait(bar, 0);  // let a late copy land (bounded) before the CTA exits
     return;
   }
@@ -138,28 +147,38 @@ __global__ void __launch_bounds__(kThreads) gray_fwd_kernel(
     }
   }
   cta_barrier();
-  if (use_tma && clamp &&
+  if (clamp &&
       (ty0 - G::R < 0 || ty0 + S::TH + G::R > H || tx0 - G::RP < 0 || tx0 + kTileW + G::RP > W))
     clamp_fix<float, G::SP, kThreads>(gt, H, W, ty0, tx0, G::R, G::RP, S::ROWS);
   float acc[S::PY][4];
-  fwd_block<K, S::PY, float>(gt + warp * S::PY * G::SP + 4 * lane, sw, acc);
-  store_block<T, S::PY>(y + n * (int64_t)H * W, H, W, ty0 + warp * S::PY, tx0 + 4 * lane,
-                        vec != 0, acc);
+  fwd_block<K, S::PY, float, !AL && sizeof(T) == 4>(gt + warp * S::PY * G::SP + 4 * lane, sw, acc);
+  store_tile<T, S::PY, AL>(y + n * (int64_t)H * W, H, W, ty0 + warp * S::PY, tx0, vec != 0,
+                           reinterpret_cast<float*>(sm + S::ROW_BUFS + warp * kRowBuf), acc);
 }
 
-template <typename T, int K>
-static cudaError_t gray_fwd_impl(const GrayArgs& a, cudaStream_t st) {
-  using S = GrayShape<K, T>;
-  cudaError_t e = set_smem_once<gray_fwd_kernel<T, K>>((size_t)S::SM_BYTES);
+template <typename T, int K, bool AL>
+static cudaError_t gray_fwd_run(const GrayArgs& a, const CUtensorMap& tm, cudaStream_t st) {
+  using S = GrayShape<K, T, AL>;
+  cudaError_t e = set_smem_once<gray_fwd_kernel<T, K, AL>>((size_t)S::SM_BYTES);
   if (e != cudaSuccess) return e;
   const int64_t tiles_x = (a.W + kTileW - 1) / kTileW;
   const int64_t tiles_y = (a.H + S::TH - 1) / S::TH;
   const int64_t grid = a.N * tiles_x * tiles_y;
   if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+  gray_fwd_kernel<T, K, AL><<<(unsigned)grid, kThreads, (size_t)S::SM_BYTES, st>>>(
+      tm, static_cast<const T*>(a.x), a.w, static_cast<T*>(a.y), (int)a.H, (int)a.W,
+      make_fastdiv((uint32_t)tiles_x), make_fastdiv((uint32_t)tiles_y), a.border, a.vec,
+      has_odd_rows(sizeof(T), a.W, a.x), dw_error_word());
+  note_launch();
+  return cudaGetLastError();
+}
+
+template <typename T, int K>
+static cudaError_t gray_fwd_impl(const GrayArgs& a, cudaStream_t st) {
+  using S = GrayShape<K, T, true>;
   CUtensorMap tm;
   std::memset(&tm, 0, sizeof(tm));
-  int use_tma = 0;
-  if (plane_tma_ok(a.x, sizeof(T), a.W)) {
+  if (a.vec && plane_tma_ok(a.x, sizeof(T), a.W)) {
     // the box is three planes deep: the R, G and B tiles of one image in one load
     EncodeFn enc = encode_fn();
     if (enc) {
@@ -168,19 +187,14 @@ static cudaError_t gray_fwd_impl(const GrayArgs& a, cudaStream_t st) {
       cuuint64_t strides[2] = {(cuuint64_t)(a.W * es), (cuuint64_t)(a.H * a.W * es)};
       cuuint32_t box[3] = {(cuuint32_t)Geo<K, sizeof(T)>::SP, (cuuint32_t)S::ROWS, 3};
       cuuint32_t estr[3] = {1, 1, 1};
-      use_tma = enc(&tm, es == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
-                    3, const_cast<void*>(a.x), dims, strides, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+      if (enc(&tm, es == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3,
+              const_cast<void*>(a.x), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
+        return gray_fwd_run<T, K, true>(a, tm, st);
     }
   }
-  gray_fwd_kernel<T, K><<<(unsigned)grid, kThreads, (size_t)S::SM_BYTES, st>>>(
-      tm, static_cast<const T*>(a.x), a.w, static_cast<T*>(a.y), (int)a.H, (int)a.W,
-      make_fastdiv((uint32_t)tiles_x), make_fastdiv((uint32_t)tiles_y), a.border, a.vec, use_tma,
-      dw_error_word());
-  note_launch();
-  return cudaGetLastError();
+  return gray_fwd_run<T, K, false>(a, tm, st);
 }
 
 template <typename T>

@@ -44,8 +44,8 @@ struct RagImage {
   int H, W, C, K;
   int nch;      // chunks per channel
   int ic_base;  // completion counter of (this image, channel 0)
-  int vec;
-  int pad;
+  int vec;  // every tensor's rows start on a chunk boundary (16 bytes FP32, 8 BF16)
+  int odd_rows;  // has_odd_rows of x and dy
 };
 
 struct RagChunk {
@@ -79,7 +79,7 @@ constexpr int rag_dw_active() {
 
 template <int K, typename T>
 struct RagShape {
-  using G = Geo<K, sizeof(T)>;
+  using G = Geo<K, sizeof(T), true>;
   static constexpr int GT = K <= 9 ? dw_groups<K>() : rag_groups<K>();
   static constexpr int WPG = rag_dw_active<K>() / GT;
   static constexpr int AT = (K + GT - 1) / GT;
@@ -93,14 +93,18 @@ struct RagShape {
 // is in use), the filter-gradient reduction rows and two ints.
 template <typename T>
 struct RagLayout {
-  using G = Geo<kRagMaxK, sizeof(T)>;
+  using G = Geo<kRagMaxK, sizeof(T), true>;
   static constexpr int TILE = round_up((kBwdTileH + 2 * G::R) * G::SP * (int)sizeof(T), 128);
   static constexpr int STAGE = 2 * TILE;          // x, then dy
   static constexpr int WB = G::WPAD * 4;          // one filter
   static constexpr int FILT = 2 * STAGE;          // [2][w, wf]
   static constexpr int RED = FILT + 4 * WB;       // [2 chunks][w, wf] filters
   static constexpr int RED_FLOATS = 66;           // K = 11: 6 rows x 11 taps
-  static constexpr int INTS = RED + kRagDwWarps * RED_FLOATS * 4;
+  // the row buffers of the 8 forward / input-gradient warps (store_rows) share
+  // the reduction rows' space: those are used at a chunk's end, behind barriers
+  static constexpr int BUF = RED;
+  static constexpr int INTS =
+      RED + (kRagDwWarps * RED_FLOATS * 4 > 8 * kRowBuf ? kRagDwWarps * RED_FLOATS * 4 : 8 * kRowBuf);
   static constexpr int SM_BYTES = INTS + 16;
   static_assert(RagShape<11, T>::AT * 11 <= RED_FLOATS && RagShape<15, T>::AT * 15 <= RED_FLOATS,
                 "reduction rows");
@@ -119,21 +123,23 @@ __device__ __forceinline__ void rag_stage(const RagParams& p, const RagChunk& ch
                                           const RagImage& im, int t, char* sm, int sb, int fb,
                                           bool filters) {
   using L = RagLayout<T>;
-  const int K = im.K, R = (K - 1) / 2, RP = geo_rp(K, sizeof(T)), SP = kTileW + 2 * RP;
+  const int K = im.K, R = (K - 1) / 2, RP = geo_rp(K, sizeof(T));
+  const int SP = geo_pitch(K, sizeof(T), true);
   const int H = im.H, W = im.W;
   const int tiles_x = (W + kTileW - 1) / kTileW;
   const int ty0 = (t / tiles_x) * kBwdTileH, tx0 = (t % tiles_x) * kTileW;
   const int64_t off = (int64_t)ch.channel * H * W;
   const bool do_fwd = p.ops & 1, do_dx = p.ops & 2, do_dw = p.ops & 4;
-  const bool clamp = p.border == 1, vec = im.vec != 0;
   T* sx = reinterpret_cast<T*>(sm + sb * L::STAGE);
   T* sdy = reinterpret_cast<T*>(sm + sb * L::STAGE + L::TILE);
+  const T* x = static_cast<const T*>(im.x);
+  const T* dy = static_cast<const T*>(im.dy);
   if (do_fwd || do_dw)
-    stage_tile_rt<T, kRagThreads>(sx, static_cast<const T*>(im.x) + off, H, W, ty0, tx0,
-                                  kBwdTileH + 2 * R, R, RP, SP, clamp, vec);
+    stage_any<T, kRagThreads>(sx, x + off, H, W, ty0, tx0, kBwdTileH + 2 * R, R, RP, SP,
+                              im.odd_rows);
   if (do_dx || do_dw)
-    stage_tile_rt<T, kRagThreads>(sdy, static_cast<const T*>(im.dy) + off, H, W, ty0, tx0,
-                                  kBwdTileH + 2 * R, R, RP, SP, false, vec);
+    stage_any<T, kRagThreads>(sdy, dy + off, H, W, ty0, tx0, kBwdTileH + 2 * R, R, RP, SP,
+                              im.odd_rows);
   // w may be NULL when neither the forward nor the input gradient is requested
   if (filters && (do_fwd || do_dx)) {
     const float* wc = im.w + (int64_t)ch.channel * K * K;
@@ -151,7 +157,7 @@ template <typename T, int K>
 __device__ __forceinline__ int rag_chunk(const RagParams& p, const RagChunk& ch,
                                          const RagImage& im, int cn, char* sm, int sb, int fb,
                                          int* s_flag) {
-  using G = Geo<K, sizeof(T)>;
+  using G = Geo<K, sizeof(T), true>;
   using S = RagShape<K, T>;
   using L = RagLayout<T>;
   constexpr int KK = K * K;
@@ -189,10 +195,22 @@ __device__ __forceinline__ int rag_chunk(const RagParams& p, const RagChunk& ch,
     }
     cp_async_commit();
     cp_async_wait_group<1>();  // this tile's copies (committed one tile earlier) have landed
-    cta_barrier();
-    const T* sx = reinterpret_cast<const T*>(sm + sb * L::STAGE);
-    const T* sdy = reinterpret_cast<const T*>(sm + sb * L::STAGE + L::TILE);
+    T* sx = reinterpret_cast<T*>(sm + sb * L::STAGE);
+    T* sdy = reinterpret_cast<T*>(sm + sb * L::STAGE + L::TILE);
     const int ty0 = (t / tiles_x) * kBwdTileH, tx0 = (t % tiles_x) * kTileW;
+    if (im.odd_rows) {
+      if (do_fwd || do_dw)
+        shift_odd_rows<T, kRagThreads>(sx, static_cast<const T*>(im.x) + off, H, W, ty0, S::ROWS,
+                                       G::R, G::RP, G::SP);
+      if (do_dx || do_dw)
+        shift_odd_rows<T, kRagThreads>(sdy, static_cast<const T*>(im.dy) + off, H, W, ty0,
+                                       S::ROWS, G::R, G::RP, G::SP);
+    }
+    cta_barrier();
+    if (clamp && (do_fwd || do_dw) &&
+        (ty0 - G::R < 0 || ty0 + kBwdTileH + G::R > H || tx0 - G::RP < 0 ||
+         tx0 + kTileW + G::RP > W))
+      clamp_fix<T, G::SP, kRagThreads>(sx, H, W, ty0, tx0, G::R, G::RP, S::ROWS);
     if (role < 2) {
       if (role == 0 ? do_fwd : do_dx) {
         const T* src = role == 0 ? sx : sdy;
@@ -203,14 +221,15 @@ __device__ __forceinline__ int rag_chunk(const RagParams& p, const RagChunk& ch,
         for (int pass = 0; pass < 16 / BR; ++pass) {
           const int r0 = wl * 16 + pass * BR;
           float o[BR][4];
-          fwd_block<K, BR, T>(src + r0 * G::SP + 4 * lane, f, o);
-          store_block<T, BR>(dst, H, W, ty0 + r0, tx0 + 4 * lane, vec, o);
+          fwd_block<K, BR, T, true>(src + r0 * G::SP + 4 * lane, f, o);
+          store_tile<T, BR, false>(dst, H, W, ty0 + r0, tx0, vec,
+                                   reinterpret_cast<float*>(sm + L::BUF + warp * kRowBuf), o);
         }
       }
     } else if (do_dw && wl < rag_dw_active<K>()) {
       constexpr int BR = bwd_block_rows<K>();
       const int r0 = part * S::DW_ROWS;
-      dw_rows<K, S::AT, S::GT, G::SP, BR, T>(sdy + (r0 + G::R) * G::SP + G::RP + 4 * lane,
+      dw_rows<K, S::AT, S::GT, G::SP, BR, T, true>(sdy + (r0 + G::R) * G::SP + G::RP + 4 * lane,
                                              sx + (r0 + a_lo) * G::SP + 4 * lane,
                                              S::DW_ROWS / BR, nrows, acc);
     }

@@ -160,8 +160,8 @@ __device__ __forceinline__ void up_fwd_body(const T* __restrict__ x, const float
     } else {
       cp_async_wait_group<0>();
     }
-    const float* sw = stages + b * U::STAGE;
-    const float* ss = sw + round_up(G::WPAD, 4);
+    float* sw = stages + b * U::STAGE;
+    float* ss = sw + round_up(G::WPAD, 4);
     up_tile<T, K>(sx, U::ZERO_OFF, scol, rowoff, sw, ss, U::SRC_COLS, cur.ty0, cur.tx0, cur.su0,
                   cur.sv0, cur.nr, Ho, Wo, fs, clamp != 0, y + (int64_t)cur.plane * Ho * Wo,
                   vec != 0);

@@ -153,7 +153,7 @@ template <typename T, int K>
 __device__ __forceinline__ void up_tile(float* __restrict__ sx, int zero_off,
                                         int* __restrict__ scol, int* __restrict__ rowoff,
                                         const float* __restrict__ sw,
-                                        const float* __restrict__ ss, int src_pitch, int ty0,
+                                        float* __restrict__ ss, int src_pitch, int ty0,
                                         int tx0, int su0, int sv0, int nr, int Ho, int Wo,
                                         const FastDiv& fs, bool clamp, T* __restrict__ yplane,
                                         bool vec) {
@@ -195,7 +195,9 @@ __device__ __forceinline__ void up_tile(float* __restrict__ sx, int zero_off,
   cta_barrier();
   float acc[PY][4];
   fwd_block_tab<K, PY>(sx + 4 * lane, rowoff + warp * PY, sw, acc);
-  store_block<T, PY>(yplane, Ho, Wo, ty0 + warp * PY, tx0 + 4 * lane, vec, acc);
+  // the staged pixels are dead: their space serves as the warps' row buffers
+  static_assert(U::SRC_ROWS * U::SRC_COLS * 4 >= kWarps * kRowBuf, "row buffers fit");
+  store_tile<T, PY, false>(yplane, Ho, Wo, ty0 + warp * PY, tx0, vec, ss + warp * kTileW, acc);
   cta_barrier();  // the expanded rows, tables and the staged pixels are free again
 }
 
