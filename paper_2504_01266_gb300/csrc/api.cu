@@ -214,13 +214,13 @@ giga_status_t run_dw_op(int op, const DwArgs& a, const DwConfig& cfg, cudaStream
       return GIGA_OK;
     case TUNE_BWD_INPUT:
       e = dispatch_k(a.K, [&](auto k) { return dw_fwd_launch<decltype(k)::value>(a, cfg, true, st); });
-      if (e == cudaSuccess) e = dw_fixup_launch(a, st);
+      if (e == cudaSuccess) e = dw_finish_launch(a, true, 0, st);
       if (e != cudaSuccess) return cuda_fail(e, "input-gradient launch");
       return GIGA_OK;
     case TUNE_BWD_FILTER:
       e = dispatch_k_filter(a.K, [&](auto k) { return dw_filter_launch<decltype(k)::value>(a, cfg, st); });
       if (e == cudaSuccess)
-        e = dw_finalize_launch(a, dw_bwd_chunks_per_plane(a.H, a.W, cfg.tiles_per_cta), st);
+        e = dw_finish_launch(a, false, dw_bwd_chunks_per_plane(a.H, a.W, cfg.tiles_per_cta), st);
       if (e != cudaSuccess) return cuda_fail(e, "filter-gradient launch");
       return GIGA_OK;
     case TUNE_BWD_FUSED: {
@@ -232,19 +232,19 @@ giga_status_t run_dw_op(int op, const DwArgs& a, const DwConfig& cfg, cudaStream
         // same shape: take the forward's tuned configuration
         int fid = tune_mode() == 0 ? 0 : tune_lookup(TUNE_FWD, a);
         DwConfig fc = tune_config(TUNE_FWD, fid < 0 ? 0 : fid, a);
-        giga_status_t s2 = run_dw_op(TUNE_BWD_INPUT, a, fc, st);
-        if (s2 != GIGA_OK) return s2;
-        return run_dw_op(TUNE_BWD_FILTER, a, cfg, st);
-      }
-      if (cfg.ring)
+        e = dispatch_k(a.K, [&](auto k) { return dw_fwd_launch<decltype(k)::value>(a, fc, true, st); });
+        if (e == cudaSuccess)
+          e = dispatch_k_filter(a.K, [&](auto k) {
+            return dw_filter_launch<decltype(k)::value>(a, cfg, st);
+          });
+      } else if (cfg.ring)
         e = dispatch_k_filter(a.K, [&](auto k) {
           return dw_bwd_ring_launch<decltype(k)::value>(a, cfg, st);
         });
       else
         e = dispatch_k_filter(a.K, [&](auto k) { return dw_bwd_launch<decltype(k)::value>(a, cfg, st); });
-      if (e == cudaSuccess) e = dw_fixup_launch(a, st);
       if (e == cudaSuccess)
-        e = dw_finalize_launch(a, dw_bwd_chunks_per_plane(a.H, a.W, cfg.tiles_per_cta), st);
+        e = dw_finish_launch(a, true, dw_bwd_chunks_per_plane(a.H, a.W, cfg.tiles_per_cta), st);
       if (e != cudaSuccess) return cuda_fail(e, "backward launch");
       return GIGA_OK;
     }

@@ -10,7 +10,8 @@
 // columns, so an edge pixel of dx is
 //   dx[p][q] = sum_{a,b} w[a][b] * sum_{i in I(p,a)} sum_{j in J(q,b)} dy[i][j].
 // The tile kernels compute the zero-border correlation everywhere; these
-// helpers then overwrite the first/last row and column with the value above.
+// helpers then overwrite the first/last row and column with the value above
+// (the ragged batch and thin BF16 planes; dw_misc.cu folds the others).
 #pragma once
 
 #include "common.cuh"

@@ -7,8 +7,7 @@
 //   g[n][c][u][v]  = sum_{a,b} w[c][K-1-a][K-1-b] * dy~[n][c][u + a - r][v + b - r]
 //                    (dy~ zero outside the image; dx = g for the zero border,
 //                    the clamp border adds the edge fold of dw_misc.cu:
-//                    dw_fold_rows_kernel / dw_fold_cols_kernel in FP32,
-//                    dw_fixup_kernel with dw_fold.cuh in BF16)
+//                    dw_finish_kernel)
 //   dw[c][a][b]    = sum_{n,i,j} dy[n][c][i][j] * x~[n][c][i + a - r][j + b - r]
 //
 // Design (one CTA of 8 warps per 64 x 128 or 32 x 128 output tile):

@@ -13,7 +13,7 @@ constexpr int kMaxKFilter = 15;  // filter gradient and the batched path
 
 // Forward (input_grad = false): y = K_w x with the border of `a`.
 // Input gradient (input_grad = true): dx = g from dy (flipped filter, zero
-// border); the clamp edge fold is a separate launch (dw_fixup_launch).
+// border); the clamp edge fold is a separate launch (dw_finish_launch).
 template <int K>
 cudaError_t dw_fwd_launch(const DwArgs& a, const DwConfig& cfg, bool input_grad,
                           cudaStream_t st);
@@ -75,11 +75,12 @@ cudaError_t dw_wait_selftest(cudaStream_t st);
 // Number of tile chunks per plane the backward pass uses for `tiles_per_cta`.
 int64_t dw_bwd_chunks_per_plane(int64_t H, int64_t W, int tiles_per_cta);
 
-// Clamp border: overwrite the edge pixels of dx with the exact adjoint.
-cudaError_t dw_fixup_launch(const DwArgs& a, cudaStream_t st);
-
-// dw[c][k] = sum over (n, chunk) of partials, in FP64, fixed order.
-cudaError_t dw_finalize_launch(const DwArgs& a, int64_t chunks_per_plane, cudaStream_t st);
+// What follows the tile passes of a backward call: with `fold` (and the clamp
+// border) the edge fold that turns g into dx; with chunks_per_plane > 0 the
+// filter gradient dw[c][k] = the sum over (n, chunk) of the partials, in FP64
+// and a fixed order.  One launch.
+cudaError_t dw_finish_launch(const DwArgs& a, bool fold, int64_t chunks_per_plane,
+                             cudaStream_t st);
 
 #define GIGA_DW_EXTERN(K)                                                                  \
   extern template cudaError_t dw_fwd_launch<K>(const DwArgs&, const DwConfig&, bool,      \

@@ -1,7 +1,9 @@
-// dw_misc.cu -- the two small kernels around the depthwise backward pass:
+// dw_misc.cu -- what follows the tile kernels of the depthwise backward pass:
 //  * the clamp-border edge fold of the input gradient, and
-//  * the FP64 fixed-order reduction of the per-CTA filter-gradient partials.
+//  * the FP64 fixed-order reduction of the per-CTA filter-gradient partials,
+// in one launch (dw_finish_kernel).
 #include <algorithm>
+#include <cstring>
 
 #include "dw_fold.cuh"
 #include "dw_kernels.cuh"
@@ -62,6 +64,8 @@ int64_t dw_bwd_chunks_per_plane(int64_t H, int64_t W, int tiles_per_cta) {
 }
 
 // ------------------------------------------------------------- edge fold
+// BF16 planes one pixel high or wide: every pixel recomputed from the
+// definition.
 template <typename T>
 __global__ void dw_fixup_kernel(const T* __restrict__ dy, const float* __restrict__ w,
                                 T* __restrict__ dx, int C, int H, int W, int K,
@@ -85,215 +89,371 @@ __global__ void dw_fixup_kernel(const T* __restrict__ dy, const float* __restric
 //   right   R[p] = sum_{e<r}  sum_a Wr[e][a] dy[p-a+r][W-1-e], Wr[e][a] = sum_{b>=r+1+e} w[a][b]
 // and at the corners the doubly-folded sums, e.g.
 //   TL = sum_{i<r,j<r} (sum_{a<=r-1-i} sum_{b<=r-1-j} w[a][b]) dy[i][j]
-// (i, d < H and j, e < W; dy outside the image reads zero).  The row kernel adds
-// T and B to the first and last row; the column kernel, launched after it,
-// adds L, R and the corner sums to the first and last column.
-constexpr int kFoldThreads = 256;
+// (i, d < H and j, e < W; dy outside the image reads zero).  BF16 results are
+// rounded to storage already, so there the edge pixels are recomputed whole by
+// the same sums with the taps that read the edge itself included.
+
+// ------------------------------------------------- fold and reduction
+// One launch with three kinds of 512-thread blocks (what a call does not need
+// has none): the filter gradient's FP64 sums, the fold of 256 pixels of the
+// first and last row or column of a plane, and the fold of a plane's corner
+// pixels, which both folds touch.  All are short and bound by latency, so they
+// run beside each other instead of one after the other.  4 x 3 x 1801 x 2399,
+// K = 3: 4.4 (rows) + 6.7 (columns) + 13.8 us (sums, a warp per tap striding
+// over the partials, uncoalesced) as three launches, 6.1 us as one; K = 15,
+// 8 x 3 x 1024^2: 52 -> 12.9 us; BF16 K = 9, 4 x 3 x 1800 x 2400: 60 (the
+// pixel-by-pixel fold 45 of it) -> 10.7 us; 4 x 3 x 257 x 251: 10.5 -> 4.3 us.
+constexpr int kFinishThreads = 512;
+constexpr int kFoldPixels = 256;  // per fold block: one thread for each of its two edges
+
+struct FinishArgs {
+  const float* partials;  // filter gradient: [N * C * chunks][KK]
+  float* dw;
+  int N, C, KK;
+  int taps, groups;  // taps per block, such groups of a filter
+  int sum_blocks;   // C * groups, or 0
+  FastDiv chunks;   // per plane
+  const void* dy;  // fold
+  const float* w;
+  void* dx;
+  int H, W, K;
+  int row_blocks, col_blocks;  // per plane; plus one corner block
+  int64_t plane0;   // first plane of this launch
+};
+
+// dw[c][k] = sum over the partial rows (image n, chunk ch) of channel c, in
+// FP64 and a fixed order: a block takes p.taps taps of one channel, a thread
+// every (512 / p.taps)-th row of one tap, eight loads in flight; then a
+// butterfly within the warp and the warps in order.  FP64 adds and
+// conversions bound it (about two a clock on an SM), so the taps are spread
+// over as many blocks as fill the GPU (finish_taps) rather than read by few
+// in whole sectors (4 x 3 x 1801 x 2399, K = 3, with the fold: 22 us with 32
+// taps per block, 6 us with one).
+__device__ __forceinline__ void finish_sums(const FinishArgs& p, double* red) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int c = (int)blockIdx.x / p.groups, g = (int)blockIdx.x - c * p.groups;
+  const int TB = p.taps;  // a power of two, at most 32
+  const int tap = TB * g + (threadIdx.x & (TB - 1));
+  const int slots = kFinishThreads / TB;
+  const uint32_t chunks = p.chunks.d;
+  const uint32_t count = (uint32_t)p.N * chunks;
+  double s = 0.0;
+  if (tap < p.KK) {
+    constexpr int U = 8;
+    for (uint32_t i0 = threadIdx.x / TB; i0 < count; i0 += U * slots) {
+      float v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const uint32_t i = i0 + u * slots;
+        v[u] = 0.f;
+        if (i < count) {
+          const uint32_t n = fdiv(i, p.chunks), ch = i - n * chunks;
+          v[u] = __ldg(p.partials + (((int64_t)n * p.C + c) * chunks + ch) * p.KK + tap);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (i0 + u * slots < count) s += (double)v[u];
+    }
+  }
+  for (int o = 16; o >= TB; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane < TB) red[warp * TB + lane] = s;
+  __syncthreads();
+  if ((int)threadIdx.x < TB && tap < p.KK) {
+    double sum = 0.0;
+    for (int w = 0; w < kFinishThreads / 32; ++w) sum += red[w * TB + threadIdx.x];
+    p.dw[(int64_t)c * p.KK + tap] = (float)sum;
+  }
+}
+
+// Taps per block: the fewest (a power of two) for which the blocks of all
+// channels fit the GPU about twice over.
+static int finish_taps(int64_t C, int KK) {
+  int taps = 1;
+  while (taps < 32 && C * ((KK + taps - 1) / taps) > 2 * (int64_t)sm_count()) taps *= 2;
+  return taps;
+}
 
 __device__ __forceinline__ float dy_at(const float* g, int H, int W, int i, int j) {
-  return (i >= 0 && i < H && j >= 0 && j < W) ? g[(int64_t)i * W + j] : 0.f;
+  return (i >= 0 && i < H && j >= 0 && j < W) ? __ldg(g + (int64_t)i * W + j) : 0.f;
 }
 
-__global__ void dw_fold_rows_kernel(const float* __restrict__ dy, const float* __restrict__ w,
-                                    float* __restrict__ dx, int C, int H, int W, int K) {
-  extern __shared__ float tab[];  // Wt[r][K], Wb[r][K]
-  const int r = (K - 1) / 2;
-  const int64_t plane = blockIdx.y;
-  const float* f = w + (plane % C) * (int64_t)K * K;
-  float* Wt = tab;
-  float* Wb = tab + r * K;
-  for (int k = threadIdx.x; k < r * K; k += blockDim.x) {
-    const int i = k / K, b = k % K;
-    float t = 0.f, u = 0.f;
-    for (int a = 0; a <= r - 1 - i; ++a) t += f[a * K + b];
-    for (int a = r + 1 + i; a < K; ++a) u += f[a * K + b];
-    Wt[k] = t;
-    Wb[k] = u;
+// Rows (columns) of dy an edge pixel's sum takes, counted from the edge, and
+// the filter rows (columns) a = lo .. hi whose weights are summed for the i-th:
+// FP32 adds the margin sums to the stored g, so row i < r takes the taps that
+// reach outside; BF16 recomputes the whole value (one rounding), so the tap
+// that reads the edge itself joins them, and row r.
+template <typename T>
+__device__ __forceinline__ int fold_depth(int r) { return sizeof(T) == 4 ? r : r + 1; }
+template <typename T>
+__device__ __forceinline__ float fold_weight(const float* f, int step, int K, int e, int i) {
+  const int r = (K - 1) / 2, full = sizeof(T) == 4 ? 0 : 1;
+  const int lo = e ? r + 1 + i - full : 0, hi = e ? K - 1 : r - 1 - i + full;
+  float t = 0.f;
+  for (int a = lo; a <= hi; ++a) t += f[a * step];
+  return t;
+}
+
+// Pixels 256 * blk .. of the first and last row (rows = true: sums T and B
+// above, one half of the block each) or column (L and R) of a plane; its
+// corner pixels are left to finish_corners.
+template <typename T>
+__device__ __forceinline__ void finish_edges(const FinishArgs& p, int64_t plane, int blk, bool rows,
+                                             float* tab) {
+  const int K = p.K, r = (K - 1) / 2, H = p.H, W = p.W, D = fold_depth<T>(r);
+  const int lim = rows ? W : H;    // length of the edge
+  const int other = rows ? H : W;  // rows (columns) across it
+  const float* f = p.w + (plane % p.C) * (int64_t)K * K;
+  float* sf = tab;                // the filter
+  float* wt = sf + K * K;         // [2][D][K] summed weights: first edge, last edge
+  float* strip = wt + 2 * D * K;  // [2][D][kFoldPixels + 2 r] of dy
+  const int SW = kFoldPixels + 2 * r;
+  const T* g = static_cast<const T*>(p.dy) + plane * (int64_t)H * W;
+  const int q0 = blk * kFoldPixels, n = min(D, other);
+  const int e = threadIdx.x / kFoldPixels, t = threadIdx.x - e * kFoldPixels;
+  const int q = q0 + t, in = e ? other - 1 : 0;
+  const bool mine = q > 0 && q < lim - 1 && !(e == 1 && other == 1);
+  T* d = static_cast<T*>(p.dx) + plane * (int64_t)H * W +
+         (rows ? (int64_t)in * W + q : (int64_t)q * W + in);
+  float s = 0.f, old = 0.f;
+  if (sizeof(T) == 4 && mine) old = Elem<T>::load(d);  // on its way while the strip arrives
+  for (int k = threadIdx.x; k < K * K; k += kFinishThreads) sf[k] = __ldg(f + k);
+  // strip[e][i][c]: i rows (columns) in from edge e, at position q0 - r + c
+  for (int k = threadIdx.x; k < 2 * D * SW; k += kFinishThreads) {
+    int es, i, c;
+    if (rows) {  // consecutive threads along the row
+      es = k / (D * SW), i = k / SW - es * D, c = k - (k / SW) * SW;
+    } else {     // along the first / last columns of a row
+      c = k / (2 * D), es = (k - c * 2 * D) / D, i = k - c * 2 * D - es * D;
+    }
+    const int at = q0 - r + c, from = es ? other - 1 - i : i;
+    float v = 0.f;
+    if (i < n && at >= 0 && at < lim)
+      v = Elem<T>::load(g + (rows ? (int64_t)from * W + at : (int64_t)at * W + from));
+    strip[(es * D + i) * SW + c] = v;
   }
   __syncthreads();
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= W) return;
-  const float* g = dy + plane * (int64_t)H * W;
-  const int rows = min(r, H);
-  float top = 0.f, bot = 0.f;
-  for (int i = 0; i < rows; ++i)
-    for (int b = 0; b < K; ++b) {
-      top = fmaf(Wt[i * K + b], dy_at(g, H, W, i, q - b + r), top);
-      bot = fmaf(Wb[i * K + b], dy_at(g, H, W, H - 1 - i, q - b + r), bot);
-    }
-  float* d = dx + plane * (int64_t)H * W;
-  if (H == 1) {
-    d[q] += top + bot;
-  } else {
-    d[q] += top;
-    d[(int64_t)(H - 1) * W + q] += bot;
-  }
-}
-
-__global__ void dw_fold_cols_kernel(const float* __restrict__ dy, const float* __restrict__ w,
-                                    float* __restrict__ dx, int C, int H, int W, int K) {
-  extern __shared__ float tab[];  // Wl[r][K], Wr[r][K], corners 4 x r x r, two row strips
-  const int r = (K - 1) / 2;
-  const int64_t plane = blockIdx.y;
-  const float* f = w + (plane % C) * (int64_t)K * K;
-  float* Wl = tab;
-  float* Wr = tab + r * K;
-  float* Ctl = tab + 2 * r * K;
-  float* Ctr = Ctl + r * r;
-  float* Cbl = Ctr + r * r;
-  float* Cbr = Cbl + r * r;
-  for (int k = threadIdx.x; k < r * K; k += blockDim.x) {
-    const int j = k / K, a = k % K;
-    float l = 0.f, rr = 0.f;
-    for (int b = 0; b <= r - 1 - j; ++b) l += f[a * K + b];
-    for (int b = r + 1 + j; b < K; ++b) rr += f[a * K + b];
-    Wl[k] = l;
-    Wr[k] = rr;
-  }
-  for (int k = threadIdx.x; k < r * r; k += blockDim.x) {
-    const int i = k / r, j = k % r;
-    float tl = 0.f, tr = 0.f, bl = 0.f, br = 0.f;
-    for (int a = 0; a < K; ++a)
-      for (int b = 0; b < K; ++b) {
-        const float v = f[a * K + b];
-        const bool top = a <= r - 1 - i, bottom = a >= r + 1 + i;
-        const bool left = b <= r - 1 - j, right = b >= r + 1 + j;
-        if (top && left) tl += v;
-        if (top && right) tr += v;
-        if (bottom && left) bl += v;
-        if (bottom && right) br += v;
-      }
-    Ctl[k] = tl;
-    Ctr[k] = tr;
-    Cbl[k] = bl;
-    Cbr[k] = br;
-  }
-  // the block's rows p0 - r .. p0 + blockDim.x - 1 + r of the first and the
-  // last r columns, staged once (neighbouring threads share K - 1 of their K
-  // rows; reading them from global memory per thread was latency-bound)
-  const float* g = dy + plane * (int64_t)H * W;
-  const int cols = min(r, W), rows = min(r, H);
-  const int p0 = blockIdx.x * blockDim.x;
-  const int strip_rows = blockDim.x + 2 * r;
-  float* sl = Cbr + r * r;           // [strip_rows][r]: columns 0 .. r - 1
-  float* sr = sl + strip_rows * r;   // [strip_rows][r]: columns W - 1 .. W - r
-  for (int k = threadIdx.x; k < strip_rows * r; k += blockDim.x) {
-    const int i = k / r, j = k - (k / r) * r;
-    const int row = p0 - r + i;
-    sl[k] = j < cols ? dy_at(g, H, W, row, j) : 0.f;
-    sr[k] = j < cols ? dy_at(g, H, W, row, W - 1 - j) : 0.f;
+  for (int k = threadIdx.x; k < 2 * D * K; k += kFinishThreads) {
+    const int ew = k / (D * K), i = k / K - ew * D, b = k - (k / K) * K;
+    wt[k] = rows ? fold_weight<T>(sf + b, K, K, ew, i) : fold_weight<T>(sf + b * K, 1, K, ew, i);
   }
   __syncthreads();
-  const int p = p0 + threadIdx.x;
-  if (p >= H) return;
-  float left = 0.f, right = 0.f;
-  for (int j = 0; j < cols; ++j)
-    for (int a = 0; a < K; ++a) {
-      // dy row p - a + r sits at strip row threadIdx.x + 2r - a
-      const int i = threadIdx.x + 2 * r - a;
-      left = fmaf(Wl[j * K + a], sl[i * r + j], left);
-      right = fmaf(Wr[j * K + a], sr[i * r + j], right);
-    }
-  // corner sums belong to the pixels of the first / last row
-  if (p == 0 || p == H - 1) {
-    for (int i = 0; i < rows; ++i)
-      for (int j = 0; j < cols; ++j) {
-        if (p == 0) {
-          left = fmaf(Ctl[i * r + j], dy_at(g, H, W, i, j), left);
-          right = fmaf(Ctr[i * r + j], dy_at(g, H, W, i, W - 1 - j), right);
-        }
-        if (p == H - 1) {
-          left = fmaf(Cbl[i * r + j], dy_at(g, H, W, H - 1 - i, j), left);
-          right = fmaf(Cbr[i * r + j], dy_at(g, H, W, H - 1 - i, W - 1 - j), right);
-        }
-      }
+  for (int i = 0; i < n; ++i)
+    for (int b = 0; b < K; ++b)
+      s = fmaf(wt[(e * D + i) * K + b], strip[(e * D + i) * SW + t + 2 * r - b], s);
+  if (other == 1) {  // a single row (column) is both edges: the first half adds both sums
+    __syncthreads();
+    if (e == 1) strip[t] = s;
+    __syncthreads();
+    s += strip[t];
   }
-  float* d = dx + plane * (int64_t)H * W + (int64_t)p * W;
-  if (W == 1) {
-    d[0] += left + right;
-  } else {
-    d[0] += left;
-    d[W - 1] += right;
+  if (mine) Elem<T>::store(d, old + s);
+}
+
+// BF16: the four corner pixels of a plane with H, W >= 2, recomputed:
+// dx = sum_{i,j <= r} C[i][j] dy[i][j], rows and columns counted from the
+// corner, C[i][j] = the sum of the taps that bring (i, j) there.
+__device__ __forceinline__ void finish_corners_bf16(const FinishArgs& p, int64_t plane,
+                                                    float* tab) {
+  const int K = p.K, r = (K - 1) / 2, H = p.H, W = p.W, D = r + 1;
+  const float* f = p.w + (plane % p.C) * (int64_t)K * K;
+  const __nv_bfloat16* g = static_cast<const __nv_bfloat16*>(p.dy) + plane * (int64_t)H * W;
+  float* wc = tab;               // [2][D][K]: a column edge's weights of filter row a
+  float* prod = wc + 2 * D * K;  // [4][D][D]
+  for (int k = threadIdx.x; k < 2 * D * K; k += kFinishThreads) {
+    const int e = k / (D * K), j = k / K - e * D, a = k - (k / K) * K;
+    wc[k] = fold_weight<__nv_bfloat16>(f + a * K, 1, K, e, j);
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < 4 * D * D; k += kFinishThreads) {
+    const int q = k / (D * D), i = k / D - q * D, j = k - (k / D) * D;
+    const int er = q >> 1, ec = q & 1;
+    const float c = fold_weight<__nv_bfloat16>(wc + (ec * D + j) * K, 1, K, er, i);
+    const int row = er ? H - 1 - i : i, col = ec ? W - 1 - j : j;
+    const bool ok = row >= 0 && row < H && col >= 0 && col < W;
+    prod[k] = ok ? c * Elem<__nv_bfloat16>::load(g + (int64_t)row * W + col) : 0.f;
+  }
+  __syncthreads();
+  if (threadIdx.x < 4) {
+    const int er = threadIdx.x >> 1, ec = threadIdx.x & 1;
+    float s = 0.f;
+    for (int k = 0; k < D * D; ++k) s += prod[threadIdx.x * D * D + k];
+    Elem<__nv_bfloat16>::store(static_cast<__nv_bfloat16*>(p.dx) + plane * (int64_t)H * W +
+                                   (er ? (int64_t)(H - 1) * W : 0) + (ec ? W - 1 : 0),
+                               s);
   }
 }
 
-cudaError_t dw_fixup_launch(const DwArgs& a, cudaStream_t st) {
-  if (a.border != 1 || a.N * a.C * a.H * a.W == 0) return cudaSuccess;
+// The corner pixels of a plane (one, two or four): the row sums, then the
+// column sums with the doubly folded corner terms.
+__device__ __forceinline__ void finish_corners(const FinishArgs& p, int64_t plane, float* tab) {
+  const int K = p.K, r = (K - 1) / 2, H = p.H, W = p.W;
+  const float* f = p.w + (plane % p.C) * (int64_t)K * K;
+  float* sf = tab;
+  float* wr = sf + K * K;       // [2][r][K]: Wt, Wb
+  float* wc = wr + 2 * r * K;   // [2][r][K]: Wl, Wr
+  float* cw = wc + 2 * r * K;   // [2][2][r][r]: corner weights (row edge, column edge)
+  float* sq = cw + 4 * r * r;   // [2][2][r + 1][r + 1]: dy counted from the corners
+  float* sums = sq + 4 * (r + 1) * (r + 1);  // [8]
+  const int S = r + 1;
+  const float* g = static_cast<const float*>(p.dy) + plane * (int64_t)H * W;
+  for (int k = threadIdx.x; k < K * K; k += kFinishThreads) sf[k] = __ldg(f + k);
+  for (int k = threadIdx.x; k < 4 * S * S; k += kFinishThreads) {
+    const int q = k / (S * S), i = k / S - q * S, j = k - (k / S) * S;
+    const int row = (q >> 1) ? H - 1 - i : i, col = (q & 1) ? W - 1 - j : j;
+    sq[k] = dy_at(g, H, W, row, col);
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < 4 * r * K; k += kFinishThreads) {
+    const int rows = k < 2 * r * K, kk = rows ? k : k - 2 * r * K;
+    const int e = kk / (r * K), i = kk / K - e * r, b = kk - (kk / K) * K;
+    float t = 0.f;
+    const int lo = e ? r + 1 + i : 0, hi = e ? K - 1 : r - 1 - i;
+    for (int a = lo; a <= hi; ++a) t += rows ? sf[a * K + b] : sf[b * K + a];
+    (rows ? wr : wc)[kk] = t;
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < 4 * r * r; k += kFinishThreads) {
+    const int q = k / (r * r), i = k / r - q * r, j = k - (k / r) * r;
+    const int er = q >> 1, ec = q & 1;
+    const int lo = er ? r + 1 + i : 0, hi = er ? K - 1 : r - 1 - i;
+    float t = 0.f;
+    for (int a = lo; a <= hi; ++a) t += wc[(ec * r + j) * K + a];
+    cw[k] = t;
+  }
+  __syncthreads();
+  const int nr = min(r, H), nc = min(r, W);
+  if (threadIdx.x < 8) {
+    // t = 0..3: sum of row edge er at column edge ec; 4..7: of column edge ec
+    // at row edge er (with the corner terms)
+    const int t = threadIdx.x, er = (t >> 1) & 1, ec = t & 1;
+    const float* s0 = sq + (er * 2 + ec) * S * S;
+    float s = 0.f;
+    if (t < 4) {
+      for (int i = 0; i < nr; ++i)
+        for (int b = 0; b < K; ++b) {
+          const int j = ec ? b - r : r - b;  // columns in from that edge
+          s = fmaf(wr[(er * r + i) * K + b], j >= 0 ? s0[i * S + j] : 0.f, s);
+        }
+    } else {
+      for (int j = 0; j < nc; ++j)
+        for (int a = 0; a < K; ++a) {
+          const int i = er ? a - r : r - a;
+          s = fmaf(wc[(ec * r + j) * K + a], i >= 0 ? s0[i * S + j] : 0.f, s);
+        }
+      for (int i = 0; i < nr; ++i)
+        for (int j = 0; j < nc; ++j)
+          for (int q = 0; q < 2; ++q)  // a single row is both row edges
+            if (q == er || H == 1)
+              s = fmaf(cw[((q * 2 + ec) * r + i) * r + j], sq[((q * 2 + ec) * S + i) * S + j], s);
+    }
+    sums[t] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x < 4) {
+    const int er = threadIdx.x >> 1, ec = threadIdx.x & 1;
+    if ((er && H == 1) || (ec && W == 1)) return;
+    float* d = static_cast<float*>(p.dx) + plane * (int64_t)H * W +
+               (er ? (int64_t)(H - 1) * W : 0) + (ec ? W - 1 : 0);
+    float v = *d;
+    v += H == 1 ? sums[ec] + sums[2 + ec] : sums[er * 2 + ec];
+    v += W == 1 ? sums[4 + er * 2] + sums[4 + er * 2 + 1] : sums[4 + er * 2 + ec];
+    *d = v;
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kFinishThreads) dw_finish_kernel(const FinishArgs p) {
+  extern __shared__ __align__(16) float fin_smem[];
+  if ((int)blockIdx.x < p.sum_blocks) {
+    finish_sums(p, reinterpret_cast<double*>(fin_smem));
+    return;
+  }
+  const uint32_t b = blockIdx.x - p.sum_blocks;
+  const uint32_t per = p.row_blocks + p.col_blocks + 1;
+  const int64_t plane = p.plane0 + b / per;
+  const int k = (int)(b - b / per * per);
+  if (k < p.row_blocks)
+    finish_edges<T>(p, plane, k, true, fin_smem);
+  else if (k < p.row_blocks + p.col_blocks)
+    finish_edges<T>(p, plane, k - p.row_blocks, false, fin_smem);
+  else if constexpr (sizeof(T) == 2)
+    finish_corners_bf16(p, plane, fin_smem);
+  else
+    finish_corners(p, plane, fin_smem);
+}
+
+cudaError_t dw_finish_launch(const DwArgs& a, bool fold, int64_t chunks_per_plane,
+                             cudaStream_t st) {
   const int r = (a.K - 1) / 2;
-  if (a.dtype == 0 && r > 0 && a.N * a.C <= 65535) {
-    const int64_t planes = a.N * a.C;
-    const dim3 grid_rows((unsigned)((a.W + kFoldThreads - 1) / kFoldThreads), (unsigned)planes);
-    const dim3 grid_cols((unsigned)((a.H + kFoldThreads - 1) / kFoldThreads), (unsigned)planes);
-    dw_fold_rows_kernel<<<grid_rows, kFoldThreads, sizeof(float) * 2 * r * a.K, st>>>(
-        static_cast<const float*>(a.dy), a.w, static_cast<float*>(a.dx), (int)a.C, (int)a.H,
-        (int)a.W, a.K);
+  const bool folds = fold && a.border == 1 && r > 0 && a.N * a.C * a.H * a.W > 0;
+  // BF16 planes one pixel high or wide, where an edge pixel lies on both edges
+  const bool thin = a.dtype != 0 && (a.H == 1 || a.W == 1);
+  if (folds && thin) {
+    const int64_t edge = edge_pixels(a.H, a.W);
+    const int64_t total = a.N * a.C * edge;
+    const int threads = 128;
+    const int64_t blocks = std::min<int64_t>((total + threads - 1) / threads, 65535);
+    dw_fixup_kernel<__nv_bfloat16><<<(unsigned)blocks, threads, 0, st>>>(
+        static_cast<const __nv_bfloat16*>(a.dy), a.w, static_cast<__nv_bfloat16*>(a.dx),
+        (int)a.C, (int)a.H, (int)a.W, a.K, edge, total);
     note_launch();
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const size_t cols_smem =
-        sizeof(float) * (2 * r * a.K + 4 * r * r + 2 * (kFoldThreads + 2 * r) * r);
-    dw_fold_cols_kernel<<<grid_cols, kFoldThreads, cols_smem, st>>>(
-        static_cast<const float*>(a.dy), a.w, static_cast<float*>(a.dx), (int)a.C, (int)a.H,
-        (int)a.W, a.K);
+  }
+  FinishArgs p;
+  std::memset(&p, 0, sizeof(p));
+  p.N = (int)a.N;
+  p.C = (int)a.C;
+  p.chunks = make_fastdiv(1);
+  size_t smem = 0;
+  int64_t blocks = 0, planes = 0, per = 0;
+  if (chunks_per_plane > 0) {
+    if (a.N * chunks_per_plane >= (1LL << 31)) return cudaErrorInvalidConfiguration;
+    p.partials = a.partials;
+    p.dw = a.dw;
+    p.KK = a.K * a.K;
+    p.taps = finish_taps(a.C, p.KK);
+    p.groups = (p.KK + p.taps - 1) / p.taps;
+    p.chunks = make_fastdiv((uint32_t)chunks_per_plane);
+    blocks = a.C * p.groups;
+    if (blocks >= (1LL << 31)) return cudaErrorInvalidConfiguration;
+    p.sum_blocks = (int)blocks;
+    smem = kFinishThreads * sizeof(double);
+  }
+  if (folds && !thin) {
+    p.dy = a.dy;
+    p.w = a.w;
+    p.dx = a.dx;
+    p.H = (int)a.H;
+    p.W = (int)a.W;
+    p.K = a.K;
+    p.row_blocks = (int)((a.W + kFoldPixels - 1) / kFoldPixels);
+    p.col_blocks = (int)((a.H + kFoldPixels - 1) / kFoldPixels);
+    planes = a.N * a.C;
+    per = (int64_t)p.row_blocks + p.col_blocks + 1;
+    const int D = a.dtype == 0 ? r : r + 1;  // fold_depth
+    const size_t edges = a.K * a.K + 2 * D * a.K + 2 * D * (kFoldPixels + 2 * r);
+    const size_t corners = a.K * a.K + 4 * D * a.K + 4 * r * r + 4 * (r + 1) * (r + 1) + 8;
+    smem = std::max(smem, std::max(edges, corners) * sizeof(float));
+  }
+  // one launch, unless the planes' fold blocks exceed a grid
+  do {
+    const int64_t now = per ? std::min<int64_t>(planes - p.plane0, (0x7fffffffLL - blocks) / per) : 0;
+    blocks += now * per;
+    if (blocks == 0) return cudaSuccess;
+    if (a.dtype == 0)
+      dw_finish_kernel<float><<<(unsigned)blocks, kFinishThreads, smem, st>>>(p);
+    else
+      dw_finish_kernel<__nv_bfloat16><<<(unsigned)blocks, kFinishThreads, smem, st>>>(p);
     note_launch();
-    return cudaGetLastError();
-  }
-  const int64_t H = a.H, W = a.W;
-  const int64_t edge = edge_pixels(H, W);
-  const int64_t total = a.N * a.C * edge;
-  const int threads = 128;
-  const int64_t blocks = std::min<int64_t>((total + threads - 1) / threads, 65535);
-  if (a.dtype == 0)
-    dw_fixup_kernel<float><<<(unsigned)blocks, threads, 0, st>>>(
-        static_cast<const float*>(a.dy), a.w, static_cast<float*>(a.dx), (int)a.C, (int)H,
-        (int)W, a.K, edge, total);
-  else
-    dw_fixup_kernel<__nv_bfloat16><<<(unsigned)blocks, threads, 0, st>>>(
-        static_cast<const __nv_bfloat16*>(a.dy), a.w, static_cast<__nv_bfloat16*>(a.dx),
-        (int)a.C, (int)H, (int)W, a.K, edge, total);
-  note_launch();
-  return cudaGetLastError();
-}
-
-// ------------------------------------------------------ FP64 reduction
-// One warp per (channel, tap): lanes stride over the (image, chunk) partials
-// in a fixed order, accumulate in FP64 and combine with a fixed butterfly, so
-// the result does not depend on scheduling.
-__global__ void dw_finalize_kernel(const float* __restrict__ partials, float* __restrict__ dw,
-                                   int64_t N, int C, int64_t chunks, int KK) {
-  const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (gw >= (int64_t)C * KK) return;
-  const int c = (int)(gw / KK), k = (int)(gw % KK);
-  double s = 0.0;
-  const int64_t count = N * chunks;
-  // idx = n * chunks + ch advances by 32 = step_n * chunks + step_ch: one
-  // division per lane instead of a 64-bit division per partial
-  int64_t n = lane / chunks, ch = lane - (lane / chunks) * chunks;
-  const int64_t step_n = 32 / chunks, step_ch = 32 - step_n * chunks;
-  for (int64_t idx = lane; idx < count; idx += 32) {
-    s += (double)partials[((n * C + c) * chunks + ch) * KK + k];
-    n += step_n;
-    ch += step_ch;
-    if (ch >= chunks) {
-      ch -= chunks;
-      ++n;
-    }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) dw[(int64_t)c * KK + k] = (float)s;
-}
-
-cudaError_t dw_finalize_launch(const DwArgs& a, int64_t chunks_per_plane, cudaStream_t st) {
-  const int KK = a.K * a.K;
-  const int64_t warps = a.C * KK;
-  const int threads = 256;
-  const int64_t blocks = (warps * 32 + threads - 1) / threads;
-  dw_finalize_kernel<<<(unsigned)blocks, threads, 0, st>>>(a.partials, a.dw, a.N, (int)a.C,
-                                                           chunks_per_plane, KK);
-  note_launch();
-  return cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    p.plane0 += now;
+    p.sum_blocks = 0;
+    blocks = 0;
+  } while (p.plane0 < planes);
+  return cudaSuccess;
 }
 
 }  // namespace giga
