@@ -49,13 +49,23 @@ def _require_cuda(*ts):
             raise ValueError("tensors must be contiguous")
 
 
+# The current stream of a device as an integer: the handle alone, without the
+# Stream object that torch.cuda.current_stream builds (2.0 us a call on the
+# Grace host against 0.1 us).
+_raw_stream = torch._C._cuda_getCurrentRawStream
+
+
 def _stream(device) -> int:
-    return torch.cuda.current_stream(device).cuda_stream
+    index = device.index
+    if index is None:
+        return torch.cuda.current_stream(device).cuda_stream
+    return _raw_stream(index)
 
 
 def dw_desc(x: torch.Tensor, K: int, border) -> _lib.giga_conv2d_desc_t:
     N, C, H, W = x.shape
-    return _lib.desc(N, C, C, H, W, K, C, _border(border), _dtype(x), _lib.GIGA_LAYOUT_NCHW)
+    return _lib.giga_conv2d_desc_t(N, C, C, H, W, K, C, _border(border), _dtype(x),
+                                   _lib.GIGA_LAYOUT_NCHW, 0)
 
 
 def workspace(d: _lib.giga_conv2d_desc_t, ops: int, device) -> torch.Tensor | None:
@@ -78,8 +88,8 @@ def conv2d_fwd(x: torch.Tensor, w: torch.Tensor, border="zero", out=None) -> tor
     _require_cuda(x, w)
     d = dw_desc(x, w.shape[-1], border)
     y = torch.empty_like(x) if out is None else out
-    ws = workspace(d, _lib.GIGA_OP_FWD, x.device)
-    _lib.check(_lib.giga_conv2d_fwd(d, _ptr(x), _ptr(w), _ptr(y), _ptr(ws), _nbytes(ws),
+    # the depthwise forward needs no workspace
+    _lib.check(_lib.giga_conv2d_fwd(d, x.data_ptr(), w.data_ptr(), y.data_ptr(), None, 0,
                                     _stream(x.device)), "giga_conv2d_fwd")
     return y
 
@@ -160,10 +170,9 @@ def conv2d_bwd_input(dy: torch.Tensor, w: torch.Tensor, border="zero", out=None)
     _require_cuda(dy, w)
     d = dw_desc(dy, w.shape[-1], border)
     dx = torch.empty_like(dy) if out is None else out
-    ws = workspace(d, _lib.GIGA_OP_BWD_INPUT, dy.device)
-    _lib.check(_lib.giga_conv2d_bwd_input(d, _ptr(dy), _ptr(w), _ptr(dx), _ptr(ws),
-                                          _nbytes(ws), _stream(dy.device)),
-               "giga_conv2d_bwd_input")
+    # the depthwise input gradient needs no workspace
+    _lib.check(_lib.giga_conv2d_bwd_input(d, dy.data_ptr(), w.data_ptr(), dx.data_ptr(), None, 0,
+                                          _stream(dy.device)), "giga_conv2d_bwd_input")
     return dx
 
 

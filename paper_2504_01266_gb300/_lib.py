@@ -147,6 +147,8 @@ _SIGS = {
 def load(path: str | None = None):
     """Load libgiga.so (raises if it has not been built)."""
     global _lib
+    if _lib is not None:  # set once, never cleared: no lock on the calls' path
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib

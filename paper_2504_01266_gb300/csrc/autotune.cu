@@ -196,6 +196,7 @@ static void ensure_loaded() {
 int tune_lookup(int op, const DwArgs& a) {
   std::lock_guard<std::mutex> lk(g_mu);
   ensure_loaded();
+  if (g_cache.empty()) return -1;
   auto it = g_cache.find(key_of(op, a));
   if (it == g_cache.end()) return -1;
   return it->second < tune_candidates(op) ? it->second : -1;
