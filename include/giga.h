@@ -326,7 +326,9 @@ giga_status_t giga_gray_conv2d_fwd(const giga_conv2d_desc_t* desc, const void* x
  * 4, 8, 16}, id 5 = two passes (input gradient by the forward-style kernel
  * in the forward's tuned configuration, filter gradient by the filter
  * kernel), id 6 = one persistent kernel whose CTAs stream (x, dy) tile pairs
- * through a ring of two or three stages (the HBM-bound small filters).  The built-in default is id 0.
+ * through a ring of two or three stages (the HBM-bound small filters).
+ * Without a stored choice a built-in rule picks the configuration from the
+ * filter size, the type, the alignment and the problem size.
  * Modes (also from the environment variable GIGA_AUTOTUNE=off|cached|full):
  *   0 off:    always the built-in default configuration;
  *   1 cached: use a cached choice when one exists (default);
@@ -344,8 +346,8 @@ int32_t giga_autotune_get_mode(void);
 giga_status_t giga_autotune_conv2d(const giga_conv2d_desc_t* desc, int32_t ops, const void* x,
                                    const void* w, void* y, const void* dy, void* dx, float* dw,
                                    void* ws, size_t ws_bytes, void* stream);
-/* The configuration id the entry points will use for (desc, op): the cached
- * choice, else 0; -1 on error. */
+/* The configuration id stored for (desc, op), which the entry points will use;
+ * 0 if there is none (the built-in rule then decides); -1 on error. */
 int32_t giga_autotune_choice(const giga_conv2d_desc_t* desc, int32_t op);
 /* Pin configuration `id` for (desc's problem class, op) in the cache, as if
  * the tuner had chosen it; used in modes 1 and 2.  GIGA_ERR_INVALID_ARG for

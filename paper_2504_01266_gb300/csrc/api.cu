@@ -230,8 +230,9 @@ giga_status_t run_dw_op(int op, const DwArgs& a, const DwConfig& cfg, cudaStream
         // best kernel (faster for the ALU-bound large filters)
         // the input-gradient pass runs the forward kernel on a problem of the
         // same shape: take the forward's tuned configuration
-        int fid = tune_mode() == 0 ? 0 : tune_lookup(TUNE_FWD, a);
-        DwConfig fc = tune_config(TUNE_FWD, fid < 0 ? 0 : fid, a);
+        const int fid = tune_mode() == 0 ? -1 : tune_lookup(TUNE_FWD, a);
+        const DwConfig fc =
+            fid < 0 ? default_config(TUNE_BWD_INPUT, a) : tune_config(TUNE_FWD, fid, a);
         e = dispatch_k(a.K, [&](auto k) { return dw_fwd_launch<decltype(k)::value>(a, fc, true, st); });
         if (e == cudaSuccess)
           e = dispatch_k_filter(a.K, [&](auto k) {
@@ -259,14 +260,13 @@ static bool stream_capturing(cudaStream_t st) {
 }
 
 static giga_status_t run_tuned(int op, const DwArgs& a, cudaStream_t st) {
-  int id = tune_mode() == 0 ? 0 : tune_lookup(op, a);
+  int id = tune_mode() == 0 ? -1 : tune_lookup(op, a);
   if (id < 0 && tune_mode() == 2 && !stream_capturing(st)) {
     giga_status_t s = tune_dw_op(op, a, st);
     if (s != GIGA_OK) return s;
     id = tune_lookup(op, a);
   }
-  if (id < 0) id = 0;
-  return run_dw_op(op, a, tune_config(op, id, a), st);
+  return run_dw_op(op, a, id < 0 ? default_config(op, a) : tune_config(op, id, a), st);
 }
 
 }  // namespace giga

@@ -122,6 +122,52 @@ DwConfig tune_config(int op, int id, const DwArgs& a) {
   return c;
 }
 
+// Without a stored choice the configuration follows from the filter size, the
+// storage type, the planes' alignment and the number T of 64 x 128 tiles
+// against the S SMs (S = 152; times in us, candidate 0 -> the choice):
+//  * forward and input gradient, T <= 2 S: 32-row tiles, because 64-row tiles
+//    leave SMs with no CTA or one (512^2 K = 21: 24 -> 15, K = 31: 46 -> 26;
+//    3 x 300 x 401 K = 15: 19 -> 15; 3 x 1080 x 1920, T = 5 S: equal).
+//    Above: the L2 prefetch where the tile load shows -- aligned FP32 K = 7, 9
+//    (16 x 3 x 2048^2: 380 -> 368, 573 -> 554) and BF16 K <= 3 (197 -> 179);
+//    FP32 K = 3 loses by it (230 -> 253), the others are equal.
+//  * both gradients:
+//    K <= 3, aligned planes, T >= 4 S: the tile ring (16 x 3 x 2048^2 FP32
+//    433 -> 384, BF16 387 -> 269; 3 x 1080 x 1920, T = 5 S: 24 -> 25, 26 -> 23;
+//    unaligned planes 167 -> 212, where its one CTA per SM stages with the
+//    warps that compute);
+//    K >= 11, T >= 2 S: two passes (3 x 1080 x 1920 K = 11: 94 -> 86, K = 15:
+//    153 -> 125; 4 x 3 x 1801 x 2400 K = 15: 1140 -> 802; T = S / 2: 29 -> 31);
+//    K = 9 (FP32: aligned) and BF16 K = 7, T >= 16 S: two passes
+//    (16 x 3 x 2048^2 FP32 K = 9 1279 -> 1246, BF16 K = 9 1374 -> 1309, K = 7
+//    923 -> 880; at T = 5 S 62 -> 64, 47 -> 52).
+DwConfig default_config(int op, const DwArgs& a) {
+  DwConfig c = tune_config(op, 0, a);
+  const int64_t S = sm_count();
+  const int64_t T = a.N * a.C * ((a.W + kTileW - 1) / kTileW) * ((a.H + 63) / 64);
+  const bool f32 = a.dtype == 0;
+  const bool aligned = a.vec && a.W % (f32 ? 4 : 8) == 0;
+  switch (op) {
+    case TUNE_FWD:
+    case TUNE_BWD_INPUT:
+      if (T <= 2 * S)
+        c.rows_per_thread = 4;
+      else
+        c.prefetch = aligned && (f32 ? a.K == 7 || a.K == 9 : a.K <= 3);
+      break;
+    case TUNE_BWD_FUSED: {
+      const bool ring = a.K <= 3 && aligned && T >= 4 * S;
+      const bool split = (a.K >= 11 && T >= 2 * S) ||
+                         (((a.K == 9 && (aligned || !f32)) || (a.K == 7 && !f32)) && T >= 16 * S);
+      if (ring || split) c = tune_config(op, split ? 5 : 6, a);
+      break;
+    }
+    default:
+      break;
+  }
+  return c;
+}
+
 static std::string key_of(int op, const DwArgs& a) {
   const double n = (double)a.N * a.C * a.H * a.W;
   const int sc = n > 0 ? (int)std::floor(std::log2(n)) : 0;
