@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1)
 // the last one, so the pair (last slot, slot 0) is adjacent too.  D
 // accumulates in TMEM over all chunks of the CTA (2 x 192 columns); each CTA
 // then writes its FP32 partial sums [tap][c][o] and a second kernel adds the
-// CTAs' partials in FP64 in CTA order.
+// CTAs' partials in a fixed order (two-float and FP64 sums).
 constexpr int kWgTileP = 64;                           // pixel positions per chunk (MMA K: 4 x 16)
 constexpr int kWgXPx = kWgTileP + 1;                   // x band: 65 pixels
 constexpr int kWgDyPx = kWgTileP + 2;                  // dy band: 66 pixels
@@ -687,18 +687,35 @@ __global__ void __launch_bounds__(kDenseThreads, 1)
   }
 }
 
-// dw[o][a][b][c] = sum over CTAs (in order, FP64) of partial[cta][3a + b][c][o].
-__global__ void dense_wgrad_finalize_kernel(const float* __restrict__ partials, int ctas,
-                                            float* __restrict__ dw) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= kDenseC * kDenseTaps * kDenseC) return;
-  const int c = idx % kDenseC;
-  const int tap = (idx / kDenseC) % kDenseTaps;
-  const int o = idx / (kDenseC * kDenseTaps);
-  double s = 0.0;
-  for (int b = 0; b < ctas; ++b)
-    s += (double)partials[(int64_t)b * kWgPartialFloats + ((int64_t)tap * kDenseC + c) * kDenseC + o];
-  dw[idx] = (float)s;
+// dw[o][a][b][c] = sum over CTAs, in a fixed order, of partial[cta][3a + b][c][o].
+// A block takes one (tap, c): 64 lanes across o read whole lines of a partial,
+// four groups of them take every fourth CTA in two-float sums, and the groups
+// add in FP64.  22 MB of partials come from L2 whatever the image size.  One
+// thread per output in dw's order read a 32-byte sector per value and added
+// 152 FP64 values in sequence: 26 us.
+constexpr int kWgFinGroups = 4;
+__global__ void __launch_bounds__(kDenseC * kWgFinGroups)
+    dense_wgrad_finalize_kernel(const float* __restrict__ partials, int ctas,
+                                float* __restrict__ dw) {
+  __shared__ double part[kWgFinGroups][kDenseC];
+  const int o = threadIdx.x % kDenseC, g = threadIdx.x / kDenseC;
+  const int tap = blockIdx.x / kDenseC, c = blockIdx.x % kDenseC;
+  const float* src = partials + ((int64_t)tap * kDenseC + c) * kDenseC + o;
+  TwoFloatSum sum;
+#pragma unroll 8
+  for (int b = g; b < ctas; b += kWgFinGroups) sum.add(__ldg(src + (int64_t)b * kWgPartialFloats));
+  double s = sum.value();
+  if (!isfinite(s)) {  // infinities, NaN or an overflow on the way
+    s = 0.0;
+    for (int b = g; b < ctas; b += kWgFinGroups) s += (double)__ldg(src + (int64_t)b * kWgPartialFloats);
+  }
+  part[g][o] = s;
+  __syncthreads();
+  if (g == 0) {
+#pragma unroll
+    for (int q = 1; q < kWgFinGroups; ++q) s += part[q][o];
+    dw[((int64_t)o * kDenseTaps + tap) * kDenseC + c] = (float)s;
+  }
 }
 
 // dgrad filter: wt[c][a][b][o] = w[o][2 - a][2 - b][c] (rotate the taps,
@@ -777,8 +794,8 @@ cudaError_t dense_wgrad_launch(const void* x, const void* dy, float* dw, int64_t
   dense_wgrad_kernel<<<grid, kDenseThreads, kWgSmem, st>>>(tx, tdy, prm);
   note_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  const int n = kDenseC * kDenseTaps * kDenseC;
-  dense_wgrad_finalize_kernel<<<(n + 255) / 256, 256, 0, st>>>(prm.partials, grid, dw);
+  dense_wgrad_finalize_kernel<<<kDenseTaps * kDenseC, kDenseC * kWgFinGroups, 0, st>>>(
+      prm.partials, grid, dw);
   note_launch();
   return cudaGetLastError();
 }
