@@ -7,15 +7,16 @@
 //    64 x 128 pixels (1 to 32, powers of 2: the plan's autotuner times them) and
 //    sorts the chunks longest first (cost K^2 per pixel);
 //  * CTAs (one per SM, 16 warps) pull chunk numbers from an atomic counter,
-//    stage each tile's x and dy once, and run the three ops on it with fixed
-//    warp roles: warps 0-3 forward, 4-7 input gradient, 8-15 filter gradient.
-//    The filter gradient's per-pixel work equals each other role's, but its
-//    inner loop reaches a lower FMA rate; for K >= 11 all 8 of its warps work
-//    (in groups of at most 3 filter rows, so the union of the filter-size
-//    bodies fits the 128 registers a thread of a 16-warp CTA has) and the
-//    three roles finish a tile at about the same time; for K <= 9, where the
-//    forward and input-gradient roles bound the tile, 4 of them work (the
-//    other 4 stage and synchronise only: 8 working warps measured no faster);
+//    stage each tile's x and dy once, and run the three ops on it: warps 0-7
+//    the forward and warps 8-15 the input gradient, 8 rows each, then all 16
+//    the filter gradient, split into groups of filter rows and tile rows.  The
+//    three cost the same per pixel, so every warp has the same work between
+//    the tile's barriers, and a scheduler has four busy warps throughout.
+//    (With fixed roles -- 4 warps forward, 4 input gradient, 4 or 8 filter
+//    gradient -- the warps of the slowest role ran alone at a tile's end, and 4
+//    of the 16 idled for K <= 9.  One 3 x 2001 x 2999 image, that -> this: K = 3
+//    155 -> 109 us, K = 5 184 -> 137, K = 9 301 -> 258, K = 11 380 -> 333, BF16 K = 3
+//    224 -> 129, K = 11 472 -> 397; forward alone K = 11 165 -> 126.)
 //  * each chunk writes one K*K vector of FP32 filter-gradient partials; the
 //    CTA that completes the last chunk of an (image, channel) -- detected with
 //    a per-(image, channel) atomic counter after a memory fence -- sums that
@@ -29,7 +30,7 @@
 namespace giga {
 
 constexpr int kRagThreads = 512;
-constexpr int kRagDwWarps = 8;  // filter-gradient warps (warps 8-15)
+constexpr int kRagWarps = kRagThreads / 32;
 constexpr int kRagTilesPerChunk = 4;  // the plan's default; the autotuner may pick 1 to 32
 constexpr int kRagMaxK = 15;
 
@@ -63,28 +64,24 @@ struct RagParams {
   int border;
 };
 
-// Filter-row groups of the 8 filter-gradient warps for K >= 11: fewer rows
-// per warp keep the accumulators within the 128 registers a thread of a
-// 16-warp CTA has (K = 11: 4 groups of at most 3 rows; K >= 13: 8 groups of
-// at most 2 rows, one warp each).
+// Filter-row groups of the filter gradient: as few as keep a warp's
+// accumulators (rows of the group x K) beside the forward's within the 128
+// registers a thread of a 16-warp CTA has.
 template <int K>
 constexpr int rag_groups() {
-  return K <= 7 ? 1 : (K <= 9 ? 2 : (K <= 11 ? 4 : 8));
-}
-// filter-gradient warps that work for this K (the others only stage and sync)
-template <int K>
-constexpr int rag_dw_active() {
-  return K <= 9 ? 4 : 8;
+  return K <= 5 ? 1 : (K <= 9 ? 2 : (K <= 11 ? 4 : 8));
 }
 
 template <int K, typename T>
 struct RagShape {
   using G = Geo<K, sizeof(T), true>;
-  static constexpr int GT = K <= 9 ? dw_groups<K>() : rag_groups<K>();
-  static constexpr int WPG = rag_dw_active<K>() / GT;
+  static constexpr int GT = rag_groups<K>();
+  static constexpr int WPG = kRagWarps / GT;
   static constexpr int AT = (K + GT - 1) / GT;
   static constexpr int DW_ROWS = kBwdTileH / WPG;
+  static constexpr int DR = 4;                      // dy rows per unrolled block
   static constexpr int ROWS = kBwdTileH + 2 * G::R;
+  static_assert(DW_ROWS % DR == 0, "whole row blocks");
 };
 
 // Shared memory, sized for the largest filter: two tile stages (x and dy
@@ -99,14 +96,14 @@ struct RagLayout {
   static constexpr int WB = G::WPAD * 4;          // one filter
   static constexpr int FILT = 2 * STAGE;          // [2][w, wf]
   static constexpr int RED = FILT + 4 * WB;       // [2 chunks][w, wf] filters
-  static constexpr int RED_FLOATS = 66;           // K = 11: 6 rows x 11 taps
-  // the row buffers of the 8 forward / input-gradient warps (store_rows) share
-  // the reduction rows' space: those are used at a chunk's end, behind barriers
+  static constexpr int RED_FLOATS = 45;           // K = 9: 5 rows x 9 taps
+  // the row buffers of store_rows, one per warp, share the reduction rows'
+  // space: those are used at a chunk's end, behind barriers
   static constexpr int BUF = RED;
-  static constexpr int INTS =
-      RED + (kRagDwWarps * RED_FLOATS * 4 > 8 * kRowBuf ? kRagDwWarps * RED_FLOATS * 4 : 8 * kRowBuf);
+  static constexpr int INTS = RED + kRagWarps * kRowBuf;
   static constexpr int SM_BYTES = INTS + 16;
-  static_assert(RagShape<11, T>::AT * 11 <= RED_FLOATS && RagShape<15, T>::AT * 15 <= RED_FLOATS,
+  static_assert(RagShape<9, T>::AT * 9 <= RED_FLOATS && RagShape<11, T>::AT * 11 <= RED_FLOATS &&
+                    RagShape<15, T>::AT * 15 <= RED_FLOATS && RED_FLOATS * 4 <= kRowBuf,
                 "reduction rows");
   static_assert(SM_BYTES <= 227 * 1024, "shared memory");
 };
@@ -149,14 +146,70 @@ __device__ __forceinline__ void rag_stage(const RagParams& p, const RagChunk& ch
   }
 }
 
+// Chunk c has written its outputs and partials.  The CTA that completes the
+// last chunk of an (image, channel) sums its filter gradient and, for the
+// clamp border, folds the edges of dx.  It runs once per chunk, outside the
+// filter sizes' bodies (K known at run time): inlined into each of them the
+// sums cost the tile loops registers (seven K = 11 images 2.82 -> 2.91 ms).
+template <typename T>
+__device__ __forceinline__ void rag_complete(const RagParams& p, int c, double* ps, int* s_flag) {
+  const bool do_dw = p.ops & 4, folds = (p.ops & 2) && p.border == 1;
+  if (do_dw || folds) {
+    __threadfence();
+    cta_barrier();
+    const RagChunk ch = p.chunks[c];
+    const RagImage im = p.images[ch.image];
+    if (threadIdx.x == 0)
+      *s_flag = atomicAdd(p.counters + 1 + im.ic_base + ch.channel, 1) == im.nch - 1;
+    cta_barrier();
+    if (*s_flag) {
+      __threadfence();
+      const int K = im.K, KK = K * K;
+      if (do_dw) {
+        // every tap's partials by GR threads, each every GR-th chunk, in
+        // two-float sums; then their FP64 values in order (one thread per tap
+        // adding FP64 took about 20 us of a CTA's time: 3 x 2001 x 3000 K = 3
+        // 124 -> 99 us)
+        const float* part = p.partials + im.partial_base + (int64_t)ch.channel * im.nch * KK;
+        const int GR = min(kRagThreads / KK, 16);
+        const int k = threadIdx.x % KK, q = threadIdx.x / KK;
+        if (q < GR) {
+          TwoFloatSum sum;
+#pragma unroll 8
+          for (int j = q; j < im.nch; j += GR) sum.add(__ldcg(part + (int64_t)j * KK + k));
+          double s = sum.value();
+          if (!isfinite(s)) {  // infinities, NaN or an overflow on the way
+            s = 0.0;
+            for (int j = q; j < im.nch; j += GR) s += (double)__ldcg(part + (int64_t)j * KK + k);
+          }
+          ps[q * KK + k] = s;
+        }
+        cta_barrier();
+        if (threadIdx.x < KK) {
+          double s = 0.0;
+          for (int g = 0; g < GR; ++g) s += ps[g * KK + threadIdx.x];
+          im.dw[(int64_t)ch.channel * KK + threadIdx.x] = (float)s;
+        }
+      }
+      if (folds) {
+        const int64_t off = (int64_t)ch.channel * im.H * im.W;
+        const int64_t edges = edge_pixels(im.H, im.W);
+        for (int64_t e = threadIdx.x; e < edges; e += kRagThreads)
+          fold_edge_pixel<T>(static_cast<const T*>(im.dy) + off, im.w + (int64_t)ch.channel * KK,
+                             static_cast<T*>(im.dx) + off, im.H, im.W, K, e);
+      }
+    }
+  }
+  cta_barrier();  // sm_red and s_flag are reused by the next chunk
+}
+
 // One chunk: its first tile is already in stage sb (copies in flight), its
 // filters in filter buffer fb.  While tile t is computed, the copies of the
 // next tile -- the next of this chunk, or the first of chunk `cn` -- go to
 // the other stage.  Returns the stage holding the next chunk's first tile.
 template <typename T, int K>
 __device__ __forceinline__ int rag_chunk(const RagParams& p, const RagChunk& ch,
-                                         const RagImage& im, int cn, char* sm, int sb, int fb,
-                                         int* s_flag) {
+                                         const RagImage& im, int cn, char* sm, int sb, int fb) {
   using G = Geo<K, sizeof(T), true>;
   using S = RagShape<K, T>;
   using L = RagLayout<T>;
@@ -172,11 +225,9 @@ __device__ __forceinline__ int rag_chunk(const RagParams& p, const RagChunk& ch,
   const bool clamp = p.border == 1, vec = im.vec != 0;
   T* yp = do_fwd ? static_cast<T*>(im.y) + off : nullptr;
   T* dxp = do_dx ? static_cast<T*>(im.dx) + off : nullptr;
-  const float* wc = (do_fwd || do_dx) ? im.w + (int64_t)ch.channel * KK : nullptr;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int role = warp < 8 ? warp >> 2 : 2, wl = warp < 8 ? (warp & 3) : warp - 8;
-  const int g = wl % S::GT;
-  const int part = wl / S::GT;
+  const int g = warp % S::GT;
+  const int part = warp / S::GT;
   const int a_lo = group_lo(g, K, S::GT);
   const int nrows = group_lo(g + 1, K, S::GT) - a_lo;
   float acc[S::AT][K];
@@ -211,27 +262,22 @@ __device__ __forceinline__ int rag_chunk(const RagParams& p, const RagChunk& ch,
         (ty0 - G::R < 0 || ty0 + kBwdTileH + G::R > H || tx0 - G::RP < 0 ||
          tx0 + kTileW + G::RP > W))
       clamp_fix<T, G::SP, kRagThreads>(sx, H, W, ty0, tx0, G::R, G::RP, S::ROWS);
-    if (role < 2) {
-      if (role == 0 ? do_fwd : do_dx) {
-        const T* src = role == 0 ? sx : sdy;
-        const float* f = role == 0 ? sm_w : sm_wf;
-        T* dst = role == 0 ? yp : dxp;
-        constexpr int BR = bwd_block_rows<K>();
-#pragma unroll 1
-        for (int pass = 0; pass < 16 / BR; ++pass) {
-          const int r0 = wl * 16 + pass * BR;
-          float o[BR][4];
-          fwd_block<K, BR, T, true>(src + r0 * G::SP + 4 * lane, f, o);
-          store_tile<T, BR, false>(dst, H, W, ty0 + r0, tx0, vec,
-                                   reinterpret_cast<float*>(sm + L::BUF + warp * kRowBuf), o);
-        }
-      }
-    } else if (do_dw && wl < rag_dw_active<K>()) {
-      constexpr int BR = bwd_block_rows<K>();
-      const int r0 = part * S::DW_ROWS;
-      dw_rows<K, S::AT, S::GT, G::SP, BR, T, true>(sdy + (r0 + G::R) * G::SP + G::RP + 4 * lane,
-                                             sx + (r0 + a_lo) * G::SP + 4 * lane,
-                                             S::DW_ROWS / BR, nrows, acc);
+    const int r8 = (warp & 7) * 8;
+    if ((warp < 8 ? do_fwd : do_dx) && ty0 + r8 < H) {
+      const T* src = warp < 8 ? sx : sdy;
+      const float* f = warp < 8 ? sm_w : sm_wf;
+      T* dst = warp < 8 ? yp : dxp;
+      float o[8][4];
+      fwd_block<K, 8, T, true>(src + r8 * G::SP + 4 * lane, f, o);
+      store_tile<T, 8, false>(dst, H, W, ty0 + r8, tx0, vec,
+                              reinterpret_cast<float*>(sm + L::BUF + warp * kRowBuf), o);
+    }
+    if (do_dw) {
+      const int r0 = part * S::DW_ROWS;  // dy rows below the image are zero: skipped
+      const int nb = min(S::DW_ROWS / S::DR, (H - ty0 - r0 + S::DR - 1) / S::DR);
+      dw_rows<K, S::AT, S::GT, G::SP, S::DR, T, true>(
+          sdy + (r0 + G::R) * G::SP + G::RP + 4 * lane, sx + (r0 + a_lo) * G::SP + 4 * lane, nb,
+          nrows, acc);
     }
     cta_barrier();  // stage sb is free for the copies two tiles ahead
     sb ^= 1;
@@ -239,7 +285,7 @@ __device__ __forceinline__ int rag_chunk(const RagParams& p, const RagChunk& ch,
 
   // filter-gradient partial of this chunk: warp butterflies, then a fixed-order
   // sum over the group's warps
-  if (role == 2 && do_dw && wl < rag_dw_active<K>()) {
+  if (do_dw) {
 #pragma unroll
     for (int s = 0; s < S::AT; ++s)
 #pragma unroll
@@ -247,11 +293,10 @@ __device__ __forceinline__ int rag_chunk(const RagParams& p, const RagChunk& ch,
         float v = acc[s][b];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) sm_red[wl * L::RED_FLOATS + s * K + b] = v;
+        if (lane == 0) sm_red[warp * L::RED_FLOATS + s * K + b] = v;
       }
   }
   cta_barrier();
-  const int ic = im.ic_base + ch.channel;
   float* part_c = p.partials + im.partial_base + (int64_t)ch.channel * im.nch * KK;
   if (do_dw) {
     const int j = ch.tile_begin / p.tpc;
@@ -265,29 +310,7 @@ __device__ __forceinline__ int rag_chunk(const RagParams& p, const RagChunk& ch,
       part_c[(int64_t)j * KK + k] = sum;
     }
   }
-  if (do_dw || (do_dx && clamp)) {
-    __threadfence();
-    cta_barrier();
-    if (threadIdx.x == 0) *s_flag = atomicAdd(p.counters + 1 + ic, 1) == im.nch - 1;
-    cta_barrier();
-    if (*s_flag) {
-      __threadfence();
-      if (do_dw) {
-        for (int k = threadIdx.x; k < KK; k += kRagThreads) {
-          double s = 0.0;
-          for (int j = 0; j < im.nch; ++j) s += (double)__ldcg(part_c + (int64_t)j * KK + k);
-          im.dw[(int64_t)ch.channel * KK + k] = (float)s;
-        }
-      }
-      if (do_dx && clamp) {
-        const int64_t edges = edge_pixels(H, W);
-        const T* gsrc = static_cast<const T*>(im.dy) + off;
-        for (int64_t e = threadIdx.x; e < edges; e += kRagThreads)
-          fold_edge_pixel<T>(gsrc, wc, dxp, H, W, K, e);
-      }
-    }
-  }
-  cta_barrier();  // sm_red and s_flag are reused by the next chunk
+  __threadfence();  // before the completion count that follows the caller's next barrier
   return sb;
 }
 
@@ -317,15 +340,16 @@ __global__ void __launch_bounds__(kRagThreads, 1) rag_kernel(RagParams p) {
     const RagChunk ch = p.chunks[c];
     const RagImage im = p.images[ch.image];
     switch (im.K) {
-      case 1: sb = rag_chunk<T, 1>(p, ch, im, cn, sm, sb, fb, s_flag); break;
-      case 3: sb = rag_chunk<T, 3>(p, ch, im, cn, sm, sb, fb, s_flag); break;
-      case 5: sb = rag_chunk<T, 5>(p, ch, im, cn, sm, sb, fb, s_flag); break;
-      case 7: sb = rag_chunk<T, 7>(p, ch, im, cn, sm, sb, fb, s_flag); break;
-      case 9: sb = rag_chunk<T, 9>(p, ch, im, cn, sm, sb, fb, s_flag); break;
-      case 11: sb = rag_chunk<T, 11>(p, ch, im, cn, sm, sb, fb, s_flag); break;
-      case 13: sb = rag_chunk<T, 13>(p, ch, im, cn, sm, sb, fb, s_flag); break;
-      default: sb = rag_chunk<T, 15>(p, ch, im, cn, sm, sb, fb, s_flag); break;
+      case 1: sb = rag_chunk<T, 1>(p, ch, im, cn, sm, sb, fb); break;
+      case 3: sb = rag_chunk<T, 3>(p, ch, im, cn, sm, sb, fb); break;
+      case 5: sb = rag_chunk<T, 5>(p, ch, im, cn, sm, sb, fb); break;
+      case 7: sb = rag_chunk<T, 7>(p, ch, im, cn, sm, sb, fb); break;
+      case 9: sb = rag_chunk<T, 9>(p, ch, im, cn, sm, sb, fb); break;
+      case 11: sb = rag_chunk<T, 11>(p, ch, im, cn, sm, sb, fb); break;
+      case 13: sb = rag_chunk<T, 13>(p, ch, im, cn, sm, sb, fb); break;
+      default: sb = rag_chunk<T, 15>(p, ch, im, cn, sm, sb, fb); break;
     }
+    rag_complete<T>(p, c, reinterpret_cast<double*>(sm + L::RED), s_flag);
     if (cn >= p.n_chunks) break;
     c = cn;
     fb ^= 1;
