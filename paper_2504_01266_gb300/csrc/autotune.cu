@@ -131,16 +131,17 @@ DwConfig tune_config(int op, int id, const DwArgs& a) {
 //    Above: the L2 prefetch where the tile load shows -- aligned FP32 K = 7, 9
 //    (16 x 3 x 2048^2: 380 -> 368, 573 -> 554) and BF16 K <= 3 (197 -> 179);
 //    FP32 K = 3 loses by it (230 -> 253), the others are equal.
-//  * both gradients:
-//    K <= 3, aligned planes, T >= 4 S: the tile ring (16 x 3 x 2048^2 FP32
-//    433 -> 384, BF16 387 -> 269; 3 x 1080 x 1920, T = 5 S: 24 -> 25, 26 -> 23;
-//    unaligned planes 167 -> 212, where its one CTA per SM stages with the
-//    warps that compute);
-//    K >= 11, T >= 2 S: two passes (3 x 1080 x 1920 K = 11: 94 -> 86, K = 15:
-//    153 -> 125; 4 x 3 x 1801 x 2400 K = 15: 1140 -> 802; T = S / 2: 29 -> 31);
-//    K = 9 (FP32: aligned) and BF16 K = 7, T >= 16 S: two passes
-//    (16 x 3 x 2048^2 FP32 K = 9 1279 -> 1246, BF16 K = 9 1374 -> 1309, K = 7
-//    923 -> 880; at T = 5 S 62 -> 64, 47 -> 52).
+//  * both gradients, fused kernel -> the choice:
+//    K <= 3, aligned planes: the tile ring from T = 16 S (FP32; 16 x 3 x 2048^2
+//    422 -> 376, at T = 10 S 38.8 -> 40.7) or 4 S (BF16; 378 -> 261, at 5 S 25.7
+//    -> 21.2); its one CTA per SM stages unaligned planes with the warps that
+//    compute (160 -> 207).
+//    Two passes: K >= 13 from T = 2 S (3 x 1080 x 1920 K = 13: 117 -> 106, 4 x 3
+//    x 1801 x 2400: 997 -> 636; K = 15: 860 -> 803); K = 11 from 4 S aligned (86
+//    -> 81), 16 S not (584 -> 572; at 5 S 91 -> 93); K = 9 aligned from 4 S (BF16
+//    67 -> 64, FP32 equal; 4 x 3 x 1024^2 111 -> 103); BF16 K = 7 from 8 S aligned
+//    (75.7 -> 73.3; 16 x 3 x 2048^2 923 -> 807; at 5 S equal), 16 S not (425 ->
+//    402); BF16 K = 5 aligned from 8 S (55 -> 51; at 5 S 34 -> 36).
 DwConfig default_config(int op, const DwArgs& a) {
   DwConfig c = tune_config(op, 0, a);
   const int64_t S = sm_count();
@@ -156,9 +157,19 @@ DwConfig default_config(int op, const DwArgs& a) {
         c.prefetch = aligned && (f32 ? a.K == 7 || a.K == 9 : a.K <= 3);
       break;
     case TUNE_BWD_FUSED: {
-      const bool ring = a.K <= 3 && aligned && T >= 4 * S;
-      const bool split = (a.K >= 11 && T >= 2 * S) ||
-                         (((a.K == 9 && (aligned || !f32)) || (a.K == 7 && !f32)) && T >= 16 * S);
+      const bool ring = a.K <= 3 && aligned && T >= (f32 ? 16 : 4) * S;
+      int64_t from = -1;  // two passes from this many tiles per SM on
+      if (a.K >= 13)
+        from = 2;
+      else if (a.K == 11)
+        from = aligned ? 4 : 16;
+      else if (a.K == 9 && aligned)
+        from = 4;
+      else if (a.K == 7 && !f32)
+        from = aligned ? 8 : 16;
+      else if (a.K == 5 && !f32 && aligned)
+        from = 8;
+      const bool split = from >= 0 && T >= from * S;
       if (ring || split) c = tune_config(op, split ? 5 : 6, a);
       break;
     }

@@ -33,8 +33,8 @@
 //    streams staged x rows past it; each warp owns a fixed group of filter
 //    rows whose FP32 accumulators persist across all tiles of the CTA, so the
 //    cross-lane reduction (warp shuffles) runs once per CTA.  In the fused
-//    backward pass, warps 0-3 compute the input gradient and warps 4-7 the
-//    filter gradient of the same staged tile, so dy and x are read once.
+//    backward pass every warp does its share of both gradients of a staged
+//    tile, so dy and x are read once.
 #pragma once
 
 #include "common.cuh"
@@ -970,52 +970,72 @@ __global__ void __launch_bounds__(kThreads, 5) dw_sep_kernel_hi_occ(
 }
 
 // -------------------------------------------------------------- backward
-// Fused backward: warps 0-3 write g (= dx for the zero border) from the staged
-// dy tile, warps 4-7 accumulate dw from the staged x and dy tiles.  A CTA owns
-// `tpc` consecutive 64 x 128 tiles of one plane and writes one K*K vector of
-// FP32 partial sums to partials[blockIdx.x].  FP32 planes with a 16-byte row
-// stride are staged by two TMA loads per tile (zeros outside the image; under
-// the clamp border the x tile of an edge tile then gets clamp_fix), others by
-// cp.async with the border applied.
+// Fused backward: the 8 warps accumulate dw from the staged x and dy tiles,
+// split into groups of filter rows and tile rows, then write g (= dx for the
+// zero border) from the dy tile, 8 rows each, so every warp has the same work
+// between a tile's barriers.  (With 4 warps for each gradient the slower role's
+// warps ran alone at a tile's end: 4 x 3 x 1801 x 2400 K = 5 161 -> 150 us, K =
+// 15 1140 -> 860; 4 x 3 x 1801 x 2399 K = 5 227 -> 206, K = 9 442 -> 413, BF16
+// K = 9 672 -> 571.)  A CTA owns `tpc` consecutive 64 x
+// 128 tiles of one plane and writes one K*K vector of FP32 partial sums to
+// partials[blockIdx.x].  Aligned planes are staged by two TMA loads per tile
+// (zeros outside the image), others by stage_any; under the clamp border the x
+// tile of an edge tile then gets clamp_fix.
+
+// How the fused backward is compiled, by filter size, type and alignment (us
+// on 16 x 3 x 2048^2 unless stated):
+//  * groups of filter rows: as few as keep the accumulators in registers.
+//    FP32 K = 7 with three CTAs of 80 registers takes 2 (771; one group and two
+//    CTAs 877), unaligned, where two CTAs fit better, 1 (1016, against 1113).
+//  * rows per unrolled block of the dx and dw bodies, and whether blocks below
+//    the image are skipped (it costs registers where they are tight: BF16 K = 5
+//    542 -> 579, FP32 K = 7 771 -> 789, K = 9 1224 -> 1295 with 8-row dx
+//    blocks; it gains at odd heights).
+//  * CTAs per SM: three where the registers allow, so that more loads are in
+//    flight (K = 3 304, against 368 with two).
+template <int K, typename T, bool AL>
+struct BwdTune {
+  static constexpr bool F32 = sizeof(T) == 4;
+  static constexpr int GROUPS =
+      K <= 5 ? 1 : (K == 7 ? (F32 && AL ? 2 : 1) : (K == 9 ? 2 : (K <= 13 ? 4 : 8)));
+  static constexpr int DX_ROWS = (K == 7 && F32) || K == 9 ? 4 : 8;
+  static constexpr int DW_ROWS = K <= 3 || (K == 5 && !AL) || (K == 7 && !F32) ? 8 : 4;
+  static constexpr bool SKIP = K <= 3 || (K == 5 && F32) || (K == 7 && !AL);
+  static constexpr int MIN_CTAS = K <= 3 || (AL && (K == 5 || (K == 7 && F32))) ? 3 : 2;
+};
+
 template <int K, typename T, bool AL>
 struct BwdShape {
   using G = GeoC<K, T, !AL>;  // FP32 compute geometry
-  static constexpr int NDX = 4;
-  static constexpr int NDW = kWarps - NDX;
-  static constexpr int GT = dw_groups<K>();
-  static constexpr int WPG = NDW / GT;              // warps per filter-row group
+  using Tune = BwdTune<K, T, AL>;
+  static constexpr int GT = Tune::GROUPS;
+  static constexpr int WPG = kWarps / GT;           // warps per filter-row group
   static constexpr int AT = (K + GT - 1) / GT;      // max filter rows per group
-  static constexpr int DW_ROWS = kBwdTileH / WPG;   // tile rows per dw warp
+  static constexpr int DW_ROWS = kBwdTileH / WPG;   // tile rows per warp (dw)
+  static constexpr int BX = Tune::DX_ROWS, BW = Tune::DW_ROWS;
   static constexpr int ROWS = kBwdTileH + 2 * G::R;  // x and dy tiles, both with the halo
   using ST = HaloTile<K, T, ROWS, !AL>;
   // byte offsets: mbarrier and abort flag, the FP32 x and dy tiles (staged
   // tiles at ST::STAGE_OFF inside them, 128-byte aligned for TMA), flipped
   // filter and reduction
-  static constexpr int SM_X = 128 + (AL ? 0 : NDX * kRowBuf);  // row buffers of the dx warps
+  static constexpr int SM_X = 128;
   static constexpr int SM_DY = SM_X + ST::BYTES;
   static constexpr int SM_W = SM_DY + ST::BYTES;
-  // the warps' filter-gradient sums are written after every warp has left the
-  // tile loop, so they reuse the x tile's space (3 CTAs per SM fit at K = 7)
+  // The x tile is dead once every warp has accumulated dw: the row buffers of
+  // store_rows use its space then (behind a barrier, so that 3 CTAs per SM
+  // fit), and after the tile loop the warps' filter-gradient sums.
+  static constexpr int SM_BUF = SM_X;
   static constexpr int SM_RED = SM_X;
   static constexpr int SM_BYTES = SM_W + G::WPAD * 4;
-  static_assert(NDW * AT * K * 4 <= ST::BYTES, "reduction rows fit the x tile");
-  static_assert(NDW % GT == 0, "filter-row groups must divide the dw warps");
-  static_assert(kBwdTileH % (WPG * 8) == 0, "dw warps own whole 8-row blocks");
-  static_assert(16 % bwd_block_rows<K>() == 0, "input-gradient warps own 16 rows");
+  static_assert(kWarps * AT * K * 4 <= ST::BYTES && kWarps * kRowBuf <= ST::BYTES,
+                "reduction rows and row buffers fit the x tile");
+  static_assert(kWarps % GT == 0 && DW_ROWS % BW == 0 && 8 % BX == 0, "whole row blocks");
 };
 
 __device__ __forceinline__ int group_lo(int g, int K, int GT) { return g * K / GT; }
 
-// CTAs per SM the backward kernel is compiled for: the small-K instances are
-// memory-bound and need fewer registers, so a third CTA adds loads in flight.
-// (The general FP32 K = 7 kernel's row buffers leave room for two.)
 template <typename T, int K, bool AL>
-constexpr int bwd_min_ctas() {
-  return (K <= 5 || (AL && K == 7 && sizeof(T) == 4)) ? 3 : 2;
-}
-
-template <typename T, int K, bool AL>
-__global__ void __launch_bounds__(kThreads, bwd_min_ctas<T, K, AL>())
+__global__ void __launch_bounds__(kThreads, BwdTune<K, T, AL>::MIN_CTAS)
     dw_bwd_kernel(const __grid_constant__ CUtensorMap tmx,
                   const __grid_constant__ CUtensorMap tmdy, const T* __restrict__ x,
                   const T* __restrict__ dy, const float* __restrict__ w, T* __restrict__ dx,
@@ -1097,58 +1117,44 @@ __global__ void __launch_bounds__(kThreads, bwd_min_ctas<T, K, AL>())
   };
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-
-  if (warp < S::NDX) {
-    // ---- input-gradient warps: 16 rows each, in blocks of BR rows
-    for (int t = t_begin; t < t_end; ++t) {
-      const int ty0 = (t / tiles_x) * kBwdTileH, tx0 = (t % tiles_x) * kTileW;
-      if (!stage(ty0, tx0)) break;
-      constexpr int BR = bwd_block_rows<K>();
+  const int g = warp % S::GT, part = warp / S::GT;
+  const int a_lo = group_lo(g, K, S::GT);
+  const int nrows = group_lo(g + 1, K, S::GT) - a_lo;
+  float acc[S::AT][K];
+#pragma unroll
+  for (int s = 0; s < S::AT; ++s)
+#pragma unroll
+    for (int b = 0; b < K; ++b) acc[s][b] = 0.f;
+  for (int t = t_begin; t < t_end; ++t) {
+    const int ty0 = (t / tiles_x) * kBwdTileH, tx0 = (t % tiles_x) * kTileW;
+    if (!stage(ty0, tx0)) break;
+    const int r0 = part * S::DW_ROWS;  // dy rows below the image are zero
+    const int left = S::Tune::SKIP ? H - ty0 : kBwdTileH;
+    const int nb = min(S::DW_ROWS, left - r0 + S::BW - 1) / S::BW;
+    dw_rows<K, S::AT, S::GT, G::SP, S::BW, float, !AL && sizeof(T) == 4>(
+        sm_dy + (r0 + G::R) * G::SP + G::RP + 4 * lane, sm_x + (r0 + a_lo) * G::SP + 4 * lane, nb,
+        nrows, acc);
+    if (!AL && !vec) cta_barrier();  // the x tile becomes the row buffers
 #pragma unroll 1
-      for (int pass = 0; pass < 16 / BR; ++pass) {
-        const int r0 = warp * 16 + pass * BR;
-        float acc[BR][4];
-        fwd_block<K, BR, float, !AL && sizeof(T) == 4>(sm_dy + r0 * G::SP + 4 * lane, sm_w, acc);
-        store_tile<T, BR, AL>(dx + plane_off, H, W, ty0 + r0, tx0, vec != 0,
-                              reinterpret_cast<float*>(sm + 128 + warp * kRowBuf), acc);
-      }
+    for (int x0 = warp * 8; x0 < min(warp * 8 + 8, left); x0 += S::BX) {
+      float o[S::BX][4];
+      fwd_block<K, S::BX, float, !AL && sizeof(T) == 4>(sm_dy + x0 * G::SP + 4 * lane, sm_w, o);
+      store_tile<T, S::BX, AL>(dx + plane_off, H, W, ty0 + x0, tx0, vec != 0,
+                               reinterpret_cast<float*>(sm + S::SM_BUF + warp * kRowBuf), o);
     }
-    cta_barrier();
-    cta_barrier();
-  } else {
-    // ---- filter-gradient warps
-    const int wi = warp - S::NDX;
-    const int g = wi % S::GT;
-    const int part = wi / S::GT;
-    const int a_lo = group_lo(g, K, S::GT);
-    const int nrows = group_lo(g + 1, K, S::GT) - a_lo;
-    float acc[S::AT][K];
-#pragma unroll
-    for (int s = 0; s < S::AT; ++s)
-#pragma unroll
-      for (int b = 0; b < K; ++b) acc[s][b] = 0.f;
-    for (int t = t_begin; t < t_end; ++t) {
-      const int ty0 = (t / tiles_x) * kBwdTileH, tx0 = (t % tiles_x) * kTileW;
-      if (!stage(ty0, tx0)) break;
-      constexpr int BR = bwd_block_rows<K>();
-      const int r0 = part * S::DW_ROWS;
-      dw_rows<K, S::AT, S::GT, G::SP, BR, float, !AL && sizeof(T) == 4>(
-          sm_dy + (r0 + G::R) * G::SP + G::RP + 4 * lane, sm_x + (r0 + a_lo) * G::SP + 4 * lane,
-          S::DW_ROWS / BR, nrows, acc);
-    }
-    // warp reduction (fixed butterfly order), one row of sm_red per warp
-    cta_barrier();
-#pragma unroll
-    for (int s = 0; s < S::AT; ++s)
-#pragma unroll
-      for (int b = 0; b < K; ++b) {
-        float v = acc[s][b];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) sm_red[(wi * S::AT + s) * K + b] = v;
-      }
-    cta_barrier();
   }
+  // warp reduction (fixed butterfly order), one row of sm_red per warp
+  cta_barrier();
+#pragma unroll
+  for (int s = 0; s < S::AT; ++s)
+#pragma unroll
+    for (int b = 0; b < K; ++b) {
+      float v = acc[s][b];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == 0) sm_red[(warp * S::AT + s) * K + b] = v;
+    }
+  cta_barrier();
   // CTA partial for every tap, summed over the warps of its group in a fixed order.
   for (int k = threadIdx.x; k < K * K; k += kThreads) {
     const int a = k / K, b = k - (k / K) * K;
@@ -1166,7 +1172,7 @@ __global__ void __launch_bounds__(kThreads, bwd_min_ctas<T, K, AL>())
 // ------------------------------------------------------- filter gradient
 // The filter gradient alone (Eq. 3's adjoint with respect to the filter):
 // dw[c][a][b] = sum over n, i, j of dy[n][c][i][j] * xs[n][c][i + a - r][j + b - r],
-// xs the border-extended input.  One CTA of 12 or 16 warps per SM, persistent over
+// xs the border-extended input.  One CTA of 8 or 12 warps per SM, persistent over
 // chunks of `tpc` consecutive 64 x 128 tiles of one plane (chunk q runs on
 // CTA q mod gridDim.x).  NS shared-memory stages hold {x tile with halo, dy
 // tile}; the copies of the tile NS - 1 items ahead are in flight while the
@@ -1182,17 +1188,23 @@ __global__ void __launch_bounds__(kThreads, bwd_min_ctas<T, K, AL>())
 constexpr int kFilterTileH = 64;
 static_assert(kFilterTileH == kBwdTileH, "both filter-gradient kernels share the chunk layout");
 
-// Warps and tap-row groups: K = 9 and 15 split into 3 equal groups (12 warps,
-// up to 170 registers for the larger accumulator set: measured faster than 5
-// groups of 3 rows on 20 warps at 96 registers); the rest use 16 warps and
-// dw_groups<K>().
+// Warps, tap-row groups and dy rows per unrolled block.  Up to K = 7 a warp
+// holds every tap (49 accumulators) and 8 warps of 8 tile rows read x rows
+// into 8-row dy blocks: 14 x rows per block instead of the 20 that two 4-row
+// blocks take, and that shared-memory traffic was what 16 warps of 4 rows
+// waited for.  16 x 3 x 2048^2, 16 warps -> 8 warps (us), FP32 / BF16: K = 5
+// 281 -> 253 / 300 -> 233, K = 7 454 -> 398 / 472 -> 404.  From K = 9 on, 12
+// warps in 3 groups (up to 168 registers): K = 9 with 8-row blocks 658 -> 638 /
+// 701 -> 664, K = 11 948 -> 935 / 1013 -> 1009, K = 13 1235 -> 1240 / 1488 ->
+// 1379 against 16 warps; 8-row blocks lose at K >= 11 (K = 11 1077, K = 15
+// 1536 -> 1737).
 template <int K>
 constexpr int filter_warps() {
-  return (K == 9 || K == 15) ? 12 : 16;
+  return K <= 7 ? 8 : 12;
 }
 template <int K>
 constexpr int filter_groups() {
-  return (K == 9 || K == 15) ? 3 : dw_groups<K>();
+  return K <= 7 ? 1 : 3;
 }
 
 template <int K, typename T, bool AL>
@@ -1205,7 +1217,7 @@ struct FilterShape {
   static constexpr int WPG = NW / GT;
   static constexpr int AT = (K + GT - 1) / GT;
   static constexpr int ROWS = kFilterTileH / WPG;  // tile rows per warp
-  static constexpr int DR = 4;                     // dy rows per unrolled block
+  static constexpr int DR = K <= 9 ? 8 : 4;        // dy rows per unrolled block
   static constexpr int X_ROWS = kFilterTileH + 2 * G::R;
   static constexpr int X_BYTES = X_ROWS * G::SP * (int)sizeof(T);
   static constexpr int DY_BYTES = kFilterTileH * DYP * (int)sizeof(T);
@@ -1391,8 +1403,8 @@ __global__ void __launch_bounds__(FilterShape<K, T, AL>::NT, 1)
 
 // ------------------------------------------- backward with a staging ring
 // Both gradients from one staged (x, dy) pair of halo tiles, like
-// dw_bwd_kernel (warps 0-3: the input gradient g, warps 4-7: the filter
-// gradient), but persistent over chunks of `tpc` consecutive tiles (chunk q
+// dw_bwd_kernel (but with warps 0-3 for the input gradient g and warps 4-7 for
+// the filter gradient), persistent over chunks of `tpc` consecutive tiles (chunk q
 // runs on CTA q mod gridDim.x, the layout of dw_filter_kernel, so the same
 // FP64 finalisation applies) with NS shared-memory stages: the copies of the
 // tile NS - 1 items ahead are in flight while the current one is computed,

@@ -26,8 +26,8 @@ def giga():
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("W", [128, 125])
-@pytest.mark.parametrize("K,per_sm", [(1, 4), (3, 2), (3, 4), (7, 16), (9, 2), (9, 16), (11, 2),
-                                      (15, 2)])
+@pytest.mark.parametrize("K,per_sm", [(1, 16), (3, 2), (3, 4), (3, 16), (5, 8), (7, 8), (7, 16),
+                                      (9, 4), (11, 4), (11, 16), (13, 2), (15, 2)])
 def test_both_sides_of_each_threshold(giga, dtype, W, K, per_sm):
     from paper_2504_01266_gb300 import _lib as L
     sms = torch.cuda.get_device_properties(0).multi_processor_count
