@@ -907,6 +907,22 @@ __device__ __forceinline__ void dw_sep_body(
       (ty0 - G::R < 0 || ty0 + S::TH + G::R > H || tx0 - G::RP < 0 || tx0 + kTileW + G::RP > W))
     clamp_fix<float, G::SP, kThreads>(st, H, W, ty0, tx0, G::R, G::RP, S::ROWS);
 
+  // The factors are read once per pass (pinned: re-read per row, the row pass
+  // alone took K broadcast loads per row of a pass that the load/store pipe
+  // bounds: 4 x 3 x 1801 x 2400, K = 15 98.9 -> 92.4 us, K = 5 72.0 -> 68.4; W =
+  // 2399 K = 15 135.5 -> 124.0).
+  float wk[KP];
+  auto load_taps = [&](const float* src) {
+#pragma unroll
+    for (int b = 0; b < KP; b += 4) {
+      const float4 t4 = lds128_pinned(src + b);
+      wk[b] = t4.x;
+      wk[b + 1] = t4.y;
+      wk[b + 2] = t4.z;
+      wk[b + 3] = t4.w;
+    }
+  };
+  load_taps(swr);
   // row pass, in place: row sr of t = columns [0, 128) of staged row sr
   for (int sr = warp; sr < S::ROWS; sr += kWarps) {
     float buf[4 * G::NV];
@@ -914,9 +930,8 @@ __device__ __forceinline__ void dw_sep_body(
     float o[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int b = 0; b < K; ++b) {
-      const float wb = swr[b];
 #pragma unroll
-      for (int px = 0; px < 4; ++px) o[px] = fmaf(wb, buf[G::OFFR + px + b], o[px]);
+      for (int px = 0; px < 4; ++px) o[px] = fmaf(wk[b], buf[G::OFFR + px + b], o[px]);
     }
     __syncwarp();  // every lane has read the row before any lane overwrites it
     *reinterpret_cast<float4*>(st + sr * G::SP + 4 * lane) = make_float4(o[0], o[1], o[2], o[3]);
@@ -924,6 +939,7 @@ __device__ __forceinline__ void dw_sep_body(
   cta_barrier();
 
   // column pass: warp w owns output rows 8w .. 8w + 7
+  load_taps(swc);
   constexpr int PY = 8;
   float acc[PY][4];
 #pragma unroll
@@ -937,11 +953,10 @@ __device__ __forceinline__ void dw_sep_body(
     for (int a = 0; a < K; ++a) {
       const int py = ir - a;
       if (py >= 0 && py < PY) {
-        const float wa = swc[a];
-        acc[py][0] = fmaf(wa, v.x, acc[py][0]);
-        acc[py][1] = fmaf(wa, v.y, acc[py][1]);
-        acc[py][2] = fmaf(wa, v.z, acc[py][2]);
-        acc[py][3] = fmaf(wa, v.w, acc[py][3]);
+        acc[py][0] = fmaf(wk[a], v.x, acc[py][0]);
+        acc[py][1] = fmaf(wk[a], v.y, acc[py][1]);
+        acc[py][2] = fmaf(wk[a], v.z, acc[py][2]);
+        acc[py][3] = fmaf(wk[a], v.w, acc[py][3]);
       }
     }
   }
@@ -960,7 +975,8 @@ __global__ void __launch_bounds__(kThreads) dw_sep_kernel(
 // The same pass compiled for five CTAs per SM (48 registers): used for FP32
 // K = 13 and 15, whose tiles (44 KB) still fit five times in shared memory and
 // whose pass waits on its tile loads (K = 15: 0.701 -> 0.689 ms on
-// 8 x 3 x 4096^2); smaller K run near the HBM rate with the default allocation.
+// 8 x 3 x 4096^2, before the factors were pinned), and for BF16 K <= 3, which
+// would take 50 registers and four CTAs (4 x 3 x 1801 x 2400: 67 -> 61 us).
 template <typename T, int K, bool AL>
 __global__ void __launch_bounds__(kThreads, 5) dw_sep_kernel_hi_occ(
     const __grid_constant__ CUtensorMap tmx, const T* __restrict__ x,

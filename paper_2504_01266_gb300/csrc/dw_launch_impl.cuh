@@ -268,10 +268,11 @@ template <typename T, int K, bool AL>
 static cudaError_t sep_run(const DwArgs& a, const CUtensorMap& tm, const float* wcol,
                            const float* wrow, cudaStream_t st) {
   using S = SepShape<K, T, AL>;
-  // FP32 K = 13, 15: the five-CTA compilation (instantiated for those only)
+  // FP32 K = 13, 15 and BF16 K <= 3: the five-CTA compilation (instantiated for
+  // those only)
   decltype(&dw_sep_kernel<T, K, AL>) kern = dw_sep_kernel<T, K, AL>;
   cudaError_t e;
-  if constexpr (AL && sizeof(T) == 4 && (K == 13 || K == 15)) {
+  if constexpr (AL && (sizeof(T) == 4 ? K == 13 || K == 15 : K <= 3)) {
     kern = dw_sep_kernel_hi_occ<T, K, AL>;
     e = set_smem_once<dw_sep_kernel_hi_occ<T, K, AL>>((size_t)S::SM_BYTES);
   } else {
