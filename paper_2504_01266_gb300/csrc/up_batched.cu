@@ -120,6 +120,7 @@ constexpr int kUp3RagWarps = 8;
 
 template <typename T>
 __global__ void __launch_bounds__(kUp3RagWarps * 32, 2) up3_rag_kernel(UpRagParams p, int n_items) {
+  __shared__ float bufs[kUp3RagWarps * kUp3Buf];
   float wt[36];
   int img_cur = -1;
   uint32_t plane_cur = 0;
@@ -146,7 +147,8 @@ __global__ void __launch_bounds__(kUp3RagWarps * 32, 2) up3_rag_kernel(UpRagPara
     const int sc = (int)im.fs.d;
     up3_item_mode<T>(im.mode, static_cast<const T*>(im.x) + (int64_t)plane * im.H * im.W,
                      static_cast<T*>(im.y) + (int64_t)plane * im.Ho * im.Wo, im.H, im.W, sc,
-                     (int)rg * kUp3Rows, cb, p.clamp, wt);
+                     (int)rg * kUp3Rows, cb, p.clamp, wt,
+                     bufs + (threadIdx.x >> 5) * kUp3Buf);
   }
 }
 

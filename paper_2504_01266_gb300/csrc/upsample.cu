@@ -67,6 +67,8 @@ __global__ void __launch_bounds__(kUp3Warps * 32) up3_poly_kernel(
     const T* __restrict__ x, const float* __restrict__ w, T* __restrict__ y, FastDiv fc, int H,
     int W, int s, FastDiv fcb, FastDiv frb, uint32_t items, int clamp) {
   if (S) s = S;
+  __shared__ float bufs[CE == 0 ? kUp3Warps * kUp3Buf : 1];
+  float* buf = CE == 0 ? bufs + (threadIdx.x >> 5) * kUp3Buf : nullptr;
   float wt[36];
   int c_cur = -1;
   for (uint32_t item = blockIdx.x * kUp3Warps + (threadIdx.x >> 5); item < items;
@@ -82,7 +84,7 @@ __global__ void __launch_bounds__(kUp3Warps * 32) up3_poly_kernel(
     }
     up3_item<T, CE, S, PX>(x + (int64_t)plane * H * W,
                            y + (int64_t)plane * H * s * ((int64_t)W * s), H, W, s, rg * kUp3Rows,
-                           cb, clamp, wt);
+                           cb, clamp, wt, buf);
   }
 }
 
@@ -250,6 +252,7 @@ static cudaError_t up3_launch(const UpArgs& a, cudaStream_t st) {
       return cudaErrorInvalidValue;
     case 7: return up3_launch_ce<T, 4, 0, 1>(a, st);
     case 8: return up3_launch_ce<T, 2, 0, 1>(a, st);
+    case 10: return up3_launch_ce<T, 0, 0, 1>(a, st);
     default: return up3_launch_ce<T, 1, 0, 1>(a, st);
   }
 }

@@ -224,6 +224,7 @@ __device__ __forceinline__ void up_tile(float* __restrict__ sx, int zero_off,
 // by row, with CE-element vector stores (s % CE == 0 and y aligned to CE
 // elements).  S is s when compiled for one scale (2, 4, 8), else 0.
 constexpr int kUp3Rows = 8;
+constexpr int kUp3Buf = 96;  // floats of a warp's row buffer (the buffered form)
 
 // Class R (0: top / left, 1: middle, 2: bottom / right): the taps (bit a:
 // tap a) that land on its input offset slot i, and that offset.
@@ -344,10 +345,21 @@ __device__ __forceinline__ void up3_weights(const float* __restrict__ wc, float 
 // 32 PX cb .. 32 PX cb + 32 PX - 1 (PX consecutive ones per lane) of the
 // plane xp (H x W), output plane yp (H s x W s).  Every lane of the warp calls
 // it.
+//
+// CE = 0 (run-time s, 5 to 8, PX = 1): scales whose s elements a lane could only
+// store 4 or 8 bytes at a time, 4 s bytes from its neighbours', so that every
+// sector was written in pieces.  The three values a lane has for an output row
+// go to `buf` (96 floats of the warp's own) and the warp stores the row's 32 s
+// elements in order, lane after lane; rows of the same class repeat the stores
+// from registers.  3 x 540 x 960 (us), FP32 / BF16: s = 5 54 -> 33 / 67 -> 37, s =
+// 6 71 -> 42 / 50 -> 44, W = 961 s = 7 304 -> 64 / 232 -> 56.  Below 5 the element
+// stores are few and the buffer costs more than it saves (3 x 1080 x 1920 s = 3
+// 67 -> 74 / 86 -> 110).
 template <typename T, int CE, int S, int PX>
 __device__ __forceinline__ void up3_item(const T* __restrict__ xp, T* __restrict__ yp, int H,
                                          int W, int s, int i0, int cb, int clamp,
-                                         const float (&wt)[36]) {
+                                         const float (&wt)[36], float* __restrict__ buf) {
+  static_assert(CE > 0 || (S == 0 && PX == 1), "the buffered form is the run-time one");
   if (S) s = S;
   const int lane = threadIdx.x & 31;
   const int J0 = (cb * 32 + lane) * PX;  // the lane's first input column
@@ -387,6 +399,19 @@ __device__ __forceinline__ void up3_item(const T* __restrict__ xp, T* __restrict
   auto col = [&](int k, int c) { return c == 0 ? cl[k] : (c == PX + 1 ? cr[k] : cm[k][c - 1]); };
   // the output blocks of input pixels (i0, J0 ..), then one block row down per row
   T* o = yp + (int64_t)i0 * s * Wo + (int64_t)J0 * s;
+  // CE = 0: element e = lane + 32 k of the warp's row segment is buf[32 C + src],
+  // src = e / s the lane and C the column class of e % s; one byte each
+  uint32_t at[2] = {0u, 0u};
+  int nv = 0;  // elements of the segment inside the image
+  if constexpr (CE == 0) {
+    nv = min(32, W - 32 * cb) * s;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (k < s) {
+        const int e = lane + 32 * k, src = e / s, v = e - src * s;
+        at[k >> 2] |= (uint32_t)(src + (v == 0 ? 0 : (v == s - 1 ? 64 : 32))) << (8 * (k & 3));
+      }
+  }
 #pragma unroll
   for (int k = 0; k < kUp3Rows; ++k, o += s * Wo) {
     if (i0 + k >= H) break;
@@ -417,7 +442,26 @@ __device__ __forceinline__ void up3_item(const T* __restrict__ xp, T* __restrict
           v[R][C][p] = acc;
         }
     }
-    if (J0 + PX <= W) {
+    if constexpr (CE == 0) {
+      T* seg = o - (int64_t)lane * s + lane;  // element `lane` of the warp's segment
+#pragma unroll
+      for (int R = 0; R < 3; ++R) {
+        __syncwarp();  // the previous class has been read
+#pragma unroll
+        for (int C = 0; C < 3; ++C) buf[32 * C + lane] = v[R][C][0];
+        __syncwarp();
+        float e[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          if (q < s) e[q] = buf[(at[q >> 2] >> (8 * (q & 3))) & 255u];
+        const int u1 = R == 0 ? 1 : (R == 1 ? s - 1 : s);
+        for (int u = R == 0 ? 0 : (R == 1 ? 1 : s - 1); u < u1; ++u) {
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            if (q < s && lane + 32 * q < nv) Elem<T>::store(seg + u * Wo + 32 * q, e[q]);
+        }
+      }
+    } else if (J0 + PX <= W) {
       up3_row<T, CE, S, PX>(o, s, v[0][0], v[0][1], v[0][2]);
 #pragma unroll
       for (int u = 1; u < (S ? S - 1 : s - 1); ++u)
@@ -446,7 +490,8 @@ __device__ __forceinline__ void up3_item(const T* __restrict__ xp, T* __restrict
 // Modes 0, 1: s = 2, 4 with two input pixels per lane (one store of 2 s
 // elements per output row; W even keeps every output row aligned); 2-4:
 // (CE, S) = (2, 2), (4, 4), (8, 8); 5: one 32-byte sector, run-time s; 6: 8
-// elements (BF16 only); 7: 4; 8: 2; 9: 1.
+// elements (BF16 only); 7: 4; 8: 2; 9: 1; 10: the buffered form, where 2 or 1
+// would be the widest and s is 5 to 8.
 inline int up3_mode(int s, const void* y, int elem_bytes, int64_t W) {
   const uintptr_t yp = reinterpret_cast<uintptr_t>(y);
   auto fits = [&](int ce) { return s % ce == 0 && yp % (uintptr_t)(ce * elem_bytes) == 0; };
@@ -459,6 +504,7 @@ inline int up3_mode(int s, const void* y, int elem_bytes, int64_t W) {
   if (fits(32 / elem_bytes)) return 5;
   if (elem_bytes == 2 && fits(8)) return 6;
   if (fits(4)) return 7;
+  if (s >= 5 && s <= 8) return 10;
   if (fits(2)) return 8;
   return 9;
 }
@@ -470,21 +516,22 @@ __host__ __device__ constexpr int up3_cols(int m) { return m <= 1 ? 64 : 32; }
 template <typename T>
 __device__ __forceinline__ void up3_item_mode(int m, const T* __restrict__ xp, T* __restrict__ yp,
                                               int H, int W, int s, int i0, int cb, int clamp,
-                                              const float (&wt)[36]) {
+                                              const float (&wt)[36], float* buf) {
   constexpr int kSector = 32 / (int)sizeof(T);
   switch (m) {
-    case 0: up3_item<T, 4, 2, 2>(xp, yp, H, W, s, i0, cb, clamp, wt); break;
-    case 1: up3_item<T, 8, 4, 2>(xp, yp, H, W, s, i0, cb, clamp, wt); break;
-    case 2: up3_item<T, 2, 2, 1>(xp, yp, H, W, s, i0, cb, clamp, wt); break;
-    case 3: up3_item<T, 4, 4, 1>(xp, yp, H, W, s, i0, cb, clamp, wt); break;
-    case 4: up3_item<T, 8, 8, 1>(xp, yp, H, W, s, i0, cb, clamp, wt); break;
-    case 5: up3_item<T, kSector, 0, 1>(xp, yp, H, W, s, i0, cb, clamp, wt); break;
+    case 0: up3_item<T, 4, 2, 2>(xp, yp, H, W, s, i0, cb, clamp, wt, buf); break;
+    case 1: up3_item<T, 8, 4, 2>(xp, yp, H, W, s, i0, cb, clamp, wt, buf); break;
+    case 2: up3_item<T, 2, 2, 1>(xp, yp, H, W, s, i0, cb, clamp, wt, buf); break;
+    case 3: up3_item<T, 4, 4, 1>(xp, yp, H, W, s, i0, cb, clamp, wt, buf); break;
+    case 4: up3_item<T, 8, 8, 1>(xp, yp, H, W, s, i0, cb, clamp, wt, buf); break;
+    case 5: up3_item<T, kSector, 0, 1>(xp, yp, H, W, s, i0, cb, clamp, wt, buf); break;
     case 6:
-      if constexpr (sizeof(T) == 2) up3_item<T, 8, 0, 1>(xp, yp, H, W, s, i0, cb, clamp, wt);
+      if constexpr (sizeof(T) == 2) up3_item<T, 8, 0, 1>(xp, yp, H, W, s, i0, cb, clamp, wt, buf);
       break;
-    case 7: up3_item<T, 4, 0, 1>(xp, yp, H, W, s, i0, cb, clamp, wt); break;
-    case 8: up3_item<T, 2, 0, 1>(xp, yp, H, W, s, i0, cb, clamp, wt); break;
-    default: up3_item<T, 1, 0, 1>(xp, yp, H, W, s, i0, cb, clamp, wt); break;
+    case 7: up3_item<T, 4, 0, 1>(xp, yp, H, W, s, i0, cb, clamp, wt, buf); break;
+    case 8: up3_item<T, 2, 0, 1>(xp, yp, H, W, s, i0, cb, clamp, wt, buf); break;
+    case 10: up3_item<T, 0, 0, 1>(xp, yp, H, W, s, i0, cb, clamp, wt, buf); break;
+    default: up3_item<T, 1, 0, 1>(xp, yp, H, W, s, i0, cb, clamp, wt, buf); break;
   }
 }
 
