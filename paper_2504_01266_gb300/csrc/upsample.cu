@@ -171,8 +171,18 @@ __device__ __forceinline__ void up_fwd_body(const T* __restrict__ x, const float
   }
 }
 
+// CTAs per SM that the kernel is compiled for (0: left to the compiler).  The
+// FMA-bound FP32 filters gain by the fourth CTA, which their 64 registers hold
+// without a spill (left alone they take 70 to 80): 3 x 1080 x 1920 s = 2, K = 9
+// 90.6 -> 88.5 us, K = 11 121.2 -> 117.3, K = 13 155.7 -> 152.9, K = 15 193.9 ->
+// 191.3.  BF16 spills at that bound and loses 1 to 3 %, K <= 7 has room anyway.
 template <typename T, int K>
-__global__ void __launch_bounds__(kThreads) up_fwd_kernel(const T* __restrict__ x,
+constexpr int up_min_ctas() {
+  return K >= 9 && sizeof(T) == 4 ? 4 : 0;
+}
+
+template <typename T, int K>
+__global__ void __launch_bounds__(kThreads, up_min_ctas<T, K>()) up_fwd_kernel(const T* __restrict__ x,
                                                           const float* __restrict__ w,
                                                           T* __restrict__ y, FastDiv fc, int H,
                                                           int W, int Ho, int Wo, FastDiv fs,
