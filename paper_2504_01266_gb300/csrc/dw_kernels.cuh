@@ -644,7 +644,7 @@ __device__ __forceinline__ void dw_rows(const TS* __restrict__ dyb, const TS* __
   }
 }
 
-// Rows per unrolled block in the backward roles: the input-gradient and the
+// Rows per unrolled block in the ring kernel's roles: the input-gradient and the
 // filter-gradient warps run different unrolled bodies on the same SM, so for
 // K >= 7 both use 4-row blocks to keep the two bodies within the
 // instruction cache together.
@@ -1422,7 +1422,7 @@ __global__ void __launch_bounds__(FilterShape<K, T, AL>::NT, 1)
 // dw_bwd_kernel (but with warps 0-3 for the input gradient g and warps 4-7 for
 // the filter gradient), persistent over chunks of `tpc` consecutive tiles (chunk q
 // runs on CTA q mod gridDim.x, the layout of dw_filter_kernel, so the same
-// FP64 finalisation applies) with NS shared-memory stages: the copies of the
+// finalisation applies) with NS shared-memory stages: the copies of the
 // tile NS - 1 items ahead are in flight while the current one is computed,
 // across chunk boundaries too.  One CTA per SM.  It suits the HBM-bound small
 // filters, whose single-stage fused kernel leaves its tile loads exposed; a

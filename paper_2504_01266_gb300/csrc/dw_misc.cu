@@ -1,6 +1,7 @@
 // dw_misc.cu -- what follows the tile kernels of the depthwise backward pass:
 //  * the clamp-border edge fold of the input gradient, and
-//  * the FP64 fixed-order reduction of the per-CTA filter-gradient partials,
+//  * the fixed-order reduction of the per-CTA filter-gradient partials (in two
+//    floats, closed in FP64),
 // in one launch (dw_finish_kernel).
 #include <algorithm>
 #include <cstring>
@@ -95,7 +96,7 @@ __global__ void dw_fixup_kernel(const T* __restrict__ dy, const float* __restric
 
 // ------------------------------------------------- fold and reduction
 // One launch with three kinds of 512-thread blocks (what a call does not need
-// has none): the filter gradient's FP64 sums, the fold of 256 pixels of the
+// has none): the filter gradient's sums, the fold of 256 pixels of the
 // first and last row or column of a plane, and the fold of a plane's corner
 // pixels, which both folds touch.  All are short and bound by latency, so they
 // run beside each other instead of one after the other.  4 x 3 x 1801 x 2399,

@@ -20,8 +20,9 @@
 //  * each chunk writes one K*K vector of FP32 filter-gradient partials; the
 //    CTA that completes the last chunk of an (image, channel) -- detected with
 //    a per-(image, channel) atomic counter after a memory fence -- sums that
-//    image-channel's partials in FP64 in chunk order (deterministic) and, for
-//    the clamp border, folds the edges of dx.  No CTA ever waits for another.
+//    image-channel's partials in a fixed order (two-float sums closed in FP64;
+//    deterministic) and, for the clamp border, folds the edges of dx.  No CTA
+//    ever waits for another.
 #pragma once
 
 #include "dw_fold.cuh"
