@@ -132,8 +132,14 @@ DwConfig tune_config(int op, int id, const DwArgs& a) {
 //    (16 x 3 x 2048^2: 380 -> 368, 573 -> 554) and BF16 K <= 3 (197 -> 179);
 //    FP32 K = 3 loses by it (230 -> 253), the others are equal.
 //  * both gradients, fused kernel -> the choice:
-//    K <= 3, aligned planes: the tile ring from T = 16 S (FP32; 16 x 3 x 2048^2
-//    422 -> 376, at T = 10 S 38.8 -> 40.7) or 4 S (BF16; 378 -> 261, at 5 S 25.7
+//    FP32 K <= 3, very many tiles: the fused kernel with two tiles per CTA, whose
+//    three CTAs per SM keep HBM busier than the ring's one, and whose CTAs work
+//    on nearer tiles than with the usual 8 or 16 each: K = 3 from T = 100 S (ring ->
+//    pairs: 8 x 3 x 2048^2, 81 S, 189 -> 201; 12 x 3 x 2048^2 307 -> 290; 8 x 3 x
+//    4096^2 793 -> 738; unaligned 16 x 3 x 2048 x 2047 598 -> 556), K = 1 from 80 S
+//    (208 -> 181).
+//    K <= 3, aligned planes: the tile ring from T = 16 S (FP32; 8 x 3 x 2048^2
+//    218 -> 189, at T = 10 S 38.8 -> 40.7) or 4 S (BF16; 378 -> 261, at 5 S 25.7
 //    -> 21.2); its one CTA per SM stages unaligned planes with the warps that
 //    compute (160 -> 207).
 //    Two passes: K >= 13 from T = 2 S (3 x 1080 x 1920 K = 13: 117 -> 106, 4 x 3
@@ -157,7 +163,8 @@ DwConfig default_config(int op, const DwArgs& a) {
         c.prefetch = aligned && (f32 ? a.K == 7 || a.K == 9 : a.K <= 3);
       break;
     case TUNE_BWD_FUSED: {
-      const bool ring = a.K <= 3 && aligned && T >= (f32 ? 16 : 4) * S;
+      const bool pairs = f32 && a.K <= 3 && T >= (a.K == 1 ? 80 : 100) * S;
+      const bool ring = !pairs && a.K <= 3 && aligned && T >= (f32 ? 16 : 4) * S;
       int64_t from = -1;  // two passes from this many tiles per SM on
       if (a.K >= 13)
         from = 2;
@@ -170,7 +177,7 @@ DwConfig default_config(int op, const DwArgs& a) {
       else if (a.K == 5 && !f32 && aligned)
         from = 8;
       const bool split = from >= 0 && T >= from * S;
-      if (ring || split) c = tune_config(op, split ? 5 : 6, a);
+      if (ring || split || pairs) c = tune_config(op, split ? 5 : (ring ? 6 : 1), a);
       break;
     }
     default:
