@@ -277,6 +277,17 @@ __device__ __forceinline__ void stage_any(T* __restrict__ sm, const T* plane, in
   }
 }
 
+// Word k of a BF16 row of `words` words, one element to the left.  The last
+// word of a row has no successor in the row (K = 15 and 31, whose halo fills
+// the pitch): the next row's first word is another warp's to write, and the
+// half it would give is past the columns in use.
+__host__ __device__ inline uint32_t shifted_word(const uint32_t* row, int k, int words) {
+  return (row[k] >> 16) | (k + 1 < words ? row[k + 1] << 16 : 0u);
+}
+
+// 4-byte words that hold the staged columns in use.
+__host__ __device__ constexpr int shift_words(int R, int RP) { return (kTileW + RP + R + 1) / 2; }
+
 // BF16 rows that stage_any left one element to the right (row addresses that
 // are not multiples of 4: every second row when W is odd) move into place.
 // Every thread calls it once its own copies have landed; it begins with a CTA
@@ -286,20 +297,20 @@ __device__ __forceinline__ void shift_odd_rows(T* __restrict__ sm, const T* plan
                                                int ty0, int rows, int R, int RP, int pitch) {
   if constexpr (sizeof(T) == 2) {
     const int lane = threadIdx.x & 31;
-    const int words = (kTileW + RP + R + 1) / 2;  // at most 80
+    const int words = shift_words(R, RP);  // at most 80
     cta_barrier();
     for (int sr = threadIdx.x >> 5; sr < rows; sr += NT / 32) {
       const int gi = ty0 - R + sr;
       if (gi < 0 || gi >= H || !row_is_odd(plane + (int64_t)gi * W)) continue;
-      uint32_t* d = reinterpret_cast<uint32_t*>(sm + sr * pitch) + lane;
+      uint32_t* d = reinterpret_cast<uint32_t*>(sm + sr * pitch);
       uint32_t v[3];
 #pragma unroll
       for (int q = 0; q < 3; ++q)
-        if (lane + 32 * q < words) v[q] = __funnelshift_r(d[32 * q], d[32 * q + 1], 16);
+        if (lane + 32 * q < words) v[q] = shifted_word(d, lane + 32 * q, pitch / 2);
       __syncwarp();
 #pragma unroll
       for (int q = 0; q < 3; ++q)
-        if (lane + 32 * q < words) d[32 * q] = v[q];
+        if (lane + 32 * q < words) d[lane + 32 * q] = v[q];
     }
   }
 }
