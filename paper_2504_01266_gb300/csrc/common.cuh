@@ -70,10 +70,13 @@ struct DwConfig {
   int ring;             // fused backward: 1 = persistent kernel with a two-stage tile ring
 };
 
-// Element access for the two storage types; arithmetic is always FP32.
+// Element access for the two storage types; arithmetic is always FP32.  load
+// takes the read-only path, which is defined only for data that the kernel does
+// not write: a pointer to non-const data does not compile.
 template <typename T> struct Elem;
 template <> struct Elem<float> {
   static __device__ __forceinline__ float load(const float* p) { return __ldg(p); }
+  static __device__ float load(float*) = delete;
   static __device__ __forceinline__ void store(float* p, float v) { *p = v; }
   static __device__ __forceinline__ void store4(float* p, float4 v) {
     *reinterpret_cast<float4*>(p) = v;
@@ -83,6 +86,7 @@ template <> struct Elem<__nv_bfloat16> {
   static __device__ __forceinline__ float load(const __nv_bfloat16* p) {
     return __bfloat162float(__ldg(p));
   }
+  static __device__ float load(__nv_bfloat16*) = delete;
   static __device__ __forceinline__ void store(__nv_bfloat16* p, float v) {
     *p = __float2bfloat16_rn(v);
   }

@@ -226,7 +226,8 @@ __device__ __forceinline__ void finish_edges(const FinishArgs& p, int64_t plane,
   T* d = static_cast<T*>(p.dx) + plane * (int64_t)H * W +
          (rows ? (int64_t)in * W + q : (int64_t)q * W + in);
   float s = 0.f, old = 0.f;
-  if (sizeof(T) == 4 && mine) old = Elem<T>::load(d);  // on its way while the strip arrives
+  if constexpr (sizeof(T) == 4)
+    if (mine) old = *d;  // on its way while the strip arrives
   for (int k = threadIdx.x; k < K * K; k += kFinishThreads) sf[k] = __ldg(f + k);
   // strip[e][i][c]: i rows (columns) in from edge e, at position q0 - r + c
   for (int k = threadIdx.x; k < 2 * D * SW; k += kFinishThreads) {
