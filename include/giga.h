@@ -18,9 +18,8 @@
  * contributions that were read from clamped positions return to the edge pixel
  * they were read from) and dw[c][a][b] = sum_{n,i,j} dy[n][c][i][j] *
  * x[n][c][i + a - r][j + b - r] (the filter is shared by the batch, so the sum
- * runs over n).  The filter gradient's partial sums are added in a fixed order, in
- * pairs of floats (about 48 bits) closed in FP64, so repeated calls on the same
- * device give bit-identical results.
+ * runs over n).  The filter gradient is reduced in FP64 in a fixed order, so
+ * repeated calls on the same device give bit-identical results.
  *
  * Conventions for every entry point:
  *   - Every pointer argument named x, y, dx, dy, w, dw, ws is a DEVICE pointer
@@ -109,7 +108,7 @@ giga_status_t giga_conv2d_bwd_input(const giga_conv2d_desc_t* desc, const void* 
  * derivative of Section 4.2.4's neighbourhood sum with respect to each filter
  * entry, dw[c][a][b] = sum over n, i, j of dy[n][c][i][j] times the pixel tap
  * (a, b) reads for output (i, j).  Per-CTA FP32 partial sums go to the
- * workspace and are added in a fixed order, in pairs of floats closed in FP64. */
+ * workspace and are summed in FP64 in a fixed order. */
 giga_status_t giga_conv2d_bwd_filter(const giga_conv2d_desc_t* desc, const void* x,
                                      const void* dy, float* dw, void* ws, size_t ws_bytes,
                                      void* stream);

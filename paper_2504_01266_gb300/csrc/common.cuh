@@ -100,23 +100,6 @@ template <> struct Elem<__nv_bfloat16> {
   }
 };
 
-// A running sum in two floats: s the rounded sum, e what rounding left out
-// (Knuth's TwoSum gives it exactly; only adding the e's rounds, 2^-24 of them,
-// so the sum is good to about 2^-48 of its largest term -- the FP64 sums of
-// FP32 partials it feeds round to the same FP32 result).  Seven FP32
-// instructions where FP64 takes a conversion and an add on a unit with 1/64 of
-// the rate.  Not for non-finite results: callers check and redo those in FP64.
-struct TwoFloatSum {
-  float s = 0.f, e = 0.f;
-  __device__ __forceinline__ void add(float x) {
-    const float t = __fadd_rn(s, x);
-    const float z = __fadd_rn(t, -s);
-    e = __fadd_rn(e, __fadd_rn(__fadd_rn(s, -__fadd_rn(t, -z)), __fadd_rn(x, -z)));
-    s = t;
-  }
-  __device__ __forceinline__ double value() const { return (double)s + (double)e; }
-};
-
 // Host-side launch accounting (giga_launch_count).
 void note_launch(int n = 1);
 

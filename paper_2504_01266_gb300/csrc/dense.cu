@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1)
 // the last one, so the pair (last slot, slot 0) is adjacent too.  D
 // accumulates in TMEM over all chunks of the CTA (2 x 192 columns); each CTA
 // then writes its FP32 partial sums [tap][c][o] and a second kernel adds the
-// CTAs' partials in a fixed order (two-float and FP64 sums).
+// CTAs' partials in FP64 in a fixed order.
 constexpr int kWgTileP = 64;                           // pixel positions per chunk (MMA K: 4 x 16)
 constexpr int kWgXPx = kWgTileP + 1;                   // x band: 65 pixels
 constexpr int kWgDyPx = kWgTileP + 2;                  // dy band: 66 pixels
@@ -687,12 +687,10 @@ __global__ void __launch_bounds__(kDenseThreads, 1)
   }
 }
 
-// dw[o][a][b][c] = sum over CTAs, in a fixed order, of partial[cta][3a + b][c][o].
-// A block takes one (tap, c): 64 lanes across o read whole lines of a partial,
-// four groups of them take every fourth CTA in two-float sums, and the groups
-// add in FP64.  22 MB of partials come from L2 whatever the image size.  One
-// thread per output in dw's order read a 32-byte sector per value and added
-// 152 FP64 values in sequence: 26 us.
+// dw[o][a][b][c] = sum over CTAs (FP64, in a fixed order) of
+// partial[cta][3a + b][c][o].  A block takes one (tap, c): 64 lanes across o read
+// whole lines of a partial, four groups of them take every fourth CTA, and the
+// groups add up.  22 MB of partials come from L2 whatever the image size.
 constexpr int kWgFinGroups = 4;
 __global__ void __launch_bounds__(kDenseC * kWgFinGroups)
     dense_wgrad_finalize_kernel(const float* __restrict__ partials, int ctas,
@@ -701,14 +699,9 @@ __global__ void __launch_bounds__(kDenseC * kWgFinGroups)
   const int o = threadIdx.x % kDenseC, g = threadIdx.x / kDenseC;
   const int tap = blockIdx.x / kDenseC, c = blockIdx.x % kDenseC;
   const float* src = partials + ((int64_t)tap * kDenseC + c) * kDenseC + o;
-  TwoFloatSum sum;
+  double s = 0.0;
 #pragma unroll 8
-  for (int b = g; b < ctas; b += kWgFinGroups) sum.add(__ldg(src + (int64_t)b * kWgPartialFloats));
-  double s = sum.value();
-  if (!isfinite(s)) {  // infinities, NaN or an overflow on the way
-    s = 0.0;
-    for (int b = g; b < ctas; b += kWgFinGroups) s += (double)__ldg(src + (int64_t)b * kWgPartialFloats);
-  }
+  for (int b = g; b < ctas; b += kWgFinGroups) s += (double)__ldg(src + (int64_t)b * kWgPartialFloats);
   part[g][o] = s;
   __syncthreads();
   if (g == 0) {

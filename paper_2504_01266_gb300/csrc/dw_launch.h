@@ -77,8 +77,8 @@ int64_t dw_bwd_chunks_per_plane(int64_t H, int64_t W, int tiles_per_cta);
 
 // What follows the tile passes of a backward call: with `fold` (and the clamp
 // border) the edge fold that turns g into dx; with chunks_per_plane > 0 the
-// filter gradient dw[c][k] = the sum over (n, chunk) of the partials, in two
-// floats closed in FP64 and a fixed order.  One launch.
+// filter gradient dw[c][k] = the sum over (n, chunk) of the partials, in FP64
+// and a fixed order.  One launch.
 cudaError_t dw_finish_launch(const DwArgs& a, bool fold, int64_t chunks_per_plane,
                              cudaStream_t st);
 

@@ -1,7 +1,6 @@
 // dw_misc.cu -- what follows the tile kernels of the depthwise backward pass:
 //  * the clamp-border edge fold of the input gradient, and
-//  * the fixed-order reduction of the per-CTA filter-gradient partials (in two
-//    floats, closed in FP64),
+//  * the fixed-order FP64 reduction of the per-CTA filter-gradient partials,
 // in one launch (dw_finish_kernel).
 #include <algorithm>
 #include <cstring>
@@ -123,13 +122,12 @@ struct FinishArgs {
 };
 
 // dw[c][k] = sum over the partial rows (image n, chunk ch) of channel c in a
-// fixed order: a block takes p.taps taps of one channel, a thread every
-// (512 / p.taps)-th row of one tap, eight loads in flight, in a two-float sum;
-// then FP64, a butterfly within the warp and the warps in order.  FP64 adds
-// and conversions run at about two a clock on an SM, so there are few of them
-// and the taps are spread over as many blocks as fill the GPU (finish_taps)
-// rather than read by few in whole sectors (4 x 3 x 1801 x 2399, K = 3, with
-// the fold: 22 us with 32 taps per block, 6 us with one, both all FP64).
+// fixed order, all in FP64: a block takes p.taps taps of one channel, a thread
+// every (512 / p.taps)-th row of one tap, eight loads in flight; then a butterfly
+// within the warp and the warps in order.  FP64 adds and conversions run at
+// about two a clock on an SM, so the taps are spread over as many blocks as fill
+// the GPU (finish_taps) rather than read by few in whole sectors (4 x 3 x 1801 x
+// 2399, K = 3, with the fold: 22 us with 32 taps per block, 6 us with one).
 __device__ __forceinline__ void finish_sums(const FinishArgs& p, double* red) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int c = (int)blockIdx.x / p.groups, g = (int)blockIdx.x - c * p.groups;
@@ -140,7 +138,6 @@ __device__ __forceinline__ void finish_sums(const FinishArgs& p, double* red) {
   const uint32_t count = (uint32_t)p.N * chunks;
   double s = 0.0;
   if (tap < p.KK) {
-    TwoFloatSum sum;
     constexpr int U = 8;
     for (uint32_t i0 = threadIdx.x / TB; i0 < count; i0 += U * slots) {
       float v[U];
@@ -155,15 +152,7 @@ __device__ __forceinline__ void finish_sums(const FinishArgs& p, double* red) {
       }
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        if (i0 + u * slots < count) sum.add(v[u]);
-    }
-    s = sum.value();
-    if (!isfinite(s)) {  // infinities, NaN or an overflow on the way
-      s = 0.0;
-      for (uint32_t i = threadIdx.x / TB; i < count; i += slots) {
-        const uint32_t n = fdiv(i, p.chunks), ch = i - n * chunks;
-        s += (double)__ldg(p.partials + (((int64_t)n * p.C + c) * chunks + ch) * p.KK + tap);
-      }
+        if (i0 + u * slots < count) s += (double)v[u];
     }
   }
   for (int o = 16; o >= TB; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);

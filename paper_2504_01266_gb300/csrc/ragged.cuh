@@ -20,9 +20,8 @@
 //  * each chunk writes one K*K vector of FP32 filter-gradient partials; the
 //    CTA that completes the last chunk of an (image, channel) -- detected with
 //    a per-(image, channel) atomic counter after a memory fence -- sums that
-//    image-channel's partials in a fixed order (two-float sums closed in FP64;
-//    deterministic) and, for the clamp border, folds the edges of dx.  No CTA
-//    ever waits for another.
+//    image-channel's partials in FP64 in a fixed order (deterministic) and, for
+//    the clamp border, folds the edges of dx.  No CTA ever waits for another.
 #pragma once
 
 #include "dw_fold.cuh"
@@ -167,22 +166,15 @@ __device__ __forceinline__ void rag_complete(const RagParams& p, int c, double* 
       __threadfence();
       const int K = im.K, KK = K * K;
       if (do_dw) {
-        // every tap's partials by GR threads, each every GR-th chunk, in
-        // two-float sums; then their FP64 values in order (one thread per tap
-        // adding FP64 took about 20 us of a CTA's time: 3 x 2001 x 3000 K = 3
-        // 124 -> 99 us)
+        // every tap's partials in FP64 by GR threads, each every GR-th chunk,
+        // then their sums in order
         const float* part = p.partials + im.partial_base + (int64_t)ch.channel * im.nch * KK;
         const int GR = min(kRagThreads / KK, 16);
         const int k = threadIdx.x % KK, q = threadIdx.x / KK;
         if (q < GR) {
-          TwoFloatSum sum;
+          double s = 0.0;
 #pragma unroll 8
-          for (int j = q; j < im.nch; j += GR) sum.add(__ldcg(part + (int64_t)j * KK + k));
-          double s = sum.value();
-          if (!isfinite(s)) {  // infinities, NaN or an overflow on the way
-            s = 0.0;
-            for (int j = q; j < im.nch; j += GR) s += (double)__ldcg(part + (int64_t)j * KK + k);
-          }
+          for (int j = q; j < im.nch; j += GR) s += (double)__ldcg(part + (int64_t)j * KK + k);
           ps[q * KK + k] = s;
         }
         cta_barrier();
