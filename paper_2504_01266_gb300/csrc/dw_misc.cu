@@ -64,8 +64,8 @@ int64_t dw_bwd_chunks_per_plane(int64_t H, int64_t W, int tiles_per_cta) {
 }
 
 // ------------------------------------------------------------- edge fold
-// BF16 planes one pixel high or wide: every pixel recomputed from the
-// definition.
+// BF16 planes one pixel high or wide, and very many very small ones
+// (fold_by_pixel): every edge pixel recomputed from the definition.
 template <typename T>
 __global__ void dw_fixup_kernel(const T* __restrict__ dy, const float* __restrict__ w,
                                 T* __restrict__ dx, int C, int H, int W, int K,
@@ -94,8 +94,8 @@ __global__ void dw_fixup_kernel(const T* __restrict__ dy, const float* __restric
 // the same sums with the taps that read the edge itself included.
 
 // ------------------------------------------------- fold and reduction
-// One launch with three kinds of 512-thread blocks (what a call does not need
-// has none): the filter gradient's sums, the fold of 256 pixels of the
+// One launch with three kinds of blocks of NT threads (what a call does not need
+// has none): the filter gradient's sums, the fold of NT / 2 pixels of the
 // first and last row or column of a plane, and the fold of a plane's corner
 // pixels, which both folds touch.  All are short and bound by latency, so they
 // run beside each other instead of one after the other.  4 x 3 x 1801 x 2399,
@@ -103,8 +103,10 @@ __global__ void dw_fixup_kernel(const T* __restrict__ dy, const float* __restric
 // over the partials, uncoalesced) as three launches, 6.1 us as one; K = 15,
 // 8 x 3 x 1024^2: 52 -> 12.9 us; BF16 K = 9, 4 x 3 x 1800 x 2400: 60 (the
 // pixel-by-pixel fold 45 of it) -> 10.7 us; 4 x 3 x 257 x 251: 10.5 -> 4.3 us.
-constexpr int kFinishThreads = 512;
-constexpr int kFoldPixels = 256;  // per fold block: one thread for each of its two edges
+//
+// NT is 512, or 128 (finish_small) where the planes' edges or the partial sums
+// are so few that most of 512 threads would idle.
+constexpr int kFinishThreads = 512, kFinishThreadsSmall = 128;
 
 struct FinishArgs {
   const float* partials;  // filter gradient: [N * C * chunks][KK]
@@ -123,17 +125,18 @@ struct FinishArgs {
 
 // dw[c][k] = sum over the partial rows (image n, chunk ch) of channel c in a
 // fixed order, all in FP64: a block takes p.taps taps of one channel, a thread
-// every (512 / p.taps)-th row of one tap, eight loads in flight; then a butterfly
+// every (NT / p.taps)-th row of one tap, eight loads in flight; then a butterfly
 // within the warp and the warps in order.  FP64 adds and conversions run at
 // about two a clock on an SM, so the taps are spread over as many blocks as fill
 // the GPU (finish_taps) rather than read by few in whole sectors (4 x 3 x 1801 x
 // 2399, K = 3, with the fold: 22 us with 32 taps per block, 6 us with one).
+template <int NT>
 __device__ __forceinline__ void finish_sums(const FinishArgs& p, double* red) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int c = (int)blockIdx.x / p.groups, g = (int)blockIdx.x - c * p.groups;
   const int TB = p.taps;  // a power of two, at most 32
   const int tap = TB * g + (threadIdx.x & (TB - 1));
-  const int slots = kFinishThreads / TB;
+  const int slots = NT / TB;
   const uint32_t chunks = p.chunks.d;
   const uint32_t count = (uint32_t)p.N * chunks;
   double s = 0.0;
@@ -160,7 +163,7 @@ __device__ __forceinline__ void finish_sums(const FinishArgs& p, double* red) {
   __syncthreads();
   if ((int)threadIdx.x < TB && tap < p.KK) {
     double sum = 0.0;
-    for (int w = 0; w < kFinishThreads / 32; ++w) sum += red[w * TB + threadIdx.x];
+    for (int w = 0; w < NT / 32; ++w) sum += red[w * TB + threadIdx.x];
     p.dw[(int64_t)c * p.KK + tap] = (float)sum;
   }
 }
@@ -193,23 +196,24 @@ __device__ __forceinline__ float fold_weight(const float* f, int step, int K, in
   return t;
 }
 
-// Pixels 256 * blk .. of the first and last row (rows = true: sums T and B
+// Pixels NT / 2 * blk .. of the first and last row (rows = true: sums T and B
 // above, one half of the block each) or column (L and R) of a plane; its
 // corner pixels are left to finish_corners.
-template <typename T>
+template <typename T, int NT>
 __device__ __forceinline__ void finish_edges(const FinishArgs& p, int64_t plane, int blk, bool rows,
                                              float* tab) {
   const int K = p.K, r = (K - 1) / 2, H = p.H, W = p.W, D = fold_depth<T>(r);
+  constexpr int P = NT / 2;
   const int lim = rows ? W : H;    // length of the edge
   const int other = rows ? H : W;  // rows (columns) across it
   const float* f = p.w + (plane % p.C) * (int64_t)K * K;
   float* sf = tab;                // the filter
   float* wt = sf + K * K;         // [2][D][K] summed weights: first edge, last edge
-  float* strip = wt + 2 * D * K;  // [2][D][kFoldPixels + 2 r] of dy
-  const int SW = kFoldPixels + 2 * r;
+  float* strip = wt + 2 * D * K;  // [2][D][SW] of dy
   const T* g = static_cast<const T*>(p.dy) + plane * (int64_t)H * W;
-  const int q0 = blk * kFoldPixels, n = min(D, other);
-  const int e = threadIdx.x / kFoldPixels, t = threadIdx.x - e * kFoldPixels;
+  const int q0 = blk * P, n = min(D, other);
+  const int SW = min(P, lim - q0) + 2 * r;  // the pixels of this block and their margins
+  const int e = threadIdx.x / P, t = threadIdx.x - e * P;
   const int q = q0 + t, in = e ? other - 1 : 0;
   const bool mine = q > 0 && q < lim - 1 && !(e == 1 && other == 1);
   T* d = static_cast<T*>(p.dx) + plane * (int64_t)H * W +
@@ -217,35 +221,38 @@ __device__ __forceinline__ void finish_edges(const FinishArgs& p, int64_t plane,
   float s = 0.f, old = 0.f;
   if constexpr (sizeof(T) == 4)
     if (mine) old = *d;  // on its way while the strip arrives
-  for (int k = threadIdx.x; k < K * K; k += kFinishThreads) sf[k] = __ldg(f + k);
-  // strip[e][i][c]: i rows (columns) in from edge e, at position q0 - r + c
-  for (int k = threadIdx.x; k < 2 * D * SW; k += kFinishThreads) {
-    int es, i, c;
-    if (rows) {  // consecutive threads along the row
-      es = k / (D * SW), i = k / SW - es * D, c = k - (k / SW) * SW;
-    } else {     // along the first / last columns of a row
-      c = k / (2 * D), es = (k - c * 2 * D) / D, i = k - c * 2 * D - es * D;
+  for (int k = threadIdx.x; k < K * K; k += NT) sf[k] = __ldg(f + k);
+  // strip[k = e D + i][c]: i rows (columns) in from edge e, at position q0 - r + c.
+  // Consecutive lanes run along the row (rows), or over the 2 D columns of one
+  // position, a power of two of lanes for them: no index is divided.
+  const int cl = rows ? 0 : 32 - __clz(2 * D - 1);  // log2 of the lanes per position
+  const int c0 = rows ? threadIdx.x & 31 : threadIdx.x >> cl, cs = rows ? 32 : NT >> cl;
+  const int k0 = rows ? threadIdx.x >> 5 : threadIdx.x & ((1 << cl) - 1);
+  for (int k = k0; k < 2 * D; k += rows ? NT / 32 : 32) {
+    const int es = k >= D, i = k - es * D, from = es ? other - 1 - i : i;
+    for (int c = c0; c < SW; c += cs) {
+      const int at = q0 - r + c;
+      float v = 0.f;
+      if (i < n && at >= 0 && at < lim)
+        v = Elem<T>::load(g + (rows ? (int64_t)from * W + at : (int64_t)at * W + from));
+      strip[k * SW + c] = v;
     }
-    const int at = q0 - r + c, from = es ? other - 1 - i : i;
-    float v = 0.f;
-    if (i < n && at >= 0 && at < lim)
-      v = Elem<T>::load(g + (rows ? (int64_t)from * W + at : (int64_t)at * W + from));
-    strip[(es * D + i) * SW + c] = v;
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < 2 * D * K; k += kFinishThreads) {
+  for (int k = threadIdx.x; k < 2 * D * K; k += NT) {
     const int ew = k / (D * K), i = k / K - ew * D, b = k - (k / K) * K;
     wt[k] = rows ? fold_weight<T>(sf + b, K, K, ew, i) : fold_weight<T>(sf + b * K, 1, K, ew, i);
   }
   __syncthreads();
-  for (int i = 0; i < n; ++i)
-    for (int b = 0; b < K; ++b)
-      s = fmaf(wt[(e * D + i) * K + b], strip[(e * D + i) * SW + t + 2 * r - b], s);
+  if (q < lim)
+    for (int i = 0; i < n; ++i)
+      for (int b = 0; b < K; ++b)
+        s = fmaf(wt[(e * D + i) * K + b], strip[(e * D + i) * SW + t + 2 * r - b], s);
   if (other == 1) {  // a single row (column) is both edges: the first half adds both sums
     __syncthreads();
-    if (e == 1) strip[t] = s;
+    if (e == 1 && q < lim) strip[t] = s;
     __syncthreads();
-    s += strip[t];
+    if (q < lim) s += strip[t];
   }
   if (mine) Elem<T>::store(d, old + s);
 }
@@ -253,6 +260,7 @@ __device__ __forceinline__ void finish_edges(const FinishArgs& p, int64_t plane,
 // BF16: the four corner pixels of a plane with H, W >= 2, recomputed:
 // dx = sum_{i,j <= r} C[i][j] dy[i][j], rows and columns counted from the
 // corner, C[i][j] = the sum of the taps that bring (i, j) there.
+template <int NT>
 __device__ __forceinline__ void finish_corners_bf16(const FinishArgs& p, int64_t plane,
                                                     float* tab) {
   const int K = p.K, r = (K - 1) / 2, H = p.H, W = p.W, D = r + 1;
@@ -260,12 +268,12 @@ __device__ __forceinline__ void finish_corners_bf16(const FinishArgs& p, int64_t
   const __nv_bfloat16* g = static_cast<const __nv_bfloat16*>(p.dy) + plane * (int64_t)H * W;
   float* wc = tab;               // [2][D][K]: a column edge's weights of filter row a
   float* prod = wc + 2 * D * K;  // [4][D][D]
-  for (int k = threadIdx.x; k < 2 * D * K; k += kFinishThreads) {
+  for (int k = threadIdx.x; k < 2 * D * K; k += NT) {
     const int e = k / (D * K), j = k / K - e * D, a = k - (k / K) * K;
     wc[k] = fold_weight<__nv_bfloat16>(f + a * K, 1, K, e, j);
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < 4 * D * D; k += kFinishThreads) {
+  for (int k = threadIdx.x; k < 4 * D * D; k += NT) {
     const int q = k / (D * D), i = k / D - q * D, j = k - (k / D) * D;
     const int er = q >> 1, ec = q & 1;
     const float c = fold_weight<__nv_bfloat16>(wc + (ec * D + j) * K, 1, K, er, i);
@@ -286,6 +294,7 @@ __device__ __forceinline__ void finish_corners_bf16(const FinishArgs& p, int64_t
 
 // The corner pixels of a plane (one, two or four): the row sums, then the
 // column sums with the doubly folded corner terms.
+template <int NT>
 __device__ __forceinline__ void finish_corners(const FinishArgs& p, int64_t plane, float* tab) {
   const int K = p.K, r = (K - 1) / 2, H = p.H, W = p.W;
   const float* f = p.w + (plane % p.C) * (int64_t)K * K;
@@ -297,14 +306,14 @@ __device__ __forceinline__ void finish_corners(const FinishArgs& p, int64_t plan
   float* sums = sq + 4 * (r + 1) * (r + 1);  // [8]
   const int S = r + 1;
   const float* g = static_cast<const float*>(p.dy) + plane * (int64_t)H * W;
-  for (int k = threadIdx.x; k < K * K; k += kFinishThreads) sf[k] = __ldg(f + k);
-  for (int k = threadIdx.x; k < 4 * S * S; k += kFinishThreads) {
+  for (int k = threadIdx.x; k < K * K; k += NT) sf[k] = __ldg(f + k);
+  for (int k = threadIdx.x; k < 4 * S * S; k += NT) {
     const int q = k / (S * S), i = k / S - q * S, j = k - (k / S) * S;
     const int row = (q >> 1) ? H - 1 - i : i, col = (q & 1) ? W - 1 - j : j;
     sq[k] = dy_at(g, H, W, row, col);
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < 4 * r * K; k += kFinishThreads) {
+  for (int k = threadIdx.x; k < 4 * r * K; k += NT) {
     const int rows = k < 2 * r * K, kk = rows ? k : k - 2 * r * K;
     const int e = kk / (r * K), i = kk / K - e * r, b = kk - (kk / K) * K;
     float t = 0.f;
@@ -313,7 +322,7 @@ __device__ __forceinline__ void finish_corners(const FinishArgs& p, int64_t plan
     (rows ? wr : wc)[kk] = t;
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < 4 * r * r; k += kFinishThreads) {
+  for (int k = threadIdx.x; k < 4 * r * r; k += NT) {
     const int q = k / (r * r), i = k / r - q * r, j = k - (k / r) * r;
     const int er = q >> 1, ec = q & 1;
     const int lo = er ? r + 1 + i : 0, hi = er ? K - 1 : r - 1 - i;
@@ -362,11 +371,11 @@ __device__ __forceinline__ void finish_corners(const FinishArgs& p, int64_t plan
   }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kFinishThreads) dw_finish_kernel(const FinishArgs p) {
+template <typename T, int NT>
+__global__ void __launch_bounds__(NT, 1536 / NT) dw_finish_kernel(const FinishArgs p) {
   extern __shared__ __align__(16) float fin_smem[];
   if ((int)blockIdx.x < p.sum_blocks) {
-    finish_sums(p, reinterpret_cast<double*>(fin_smem));
+    finish_sums<NT>(p, reinterpret_cast<double*>(fin_smem));
     return;
   }
   const uint32_t b = blockIdx.x - p.sum_blocks;
@@ -374,22 +383,47 @@ __global__ void __launch_bounds__(kFinishThreads) dw_finish_kernel(const FinishA
   const int64_t plane = p.plane0 + b / per;
   const int k = (int)(b - b / per * per);
   if (k < p.row_blocks)
-    finish_edges<T>(p, plane, k, true, fin_smem);
+    finish_edges<T, NT>(p, plane, k, true, fin_smem);
   else if (k < p.row_blocks + p.col_blocks)
-    finish_edges<T>(p, plane, k - p.row_blocks, false, fin_smem);
+    finish_edges<T, NT>(p, plane, k - p.row_blocks, false, fin_smem);
   else if constexpr (sizeof(T) == 2)
-    finish_corners_bf16(p, plane, fin_smem);
+    finish_corners_bf16<NT>(p, plane, fin_smem);
   else
-    finish_corners(p, plane, fin_smem);
+    finish_corners<NT>(p, plane, fin_smem);
+}
+
+// Blocks of 128 threads: where the planes' edges fit two of their fold blocks, or
+// without a fold where 1024 partial sums (eight per thread) are all a block adds.
+static bool finish_small(const DwArgs& a, bool folds, int64_t rows, int taps) {
+  return folds ? std::max(a.H, a.W) <= 128 : rows * taps <= 1024;
+}
+
+template <int NT>
+static void finish_run(const DwArgs& a, const FinishArgs& p, unsigned blocks, size_t smem,
+                       cudaStream_t st) {
+  if (a.dtype == 0)
+    dw_finish_kernel<float, NT><<<blocks, NT, smem, st>>>(p);
+  else
+    dw_finish_kernel<__nv_bfloat16, NT><<<blocks, NT, smem, st>>>(p);
+}
+
+// BF16 planes one pixel high or wide, where an edge pixel lies on both edges;
+// and more planes than their fold blocks run at once (12 of 128 threads per SM,
+// three per plane) with so few taps at their edges that a thread per edge pixel
+// does less than a block spends on its tables: at most 800 per plane, from 4 x S
+// planes on (4096 planes, thread per pixel against blocks, us: 7 x 7 K = 3 6 / 17,
+// K = 5 15 / 19; 14 x 14 K = 3 9 / 17, K = 5 23 / 19).
+static bool fold_by_pixel(const DwArgs& a) {
+  return a.H == 1 || a.W == 1 ||
+         (a.N * a.C >= 4 * (int64_t)sm_count() && edge_pixels(a.H, a.W) * a.K * a.K <= 800);
 }
 
 cudaError_t dw_finish_launch(const DwArgs& a, bool fold, int64_t chunks_per_plane,
                              cudaStream_t st) {
   const int r = (a.K - 1) / 2;
   const bool folds = fold && a.border == 1 && r > 0 && a.N * a.C * a.H * a.W > 0;
-  // BF16 planes one pixel high or wide, where an edge pixel lies on both edges
-  const bool thin = a.dtype != 0 && (a.H == 1 || a.W == 1);
-  if (folds && thin) {
+  const bool by_pixel = folds && a.dtype != 0 && fold_by_pixel(a);
+  if (by_pixel) {
     const int64_t edge = edge_pixels(a.H, a.W);
     const int64_t total = a.N * a.C * edge;
     const int threads = 128;
@@ -408,32 +442,36 @@ cudaError_t dw_finish_launch(const DwArgs& a, bool fold, int64_t chunks_per_plan
   p.chunks = make_fastdiv(1);
   size_t smem = 0;
   int64_t blocks = 0, planes = 0, per = 0;
+  const bool edges_too = folds && !by_pixel;
+  const int taps = chunks_per_plane > 0 ? finish_taps(a.C, a.K * a.K) : 1;
+  const bool small = finish_small(a, edges_too, a.N * chunks_per_plane, taps);
+  const int nt = small ? kFinishThreadsSmall : kFinishThreads, P = nt / 2;
   if (chunks_per_plane > 0) {
     if (a.N * chunks_per_plane >= (1LL << 31)) return cudaErrorInvalidConfiguration;
     p.partials = a.partials;
     p.dw = a.dw;
     p.KK = a.K * a.K;
-    p.taps = finish_taps(a.C, p.KK);
+    p.taps = taps;
     p.groups = (p.KK + p.taps - 1) / p.taps;
     p.chunks = make_fastdiv((uint32_t)chunks_per_plane);
     blocks = a.C * p.groups;
     if (blocks >= (1LL << 31)) return cudaErrorInvalidConfiguration;
     p.sum_blocks = (int)blocks;
-    smem = kFinishThreads * sizeof(double);
+    smem = nt * sizeof(double);
   }
-  if (folds && !thin) {
+  if (edges_too) {
     p.dy = a.dy;
     p.w = a.w;
     p.dx = a.dx;
     p.H = (int)a.H;
     p.W = (int)a.W;
     p.K = a.K;
-    p.row_blocks = (int)((a.W + kFoldPixels - 1) / kFoldPixels);
-    p.col_blocks = (int)((a.H + kFoldPixels - 1) / kFoldPixels);
+    p.row_blocks = (int)((a.W + P - 1) / P);
+    p.col_blocks = (int)((a.H + P - 1) / P);
     planes = a.N * a.C;
     per = (int64_t)p.row_blocks + p.col_blocks + 1;
     const int D = a.dtype == 0 ? r : r + 1;  // fold_depth
-    const size_t edges = a.K * a.K + 2 * D * a.K + 2 * D * (kFoldPixels + 2 * r);
+    const size_t edges = a.K * a.K + 2 * D * a.K + 2 * D * (P + 2 * r);
     const size_t corners = a.K * a.K + 4 * D * a.K + 4 * r * r + 4 * (r + 1) * (r + 1) + 8;
     smem = std::max(smem, std::max(edges, corners) * sizeof(float));
   }
@@ -442,10 +480,10 @@ cudaError_t dw_finish_launch(const DwArgs& a, bool fold, int64_t chunks_per_plan
     const int64_t now = per ? std::min<int64_t>(planes - p.plane0, (0x7fffffffLL - blocks) / per) : 0;
     blocks += now * per;
     if (blocks == 0) return cudaSuccess;
-    if (a.dtype == 0)
-      dw_finish_kernel<float><<<(unsigned)blocks, kFinishThreads, smem, st>>>(p);
+    if (small)
+      finish_run<kFinishThreadsSmall>(a, p, (unsigned)blocks, smem, st);
     else
-      dw_finish_kernel<__nv_bfloat16><<<(unsigned)blocks, kFinishThreads, smem, st>>>(p);
+      finish_run<kFinishThreads>(a, p, (unsigned)blocks, smem, st);
     note_launch();
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
