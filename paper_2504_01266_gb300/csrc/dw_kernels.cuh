@@ -213,50 +213,71 @@ __device__ __forceinline__ void stage_any(T* __restrict__ sm, const T* plane, in
   const bool inside = j0 >= 1 && j0 + kTileW <= W;
   const T* row = plane + (int64_t)(ty0 - R + w0) * W;
   T* dst = sm + w0 * pitch;
-  for (int sr = w0; sr < rows; sr += NT / 32) {
-    const int gi = ty0 - R + sr;
-    const bool row_ok = gi >= 0 && gi < H;
-    if (inside && row_ok) {
-      const uint32_t a = (uint32_t)reinterpret_cast<uintptr_t>(row) & 15u;
-      if constexpr (ES == 4) {
-        if (a == 0) {
-          cp_async16(dst + 4 * lane, row + j0 + 4 * lane, true);
-        } else if (a == 8) {
-#pragma unroll
-          for (int q = 0; q < 2; ++q)
-            cp_async8(dst + 2 * lane + 64 * q, row + j0 + 2 * lane + 64 * q, true);
-        } else {
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            cp_async4(dst + lane + 32 * q, row + j0 + lane + 32 * q, true);
-        }
+  if (ES == 4 && 2 * H < rows) {
+    // most rows lie outside the image: one store a lane for those (a loop of its
+    // own, because the choice inside the other costs that one registers: 8 x 512
+    // planes of 7 x 7, K = 3 34 -> 26 us; inside, W = 2399 K = 3 75 -> 77)
+    for (int sr = w0; sr < rows; sr += NT / 32) {
+      if (ty0 - R + sr < 0 || ty0 - R + sr >= H) {
+        *reinterpret_cast<float4*>(dst + 4 * lane) = make_float4(0.f, 0.f, 0.f, 0.f);
       } else {
-        if ((a & 7) == 0) {
-          cp_async8(dst + 4 * lane, row + j0 + 4 * lane, true);
-        } else {
-          const int p = row_is_odd(row);
-#pragma unroll
-          for (int q = 0; q < 2; ++q)
-            cp_async4(reinterpret_cast<float*>(dst + 2 * lane + 64 * q),
-                      row + j0 - p + 2 * lane + 64 * q, true);
+        for (int q = 0; q < 4; ++q) {
+          const int j = j0 + lane + 32 * q;
+          const bool in = j >= 0 && j < W;
+          cp_async4(reinterpret_cast<float*>(dst) + lane + 32 * q, in ? row + j : plane, in);
         }
       }
-    } else if constexpr (ES == 4) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int j = j0 + lane + 32 * q;
-        const bool in = row_ok && j >= 0 && j < W;
-        cp_async4(dst + lane + 32 * q, in ? row + j : plane, in);
-      }
-    } else {
-      const int p = row_is_odd(row);
-#pragma unroll
-      for (int q = 0; q < 2; ++q)
-        stage_bf16_word(reinterpret_cast<uint32_t*>(dst) + lane + 32 * q, row,
-                        j0 - p + 2 * (lane + 32 * q), W, row_ok);
+      row += (int64_t)(NT / 32) * W;
+      dst += NT / 32 * pitch;
     }
-    row += (int64_t)(NT / 32) * W;
-    dst += NT / 32 * pitch;
+  } else {
+    for (int sr = w0; sr < rows; sr += NT / 32) {
+      const int gi = ty0 - R + sr;
+      const bool row_ok = gi >= 0 && gi < H;
+      if (inside && row_ok) {
+        const uint32_t a = (uint32_t)reinterpret_cast<uintptr_t>(row) & 15u;
+        if constexpr (ES == 4) {
+          if (a == 0) {
+            cp_async16(dst + 4 * lane, row + j0 + 4 * lane, true);
+          } else if (a == 8) {
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+              cp_async8(dst + 2 * lane + 64 * q, row + j0 + 2 * lane + 64 * q, true);
+          } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              cp_async4(dst + lane + 32 * q, row + j0 + lane + 32 * q, true);
+          }
+        } else {
+          if ((a & 7) == 0) {
+            cp_async8(dst + 4 * lane, row + j0 + 4 * lane, true);
+          } else {
+            const int p = row_is_odd(row);
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+              cp_async4(reinterpret_cast<float*>(dst + 2 * lane + 64 * q),
+                        row + j0 - p + 2 * lane + 64 * q, true);
+          }
+        }
+      } else if constexpr (ES == 4) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int j = j0 + lane + 32 * q;
+          const bool in = row_ok && j >= 0 && j < W;
+          cp_async4(dst + lane + 32 * q, in ? row + j : plane, in);
+        }
+      } else if (!row_ok) {  // most rows of a tile over a small image: one store a lane
+        *reinterpret_cast<uint2*>(dst + 4 * lane) = make_uint2(0u, 0u);
+      } else {
+        const int p = row_is_odd(row);
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+          stage_bf16_word(reinterpret_cast<uint32_t*>(dst) + lane + 32 * q, row,
+                          j0 - p + 2 * (lane + 32 * q), W, true);
+      }
+      row += (int64_t)(NT / 32) * W;
+      dst += NT / 32 * pitch;
+    }
   }
   // columns kTileW .. kTileW + RP + R - 1 of every row (BF16: whole words, one
   // more column where rows are to be shifted)
