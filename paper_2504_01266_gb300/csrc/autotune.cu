@@ -12,6 +12,7 @@
 // Problem class: (op, dtype, K, border, floor(log2(N*C*H*W))).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -73,14 +74,15 @@ static int auto_tiles_per_cta(const DwArgs& a) {
 // The persistent filter kernel runs one CTA per SM over chunks dealt round
 // robin; a chunk ends with a reduction of the accumulators costing about a
 // fifth of a tile.  Pick the chunk length (<= 16 tiles) minimising the
-// busiest CTA's rounds x (tiles + 0.2).
-static int auto_filter_tiles_per_chunk(const DwArgs& a) {
+// busiest CTA's rounds x (tiles + 0.2), of at most max_tiles.
+static int auto_filter_tiles_per_chunk(const DwArgs& a, int max_tiles = 16) {
   const int64_t tpp = (int64_t)((a.W + kTileW - 1) / kTileW) * (int64_t)((a.H + 63) / 64);
   const int64_t planes = a.N * a.C;
   const int64_t G = sm_count();
   int best = 1;
   double best_cost = 1e300;
   for (int tpc = 16; tpc >= 1; tpc /= 2) {
+    if (tpc > max_tiles) continue;
     const int64_t chunks = planes * ((tpp + tpc - 1) / tpc);
     const double cost = (double)((chunks + G - 1) / G) * (tpc + 0.2);
     if (cost < best_cost * 0.999) {
@@ -89,6 +91,16 @@ static int auto_filter_tiles_per_chunk(const DwArgs& a) {
     }
   }
   return best;
+}
+
+// Chunk length of both gradients as two passes: a lane of the filter kernel adds
+// the terms of a chunk one after the other in FP32, 4 rows of every tile for K <=
+// 7, 8 for K = 11, 16 else.  No more tiles than keep that as short as four warps
+// of a fused kernel with the automatic chunks do: 16 rows for K <= 7, 32 for K = 9
+// and 11, 64 above.
+static int split_tiles_per_chunk(const DwArgs& a) {
+  return auto_filter_tiles_per_chunk(
+      a, std::min(16, (a.K == 9 ? 2 : 4) * auto_tiles_per_cta(a)));
 }
 
 DwConfig tune_config(int op, int id, const DwArgs& a) {
@@ -115,7 +127,7 @@ DwConfig tune_config(int op, int id, const DwArgs& a) {
       if (id == 5 || id == 6) {
         c.split = id == 5;
         c.ring = id == 6;
-        c.tiles_per_cta = auto_filter_tiles_per_chunk(a);
+        c.tiles_per_cta = c.split ? split_tiles_per_chunk(a) : auto_filter_tiles_per_chunk(a);
       }
       break;
   }

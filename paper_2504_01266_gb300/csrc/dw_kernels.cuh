@@ -618,10 +618,12 @@ __device__ __forceinline__ void fwd_block(const TS* __restrict__ win,
 // staged x row (block row 0 + a_lo) at the lane's first column.  NR is a
 // compile-time constant: the unrolled body has no data-dependent control flow
 // (with a run-time row count the accumulators live across guarded paths and
-// are copied where those paths merge).
-template <int K, int NR, int AT, int DYP, int DR, typename TS, bool RAW>
+// are copied where those paths merge).  With SETS = 2 the two halves of a block's
+// dy rows have accumulators of their own (rows AT .. 2 AT - 1 of acc): half as
+// many terms are added one after the other.
+template <int K, int NR, int AT, int DYP, int DR, typename TS, bool RAW, int SETS>
 __device__ __forceinline__ void dw_block(const TS* __restrict__ dyb,
-                                         const TS* __restrict__ xw, float (&acc)[AT][K]) {
+                                         const TS* __restrict__ xw, float (&acc)[SETS * AT][K]) {
   static_assert(NR >= 1 && NR <= AT, "row count");
   using G = Geo<K, sizeof(TS), RAW>;
   float d[DR][4];
@@ -644,8 +646,10 @@ __device__ __forceinline__ void dw_block(const TS* __restrict__ dyb,
 #pragma unroll
         for (int b = 0; b < K; ++b)
 #pragma unroll
-          for (int px = 0; px < 4; ++px)
-            acc[s][b] = fmaf(d[py][px], buf[G::OFFR + px + b], acc[s][b]);
+          for (int px = 0; px < 4; ++px) {
+            float& t = acc[py * SETS / DR * AT + s][b];
+            t = fmaf(d[py][px], buf[G::OFFR + px + b], t);
+          }
       }
     }
   }
@@ -655,23 +659,23 @@ __device__ __forceinline__ void dw_block(const TS* __restrict__ dyb,
 // `nrows` rows.  Splitting K rows into GT groups gives groups of AT or
 // AT - 1 rows; the branch on the (warp-uniform, fixed) row count is taken
 // once, outside the unrolled bodies.
-template <int K, int AT, int GT, int DYP, int DR, typename TS, bool RAW>
+template <int K, int AT, int GT, int DYP, int DR, typename TS, bool RAW, int SETS = 1>
 __device__ __forceinline__ void dw_rows(const TS* __restrict__ dyb, const TS* __restrict__ xw,
-                                        int nblocks, int nrows, float (&acc)[AT][K]) {
+                                        int nblocks, int nrows, float (&acc)[SETS * AT][K]) {
   constexpr int SP = Geo<K, sizeof(TS), RAW>::SP;
   if constexpr (K % GT == 0) {
 #pragma unroll 1
     for (int i = 0; i < nblocks; ++i)
-      dw_block<K, AT, AT, DYP, DR, TS, RAW>(dyb + i * DR * DYP, xw + i * DR * SP, acc);
+      dw_block<K, AT, AT, DYP, DR, TS, RAW, SETS>(dyb + i * DR * DYP, xw + i * DR * SP, acc);
   } else {
     if (nrows == AT) {
 #pragma unroll 1
       for (int i = 0; i < nblocks; ++i)
-        dw_block<K, AT, AT, DYP, DR, TS, RAW>(dyb + i * DR * DYP, xw + i * DR * SP, acc);
+        dw_block<K, AT, AT, DYP, DR, TS, RAW, SETS>(dyb + i * DR * DYP, xw + i * DR * SP, acc);
     } else {
 #pragma unroll 1
       for (int i = 0; i < nblocks; ++i)
-        dw_block<K, AT - 1, AT, DYP, DR, TS, RAW>(dyb + i * DR * DYP, xw + i * DR * SP, acc);
+        dw_block<K, AT - 1, AT, DYP, DR, TS, RAW, SETS>(dyb + i * DR * DYP, xw + i * DR * SP, acc);
     }
   }
 }
@@ -1241,7 +1245,7 @@ static_assert(kFilterTileH == kBwdTileH, "both filter-gradient kernels share the
 // into 8-row dy blocks: 14 x rows per block instead of the 20 that two 4-row
 // blocks take, and that shared-memory traffic was what 16 warps of 4 rows
 // waited for.  16 x 3 x 2048^2, 16 warps -> 8 warps (us), FP32 / BF16: K = 5
-// 281 -> 253 / 300 -> 233, K = 7 454 -> 398 / 472 -> 404.  From K = 9 on, 12
+// 281 -> 253 / 300 -> 233, K = 7 458 -> 412 / 488 -> 447.  From K = 9 on, 12
 // warps in 3 groups (up to 168 registers): K = 9 with 8-row blocks 658 -> 638 /
 // 701 -> 664, K = 11 948 -> 935 / 1013 -> 1009, K = 13 1235 -> 1240 / 1488 ->
 // 1379 against 16 warps; 8-row blocks lose at K >= 11 (K = 11 1077, K = 15
@@ -1255,6 +1259,17 @@ constexpr int filter_groups() {
   return K <= 7 ? 1 : 3;
 }
 
+// Accumulators per tap and lane: two where fewer warps leave a lane twice the
+// rows that 16 warps would, so that no more terms are added one after the other
+// in FP32 than there (4 rows of a tile up to K = 7, 8 at K = 11).  With one, the
+// error against FP64 was 1.3 times that of 16 warps; the second costs registers
+// that are free but at BF16 K = 7, where two CTAs per SM become one (16 x 3 x
+// 2048^2 411 -> 448 us, W = 2399 227 -> 293).
+template <int K>
+constexpr int filter_sets() {
+  return K <= 7 || K == 11 ? 2 : 1;
+}
+
 template <int K, typename T, bool AL>
 struct FilterShape {
   using G = Geo<K, sizeof(T), !AL>;  // tiles stay in the storage type (no widening pass)
@@ -1266,6 +1281,7 @@ struct FilterShape {
   static constexpr int AT = (K + GT - 1) / GT;
   static constexpr int ROWS = kFilterTileH / WPG;  // tile rows per warp
   static constexpr int DR = K <= 9 ? 8 : 4;        // dy rows per unrolled block
+  static constexpr int SETS = filter_sets<K>();
   static constexpr int X_ROWS = kFilterTileH + 2 * G::R;
   static constexpr int X_BYTES = X_ROWS * G::SP * (int)sizeof(T);
   static constexpr int DY_BYTES = kFilterTileH * DYP * (int)sizeof(T);
@@ -1372,9 +1388,9 @@ __global__ void __launch_bounds__(FilterShape<K, T, AL>::NT, 1)
     cp_async_commit();
   }
 
-  float acc[S::AT][K];
+  float acc[S::SETS * S::AT][K];
 #pragma unroll
-  for (int s = 0; s < S::AT; ++s)
+  for (int s = 0; s < S::SETS * S::AT; ++s)
 #pragma unroll
     for (int b = 0; b < K; ++b) acc[s][b] = 0.f;
 
@@ -1412,7 +1428,7 @@ __global__ void __launch_bounds__(FilterShape<K, T, AL>::NT, 1)
       tile_origin(cs.t, ty0, tx0);
       clamp_fix<T, G::SP, S::NT>(sx, H, W, ty0, tx0, G::R, G::RP, S::X_ROWS);
     }
-    dw_rows<K, S::AT, S::GT, S::DYP, S::DR, T, !AL>(
+    dw_rows<K, S::AT, S::GT, S::DYP, S::DR, T, !AL, S::SETS>(
         sdy + part * S::ROWS * S::DYP + 4 * lane, sx + (part * S::ROWS + a_lo) * G::SP + 4 * lane,
         S::ROWS / S::DR, nrows, acc);
     const bool chunk_end = cs.t + 1 == cs.t_end;
@@ -1422,10 +1438,14 @@ __global__ void __launch_bounds__(FilterShape<K, T, AL>::NT, 1)
 #pragma unroll
         for (int b = 0; b < K; ++b) {
           float v = acc[s][b];
+          acc[s][b] = 0.f;
+          if constexpr (S::SETS == 2) {
+            v += acc[S::AT + s][b];
+            acc[S::AT + s][b] = 0.f;
+          }
 #pragma unroll
           for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
           if (lane == 0) sm_red[(warp * S::AT + s) * K + b] = v;
-          acc[s][b] = 0.f;
         }
     }
     cta_barrier();  // stage sb is free again; sm_red is complete
@@ -1470,6 +1490,10 @@ struct RingShape {
   static constexpr int AT = (K + GT - 1) / GT;
   static constexpr int DW_ROWS = kBwdTileH / WPG;
   static constexpr int BR = bwd_block_rows<K>();
+  // K <= 3 (the built-in choice from a tile count on, with up to 16 tiles per
+  // chunk): two accumulators per tap, added to the chunk's sum after every tile, so
+  // that FP32 adds no more terms one after the other than in chunks of one tile
+  static constexpr int SETS = K <= 3 ? 2 : 1;
   static constexpr int ROWS = kBwdTileH + 2 * G::R;
   static constexpr int T_BYTES = round_up(ROWS * G::SP * (int)sizeof(T), 128);
   static constexpr int STAGE_BYTES = 2 * T_BYTES;  // x, then dy (both with the halo)
@@ -1574,11 +1598,15 @@ __global__ void __launch_bounds__(kThreads, 1)
     cp_async_commit();
   }
 
-  float acc[S::AT][K];
+  float acc[S::SETS * S::AT][K];
+  float sum[S::AT][K];  // the chunk's (SETS = 2)
 #pragma unroll
-  for (int s = 0; s < S::AT; ++s)
+  for (int s = 0; s < S::SETS * S::AT; ++s)
 #pragma unroll
-    for (int b = 0; b < K; ++b) acc[s][b] = 0.f;
+    for (int b = 0; b < K; ++b) {
+      acc[s][b] = 0.f;
+      if (s < S::AT) sum[s][b] = 0.f;
+    }
   int nchunk = 0;  // chunks this CTA has finished (filter buffer parity)
   bool chunk_start = true;
 
@@ -1637,9 +1665,18 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     } else {
       const int r0 = part * S::DW_ROWS;
-      dw_rows<K, S::AT, S::GT, G::SP, S::BR, T, !AL>(
+      dw_rows<K, S::AT, S::GT, G::SP, S::BR, T, !AL, S::SETS>(
           sdy + (r0 + G::R) * G::SP + G::RP + 4 * lane, sx + (r0 + a_lo) * G::SP + 4 * lane,
           S::DW_ROWS / S::BR, nrows, acc);
+      if constexpr (S::SETS == 2) {
+#pragma unroll
+        for (int s = 0; s < S::AT; ++s)
+#pragma unroll
+          for (int b = 0; b < K; ++b) {
+            sum[s][b] += acc[s][b] + acc[S::AT + s][b];
+            acc[s][b] = acc[S::AT + s][b] = 0.f;
+          }
+      }
     }
     const bool chunk_end = cs.t + 1 == cs.t_end;
     if (chunk_end && dw_warp) {
@@ -1647,11 +1684,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int s = 0; s < S::AT; ++s)
 #pragma unroll
         for (int b = 0; b < K; ++b) {
-          float v = acc[s][b];
+          float& t = S::SETS == 2 ? sum[s][b] : acc[s][b];
+          float v = t;
+          t = 0.f;
 #pragma unroll
           for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
           if (lane == 0) sm_red[(wl * S::AT + s) * K + b] = v;
-          acc[s][b] = 0.f;
         }
     }
     cta_barrier();  // stage sb is free again; sm_red is complete
