@@ -530,13 +530,17 @@ __device__ __forceinline__ void store_rows(T* __restrict__ plane, int H, int W, 
   }
 }
 
-// Kernels compiled for aligned planes (AL) always store whole chunks; the
-// others choose per launch.  gj = tx0 + 4 * lane.
-template <typename T, int PY, bool AL>
+// How a kernel is compiled for its planes' alignment (AL): any planes
+// (stage_any, stores chosen per launch); inputs that TMA can load, output rows
+// at any alignment (a view into a larger tensor, say); both aligned.
+constexpr int kAnyPlanes = 0, kTmaLoads = 1, kAligned = 2;
+
+// The store that goes with it.  gj = tx0 + 4 * lane.
+template <typename T, int PY, int AL>
 __device__ __forceinline__ void store_tile(T* __restrict__ plane, int H, int W, int gi0, int tx0,
                                            bool vec, float* __restrict__ buf,
                                            const float (&acc)[PY][4]) {
-  if (AL || vec)
+  if (AL == kAligned || (AL == kAnyPlanes && vec))
     store_block<T, PY>(plane, H, W, gi0, tx0 + 4 * (int)(threadIdx.x & 31), acc);
   else
     store_rows<T, PY>(plane, H, W, gi0, tx0, buf, acc);
@@ -696,11 +700,9 @@ constexpr int bwd_block_rows() {
 // shared memory: while a tile is computed, the cp.async copies of the next
 // tile and of its plane's filter are in flight.  With flip = 1 the filter is
 // rotated by 180 degrees: that computes g (input gradient, zero border) from dy.
-// AL: input planes a TMA load can address and output rows that start on a
-// chunk boundary; the other compilation stages any plane (stage_any)
-// and stores any row (store_rows).  Apart, the aligned kernel carries neither
-// the code nor the registers of the general one.
-template <int K, int PY, typename T, bool AL>
+// AL (kAnyPlanes ..): apart, the aligned kernel carries neither the code nor the
+// registers of the general one.
+template <int K, int PY, typename T, int AL>
 struct FwdShape {
   using G = GeoC<K, T, !AL>;  // FP32 compute geometry
   static constexpr int TH = kWarps * PY;
@@ -709,12 +711,12 @@ struct FwdShape {
   static constexpr int W_OFF = ST::BYTES;  // FP32 tile (128-aligned), then the filter
   static constexpr int STAGE_BYTES = round_up(W_OFF + G::WPAD * 4, 128);
   // two mbarriers and the abort flag, then the row buffers of store_rows
-  static constexpr int HEAD = 128 + (AL ? 0 : kWarps * kRowBuf);
+  static constexpr int HEAD = 128 + (AL == kAligned ? 0 : kWarps * kRowBuf);
   static constexpr int SM_BYTES = HEAD + 2 * STAGE_BYTES;
   static constexpr int SM_BYTES_1 = HEAD + STAGE_BYTES;  // one tile per CTA
 };
 
-template <typename T, int K, int PY, bool AL>
+template <typename T, int K, int PY, int AL>
 __device__ __forceinline__ void dw_fwd_body(
     const CUtensorMap& tmx, const T* __restrict__ x, const float* __restrict__ w,
     T* __restrict__ y, FastDiv fc, int H, int W, FastDiv ftx, FastDiv fty, int64_t num_tiles,
@@ -748,7 +750,7 @@ __device__ __forceinline__ void dw_fwd_body(
     float* sw = reinterpret_cast<float*>(buf + S::W_OFF);
     const int c = plane - (int)(fdiv((uint32_t)plane, fc) * fc.d);
     stage_filter_async<K>(sw, w + (int64_t)c * K * K, flip != 0, kThreads);
-    if constexpr (AL) {
+    if constexpr (AL != kAnyPlanes) {
       cp_async_commit();
       if (threadIdx.x == 0) {
         fence_proxy_async();
@@ -792,7 +794,7 @@ __device__ __forceinline__ void dw_fwd_body(
     int ty0, tx0, plane;
     coords(t, ty0, tx0, plane);
     char* buf = sm + S::HEAD + sb * S::STAGE_BYTES;
-    if constexpr (AL) {
+    if constexpr (AL != kAnyPlanes) {
       if (!mbar_wait(bars + sb, (phase >> sb) & 1u)) {
         record_error(err, kDevErrTimeout);
         *s_abort = 1;
@@ -825,7 +827,7 @@ __device__ __forceinline__ void dw_fwd_body(
     mbar_wait(bars + (sb ^ 1), (phase >> (sb ^ 1)) & 1u);
 }
 
-template <typename T, int K, int PY, bool AL>
+template <typename T, int K, int PY, int AL>
 __global__ void __launch_bounds__(kThreads) dw_fwd_kernel(
     const __grid_constant__ CUtensorMap tmx, const T* __restrict__ x, const float* __restrict__ w,
     T* __restrict__ y, FastDiv fc, int H, int W, FastDiv ftx, FastDiv fty, int64_t num_tiles,
@@ -839,7 +841,7 @@ __global__ void __launch_bounds__(kThreads) dw_fwd_kernel(
 // of shared memory and the extra CTA per SM hides more of each CTA's tile
 // load; other sizes keep the default allocation (with this bound K = 3 and 15
 // lose registers they need).
-template <typename T, int K, int PY, bool AL>
+template <typename T, int K, int PY, int AL>
 __global__ void __launch_bounds__(kThreads, 5) dw_fwd_kernel_hi_occ(
     const __grid_constant__ CUtensorMap tmx, const T* __restrict__ x, const float* __restrict__ w,
     T* __restrict__ y, FastDiv fc, int H, int W, FastDiv ftx, FastDiv fty, int64_t num_tiles,
@@ -857,18 +859,18 @@ __global__ void __launch_bounds__(kThreads, 5) dw_fwd_kernel_hi_occ(
 // widened); the row pass writes t over the first 128 columns of the same
 // staged row (a warp owns whole rows and reads a row completely before it
 // writes it), then the column pass runs down t in 8-row register blocks.
-template <int K, typename T, bool AL>
+template <int K, typename T, int AL>
 struct SepShape {
   using G = GeoC<K, T, !AL>;
   static constexpr int TH = 64;
   static constexpr int ROWS = TH + 2 * G::R;
   using ST = HaloTile<K, T, ROWS, !AL>;
-  static constexpr int HEAD = 128 + (AL ? 0 : kWarps * kRowBuf);  // mbarrier, abort flag; row buffers
+  static constexpr int HEAD = 128 + (AL == kAligned ? 0 : kWarps * kRowBuf);  // mbarrier, abort flag; row buffers
   static constexpr int W_OFF = HEAD + ST::BYTES;  // wrow then wcol, K floats each (padded)
   static constexpr int SM_BYTES = W_OFF + 2 * round_up(K, 4) * 4;
 };
 
-template <typename T, int K, bool AL>
+template <typename T, int K, int AL>
 __device__ __forceinline__ void dw_sep_body(
     const CUtensorMap& tmx, const T* __restrict__ x, const float* __restrict__ wcol,
     const float* __restrict__ wrow, T* __restrict__ y, FastDiv fc, int H, int W, FastDiv ftx,
@@ -906,7 +908,7 @@ __device__ __forceinline__ void dw_sep_body(
   }
   cta_barrier();
   T* staged = reinterpret_cast<T*>(sm + S::HEAD + ST::STAGE_OFF);
-  if constexpr (AL) {
+  if constexpr (AL != kAnyPlanes) {
     cp_async_commit();
     if (threadIdx.x == 0) {
       fence_proxy_async();
@@ -1000,7 +1002,7 @@ __device__ __forceinline__ void dw_sep_body(
                         reinterpret_cast<float*>(sm + 128 + warp * kRowBuf), acc);
 }
 
-template <typename T, int K, bool AL>
+template <typename T, int K, int AL>
 __global__ void __launch_bounds__(kThreads) dw_sep_kernel(
     const __grid_constant__ CUtensorMap tmx, const T* __restrict__ x,
     const float* __restrict__ wcol, const float* __restrict__ wrow, T* __restrict__ y, FastDiv fc,
@@ -1013,7 +1015,7 @@ __global__ void __launch_bounds__(kThreads) dw_sep_kernel(
 // whose pass waits on its tile loads (K = 15: 0.701 -> 0.689 ms on
 // 8 x 3 x 4096^2, before the factors were pinned), and for BF16 K <= 3, which
 // would take 50 registers and four CTAs (4 x 3 x 1801 x 2400: 67 -> 61 us).
-template <typename T, int K, bool AL>
+template <typename T, int K, int AL>
 __global__ void __launch_bounds__(kThreads, 5) dw_sep_kernel_hi_occ(
     const __grid_constant__ CUtensorMap tmx, const T* __restrict__ x,
     const float* __restrict__ wcol, const float* __restrict__ wrow, T* __restrict__ y, FastDiv fc,
@@ -1045,7 +1047,7 @@ __global__ void __launch_bounds__(kThreads, 5) dw_sep_kernel_hi_occ(
 //    blocks; it gains at odd heights).
 //  * CTAs per SM: three where the registers allow, so that more loads are in
 //    flight (K = 3 304, against 368 with two).
-template <int K, typename T, bool AL>
+template <int K, typename T, int AL>
 struct BwdTune {
   static constexpr bool F32 = sizeof(T) == 4;
   static constexpr int GROUPS =
@@ -1056,7 +1058,7 @@ struct BwdTune {
   static constexpr int MIN_CTAS = K <= 3 || (AL && (K == 5 || (K == 7 && F32))) ? 3 : 2;
 };
 
-template <int K, typename T, bool AL>
+template <int K, typename T, int AL>
 struct BwdShape {
   using G = GeoC<K, T, !AL>;  // FP32 compute geometry
   using Tune = BwdTune<K, T, AL>;
@@ -1086,7 +1088,7 @@ struct BwdShape {
 
 __device__ __forceinline__ int group_lo(int g, int K, int GT) { return g * K / GT; }
 
-template <typename T, int K, bool AL>
+template <typename T, int K, int AL>
 __global__ void __launch_bounds__(kThreads, BwdTune<K, T, AL>::MIN_CTAS)
     dw_bwd_kernel(const __grid_constant__ CUtensorMap tmx,
                   const __grid_constant__ CUtensorMap tmdy, const T* __restrict__ x,
@@ -1130,7 +1132,7 @@ __global__ void __launch_bounds__(kThreads, BwdTune<K, T, AL>::MIN_CTAS)
   // false if a TMA wait gave up (every thread then leaves its tile loop).
   auto stage = [&](int ty0, int tx0) -> bool {
     cta_barrier();
-    if constexpr (AL) {
+    if constexpr (AL != kAnyPlanes) {
       cp_async_commit();
       if (threadIdx.x == 0) {
         fence_proxy_async();
@@ -1186,7 +1188,7 @@ __global__ void __launch_bounds__(kThreads, BwdTune<K, T, AL>::MIN_CTAS)
     dw_rows<K, S::AT, S::GT, G::SP, S::BW, float, !AL && sizeof(T) == 4>(
         sm_dy + (r0 + G::R) * G::SP + G::RP + 4 * lane, sm_x + (r0 + a_lo) * G::SP + 4 * lane, nb,
         nrows, acc);
-    if (!AL && !vec) cta_barrier();  // the x tile becomes the row buffers
+    if (AL != kAligned && !vec) cta_barrier();  // the x tile becomes the row buffers
 #pragma unroll 1
     for (int x0 = warp * 8; x0 < min(warp * 8 + 8, left); x0 += S::BX) {
       float o[S::BX][4];
@@ -1270,7 +1272,7 @@ constexpr int filter_sets() {
   return K <= 7 || K == 11 ? 2 : 1;
 }
 
-template <int K, typename T, bool AL>
+template <int K, typename T, int AL>
 struct FilterShape {
   using G = Geo<K, sizeof(T), !AL>;  // tiles stay in the storage type (no widening pass)
   static constexpr int DYP = geo_pitch(1, sizeof(T), !AL);  // dy tile pitch (no halo)
@@ -1295,7 +1297,7 @@ struct FilterShape {
   static_assert(SM_BYTES <= 227 * 1024, "shared memory");
 };
 
-template <typename T, int K, bool AL>
+template <typename T, int K, int AL>
 __global__ void __launch_bounds__(FilterShape<K, T, AL>::NT, 1)
     dw_filter_kernel(const __grid_constant__ CUtensorMap tmx,
                      const __grid_constant__ CUtensorMap tmdy, const T* __restrict__ x,
@@ -1350,7 +1352,7 @@ __global__ void __launch_bounds__(FilterShape<K, T, AL>::NT, 1)
     tile_origin(it.t, ty0, tx0);
     T* sx = reinterpret_cast<T*>(sm + sb * S::STAGE_BYTES);
     T* sdy = reinterpret_cast<T*>(sm + sb * S::STAGE_BYTES + S::DY_OFF);
-    if constexpr (AL) {
+    if constexpr (AL != kAnyPlanes) {
       if (threadIdx.x == 0) {
         fence_proxy_async();
         mbar_expect_tx(bars + sb, (uint32_t)(S::X_BYTES + S::DY_BYTES));
@@ -1481,7 +1483,7 @@ __global__ void __launch_bounds__(FilterShape<K, T, AL>::NT, 1)
 // tuning candidate for every K.  Tiles stay in the storage type (BF16 rows
 // are widened as they enter registers).  The rotated filter of a chunk's
 // channel goes to one of two buffers (chunk parity), written by the g warps.
-template <int K, typename T, bool AL>
+template <int K, typename T, int AL>
 struct RingShape {
   using G = Geo<K, sizeof(T), !AL>;
   static constexpr int NT = kThreads;
@@ -1498,7 +1500,7 @@ struct RingShape {
   static constexpr int T_BYTES = round_up(ROWS * G::SP * (int)sizeof(T), 128);
   static constexpr int STAGE_BYTES = 2 * T_BYTES;  // x, then dy (both with the halo)
   // three stages where they fit (two tiles in flight while one is computed)
-  static constexpr int BUFS = AL ? 0 : 4 * kRowBuf;  // row buffers of the dx warps
+  static constexpr int BUFS = AL == kAligned ? 0 : 4 * kRowBuf;  // row buffers of the dx warps
   static constexpr int NS = 3 * STAGE_BYTES + 2 * Geo<K>::WPAD * 4 + 4 * AT * K * 4 + BUFS + 64 <=
                                     227 * 1024
                                 ? 3
@@ -1512,7 +1514,7 @@ struct RingShape {
   static_assert(SM_BYTES <= 227 * 1024, "shared memory");
 };
 
-template <typename T, int K, bool AL>
+template <typename T, int K, int AL>
 __global__ void __launch_bounds__(kThreads, 1)
     dw_bwd_ring_kernel(const __grid_constant__ CUtensorMap tmx,
                        const __grid_constant__ CUtensorMap tmdy, const T* __restrict__ x,
@@ -1561,7 +1563,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tile_origin(it.t, ty0, tx0);
     T* sx = reinterpret_cast<T*>(sm + sb * S::STAGE_BYTES);
     T* sdy = reinterpret_cast<T*>(sm + sb * S::STAGE_BYTES + S::T_BYTES);
-    if constexpr (AL) {
+    if constexpr (AL != kAnyPlanes) {
       if (threadIdx.x == 0) {
         fence_proxy_async();
         mbar_expect_tx(bars + sb, (uint32_t)(2 * S::ROWS * G::SP * (int)sizeof(T)));

@@ -13,7 +13,7 @@ namespace giga {
 // The forward kernel of a launch: for FP32 K = 7 with one tile per CTA the
 // five-CTA-per-SM compilation (instantiated for that case only), else the
 // default one.  Raises the kernel's shared-memory limit first.
-template <typename T, int K, int PY, bool AL>
+template <typename T, int K, int PY, int AL>
 static cudaError_t fwd_kernel_for(bool persistent, size_t smem,
                                   decltype(&dw_fwd_kernel<T, K, PY, AL>)* kern) {
   if constexpr (sizeof(T) == 4 && K == 7 && PY == 8) {
@@ -29,9 +29,9 @@ static cudaError_t fwd_kernel_for(bool persistent, size_t smem,
 // persistent = 0 (the default, fastest on the measured workloads): one tile
 // per CTA and a single shared-memory stage (the kernel's prefetch branch never
 // runs because gridDim.x >= tiles); 1: as many CTAs as fit on the GPU, each
-// with two stages -- an autotuning candidate.  AL: the compilation for planes
-// that TMA loads and whole-chunk stores can address (`tm` is their map).
-template <typename T, int K, int PY, bool AL>
+// with two stages -- an autotuning candidate.  AL: the compilation for the
+// planes' alignment (`tm` is the map of TMA's input).
+template <typename T, int K, int PY, int AL>
 static cudaError_t fwd_run(const DwArgs& a, const CUtensorMap& tm, bool input_grad,
                            bool persistent, bool prefetch, cudaStream_t st) {
   using S = FwdShape<K, PY, T, AL>;
@@ -82,11 +82,12 @@ static cudaError_t fwd_impl(const DwArgs& a, bool input_grad, bool persistent, b
   const void* in = input_grad ? a.dy : a.x;
   CUtensorMap tm;
   std::memset(&tm, 0, sizeof(tm));
-  if (a.vec && plane_tma_ok(in, sizeof(T), a.W) &&
+  if (plane_tma_ok(in, sizeof(T), a.W) &&
       make_plane_map(&tm, in, sizeof(T), a.W, a.H, a.N * a.C, Geo<K, sizeof(T)>::SP,
-                     FwdShape<K, PY, T, true>::ROWS))
-    return fwd_run<T, K, PY, true>(a, tm, input_grad, persistent, prefetch, st);
-  return fwd_run<T, K, PY, false>(a, tm, input_grad, persistent, prefetch, st);
+                     FwdShape<K, PY, T, kAligned>::ROWS))
+    return a.vec ? fwd_run<T, K, PY, kAligned>(a, tm, input_grad, persistent, prefetch, st)
+                 : fwd_run<T, K, PY, kTmaLoads>(a, tm, input_grad, persistent, prefetch, st);
+  return fwd_run<T, K, PY, kAnyPlanes>(a, tm, input_grad, persistent, prefetch, st);
 }
 
 template <int K>
@@ -101,21 +102,20 @@ cudaError_t dw_fwd_launch(const DwArgs& a, const DwConfig& cfg, bool input_grad,
              : fwd_impl<__nv_bfloat16, K, 8>(a, input_grad, pers, pf, st);
 }
 
-// Tensor maps of x and dy for the aligned kernels, boxes of ROWS x SP (dy: of
-// rows_dy x pitch_dy); false: the general kernels run (`vec`: every tensor's
-// rows start on a chunk boundary).
+// Tensor maps of x and dy for TMA's loads, boxes of ROWS x SP (dy: of rows_dy x
+// pitch_dy); false: the kernels for any planes run.
 template <typename T, int K>
 static bool xdy_maps(const DwArgs& a, int rows, int rows_dy, int pitch_dy, CUtensorMap* tmx,
                      CUtensorMap* tmdy) {
   constexpr int es = sizeof(T);
   std::memset(tmx, 0, sizeof(*tmx));
   std::memset(tmdy, 0, sizeof(*tmdy));
-  return a.vec && plane_tma_ok(a.x, es, a.W) && plane_tma_ok(a.dy, es, a.W) &&
+  return plane_tma_ok(a.x, es, a.W) && plane_tma_ok(a.dy, es, a.W) &&
          make_plane_map(tmx, a.x, es, a.W, a.H, a.N * a.C, Geo<K, es>::SP, rows) &&
          make_plane_map(tmdy, a.dy, es, a.W, a.H, a.N * a.C, pitch_dy, rows_dy);
 }
 
-template <typename T, int K, bool AL>
+template <typename T, int K, int AL>
 static cudaError_t bwd_run(const DwArgs& a, const CUtensorMap& tmx, const CUtensorMap& tmdy,
                            const DwConfig& cfg, cudaStream_t st) {
   using S = BwdShape<K, T, AL>;
@@ -139,11 +139,12 @@ static cudaError_t bwd_run(const DwArgs& a, const CUtensorMap& tmx, const CUtens
 
 template <typename T, int K>
 static cudaError_t bwd_impl(const DwArgs& a, const DwConfig& cfg, cudaStream_t st) {
-  constexpr int rows = BwdShape<K, T, true>::ROWS;
+  constexpr int rows = BwdShape<K, T, kAligned>::ROWS;
   CUtensorMap tmx, tmdy;
-  return xdy_maps<T, K>(a, rows, rows, Geo<K, sizeof(T)>::SP, &tmx, &tmdy)
-             ? bwd_run<T, K, true>(a, tmx, tmdy, cfg, st)
-             : bwd_run<T, K, false>(a, tmx, tmdy, cfg, st);
+  if (!xdy_maps<T, K>(a, rows, rows, Geo<K, sizeof(T)>::SP, &tmx, &tmdy))
+    return bwd_run<T, K, kAnyPlanes>(a, tmx, tmdy, cfg, st);
+  return a.vec ? bwd_run<T, K, kAligned>(a, tmx, tmdy, cfg, st)
+               : bwd_run<T, K, kTmaLoads>(a, tmx, tmdy, cfg, st);
 }
 
 template <int K>
@@ -155,7 +156,7 @@ cudaError_t dw_bwd_launch(const DwArgs& a, const DwConfig& cfg, cudaStream_t st)
   }
 }
 
-template <typename T, int K, bool AL>
+template <typename T, int K, int AL>
 static cudaError_t bwd_ring_run(const DwArgs& a, const CUtensorMap& tmx, const CUtensorMap& tmdy,
                                 const DwConfig& cfg, cudaStream_t st) {
   using S = RingShape<K, T, AL>;
@@ -192,11 +193,12 @@ static cudaError_t bwd_ring_run(const DwArgs& a, const CUtensorMap& tmx, const C
 
 template <typename T, int K>
 static cudaError_t bwd_ring_impl(const DwArgs& a, const DwConfig& cfg, cudaStream_t st) {
-  constexpr int rows = RingShape<K, T, true>::ROWS;
+  constexpr int rows = RingShape<K, T, kAligned>::ROWS;
   CUtensorMap tmx, tmdy;
-  return xdy_maps<T, K>(a, rows, rows, Geo<K, sizeof(T)>::SP, &tmx, &tmdy)
-             ? bwd_ring_run<T, K, true>(a, tmx, tmdy, cfg, st)
-             : bwd_ring_run<T, K, false>(a, tmx, tmdy, cfg, st);
+  if (!xdy_maps<T, K>(a, rows, rows, Geo<K, sizeof(T)>::SP, &tmx, &tmdy))
+    return bwd_ring_run<T, K, kAnyPlanes>(a, tmx, tmdy, cfg, st);
+  return a.vec ? bwd_ring_run<T, K, kAligned>(a, tmx, tmdy, cfg, st)
+               : bwd_ring_run<T, K, kTmaLoads>(a, tmx, tmdy, cfg, st);
 }
 
 template <int K>
@@ -209,7 +211,7 @@ cudaError_t dw_bwd_ring_launch(const DwArgs& a, const DwConfig& cfg, cudaStream_
   }
 }
 
-template <typename T, int K, bool AL>
+template <typename T, int K, int AL>
 static cudaError_t filter_run(const DwArgs& a, const CUtensorMap& tmx, const CUtensorMap& tmdy,
                               const DwConfig& cfg, cudaStream_t st) {
   using S = FilterShape<K, T, AL>;
@@ -249,9 +251,9 @@ static cudaError_t filter_run(const DwArgs& a, const CUtensorMap& tmx, const CUt
 template <typename T, int K>
 static cudaError_t filter_impl(const DwArgs& a, const DwConfig& cfg, cudaStream_t st) {
   CUtensorMap tmx, tmdy;
-  return xdy_maps<T, K>(a, FilterShape<K, T, true>::X_ROWS, kFilterTileH, kTileW, &tmx, &tmdy)
-             ? filter_run<T, K, true>(a, tmx, tmdy, cfg, st)
-             : filter_run<T, K, false>(a, tmx, tmdy, cfg, st);
+  return xdy_maps<T, K>(a, FilterShape<K, T, kAligned>::X_ROWS, kFilterTileH, kTileW, &tmx, &tmdy)
+             ? filter_run<T, K, kAligned>(a, tmx, tmdy, cfg, st)
+             : filter_run<T, K, kAnyPlanes>(a, tmx, tmdy, cfg, st);
 }
 
 template <int K>
@@ -264,7 +266,7 @@ cudaError_t dw_filter_launch(const DwArgs& a, const DwConfig& cfg, cudaStream_t 
   }
 }
 
-template <typename T, int K, bool AL>
+template <typename T, int K, int AL>
 static cudaError_t sep_run(const DwArgs& a, const CUtensorMap& tm, const float* wcol,
                            const float* wrow, cudaStream_t st) {
   using S = SepShape<K, T, AL>;
@@ -272,7 +274,7 @@ static cudaError_t sep_run(const DwArgs& a, const CUtensorMap& tm, const float* 
   // those only)
   decltype(&dw_sep_kernel<T, K, AL>) kern = dw_sep_kernel<T, K, AL>;
   cudaError_t e;
-  if constexpr (AL && (sizeof(T) == 4 ? K == 13 || K == 15 : K <= 3)) {
+  if constexpr (AL == kAligned && (sizeof(T) == 4 ? K == 13 || K == 15 : K <= 3)) {
     kern = dw_sep_kernel_hi_occ<T, K, AL>;
     e = set_smem_once<dw_sep_kernel_hi_occ<T, K, AL>>((size_t)S::SM_BYTES);
   } else {
@@ -314,11 +316,12 @@ static cudaError_t sep_impl(const DwArgs& a, const float* wcol, const float* wro
                             cudaStream_t st) {
   CUtensorMap tm;
   std::memset(&tm, 0, sizeof(tm));
-  if (a.vec && plane_tma_ok(a.x, sizeof(T), a.W) &&
+  if (plane_tma_ok(a.x, sizeof(T), a.W) &&
       make_plane_map(&tm, a.x, sizeof(T), a.W, a.H, a.N * a.C, Geo<K, sizeof(T)>::SP,
-                     SepShape<K, T, true>::ROWS))
-    return sep_run<T, K, true>(a, tm, wcol, wrow, st);
-  return sep_run<T, K, false>(a, tm, wcol, wrow, st);
+                     SepShape<K, T, kAligned>::ROWS))
+    return a.vec ? sep_run<T, K, kAligned>(a, tm, wcol, wrow, st)
+                 : sep_run<T, K, kTmaLoads>(a, tm, wcol, wrow, st);
+  return sep_run<T, K, kAnyPlanes>(a, tm, wcol, wrow, st);
 }
 
 template <int K>

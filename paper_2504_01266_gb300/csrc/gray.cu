@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(256) gray_kernel(const T* __restrict__ x, T* _
 // slices -- one TMA load with a box three planes deep, or cp.async -- then
 // every staged cell becomes its gray value (FP32: in place over the red
 // slice; BF16: into a separate FP32 tile in the compute geometry).
-template <int K, typename T, bool AL>
+template <int K, typename T, int AL>
 struct GrayShape {
   using G = GeoC<K, T, !AL>;
   using GS = Geo<K, sizeof(T), !AL>;
@@ -68,7 +68,7 @@ struct GrayShape {
                 "row buffers fit the dead slices");
 };
 
-template <typename T, int K, bool AL>
+template <typename T, int K, int AL>
 __global__ void __launch_bounds__(kThreads) gray_fwd_kernel(
     const __grid_constant__ CUtensorMap tmx, const T* __restrict__ x, const float* __restrict__ w,
     T* __restrict__ y, int H, int W, FastDiv ftx, FastDiv fty, int clamp, int vec, int odd_rows,
@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(kThreads) gray_fwd_kernel(
     mbar_init_fence();
   }
   cta_barrier();
-  if constexpr (AL) {
+  if constexpr (AL != kAnyPlanes) {
     cp_async_commit();
     if (threadIdx.x == 0) {
       fence_proxy_async();
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kThreads) gray_fwd_kernel(
                            reinterpret_cast<float*>(sm + S::ROW_BUFS + warp * kRowBuf), acc);
 }
 
-template <typename T, int K, bool AL>
+template <typename T, int K, int AL>
 static cudaError_t gray_fwd_run(const GrayArgs& a, const CUtensorMap& tm, cudaStream_t st) {
   using S = GrayShape<K, T, AL>;
   cudaError_t e = set_smem_once<gray_fwd_kernel<T, K, AL>>((size_t)S::SM_BYTES);
@@ -175,10 +175,10 @@ static cudaError_t gray_fwd_run(const GrayArgs& a, const CUtensorMap& tm, cudaSt
 
 template <typename T, int K>
 static cudaError_t gray_fwd_impl(const GrayArgs& a, cudaStream_t st) {
-  using S = GrayShape<K, T, true>;
+  using S = GrayShape<K, T, kAligned>;
   CUtensorMap tm;
   std::memset(&tm, 0, sizeof(tm));
-  if (a.vec && plane_tma_ok(a.x, sizeof(T), a.W)) {
+  if (plane_tma_ok(a.x, sizeof(T), a.W)) {
     // the box is three planes deep: the R, G and B tiles of one image in one load
     EncodeFn enc = encode_fn();
     if (enc) {
@@ -191,10 +191,11 @@ static cudaError_t gray_fwd_impl(const GrayArgs& a, cudaStream_t st) {
               const_cast<void*>(a.x), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
               CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
-        return gray_fwd_run<T, K, true>(a, tm, st);
+        return a.vec ? gray_fwd_run<T, K, kAligned>(a, tm, st)
+                     : gray_fwd_run<T, K, kTmaLoads>(a, tm, st);
     }
   }
-  return gray_fwd_run<T, K, false>(a, tm, st);
+  return gray_fwd_run<T, K, kAnyPlanes>(a, tm, st);
 }
 
 template <typename T>

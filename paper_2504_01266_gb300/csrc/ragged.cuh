@@ -262,7 +262,7 @@ __device__ __forceinline__ int rag_chunk(const RagParams& p, const RagChunk& ch,
       T* dst = warp < 8 ? yp : dxp;
       float o[8][4];
       fwd_block<K, 8, T, true>(src + r8 * G::SP + 4 * lane, f, o);
-      store_tile<T, 8, false>(dst, H, W, ty0 + r8, tx0, vec,
+      store_tile<T, 8, kAnyPlanes>(dst, H, W, ty0 + r8, tx0, vec,
                               reinterpret_cast<float*>(sm + L::BUF + warp * kRowBuf), o);
     }
     if (do_dw) {

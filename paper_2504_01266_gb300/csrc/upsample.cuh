@@ -197,7 +197,7 @@ __device__ __forceinline__ void up_tile(float* __restrict__ sx, int zero_off,
   fwd_block_tab<K, PY>(sx + 4 * lane, rowoff + warp * PY, sw, acc);
   // the staged pixels are dead: their space serves as the warps' row buffers
   static_assert(U::SRC_ROWS * U::SRC_COLS * 4 >= kWarps * kRowBuf, "row buffers fit");
-  store_tile<T, PY, false>(yplane, Ho, Wo, ty0 + warp * PY, tx0, vec, ss + warp * kTileW, acc);
+  store_tile<T, PY, kAnyPlanes>(yplane, Ho, Wo, ty0 + warp * PY, tx0, vec, ss + warp * kTileW, acc);
   cta_barrier();  // the expanded rows, tables and the staged pixels are free again
 }
 
