@@ -134,8 +134,16 @@ DwConfig tune_config(int op, int id, const DwArgs& a) {
   return c;
 }
 
+// Inputs that TMA can load: rows and bases on 16-byte boundaries (BF16 bases 8
+// bytes off one still allow 8-byte accesses, DwArgs::vec, but not TMA).  Without
+// pointers, as in a query, the row length decides.
+static bool inputs_aligned(const DwArgs& a) {
+  return a.W * (a.dtype == 0 ? 4 : 2) % 16 == 0 && reinterpret_cast<uintptr_t>(a.x) % 16 == 0 &&
+         reinterpret_cast<uintptr_t>(a.dy) % 16 == 0;
+}
+
 // Without a stored choice the configuration follows from the filter size, the
-// storage type, the planes' alignment and the number T of 64 x 128 tiles
+// storage type, the inputs' alignment and the number T of 64 x 128 tiles
 // against the S SMs (S = 152; times in us, candidate 0 -> the choice):
 //  * forward and input gradient, T <= 2 S: 32-row tiles, because 64-row tiles
 //    leave SMs with no CTA or one (512^2 K = 21: 24 -> 15, K = 31: 46 -> 26;
@@ -153,7 +161,8 @@ DwConfig tune_config(int op, int id, const DwArgs& a) {
 //    K <= 3, aligned planes: the tile ring from T = 16 S (FP32; 8 x 3 x 2048^2
 //    218 -> 189, at T = 10 S 38.8 -> 40.7) or 4 S (BF16; 378 -> 261, at 5 S 25.7
 //    -> 21.2); its one CTA per SM stages unaligned planes with the warps that
-//    compute (160 -> 207).
+//    compute (160 -> 207), and its four dx warps store rows at any alignment slowly
+//    (BF16 4 x 3 x 1801 x 2400, aligned inputs only: 143 -> 194).
 //    Two passes: K >= 13 from T = 2 S (3 x 1080 x 1920 K = 13: 117 -> 106, 4 x 3
 //    x 1801 x 2400: 997 -> 636; K = 15: 860 -> 803); K = 11 from 4 S aligned (86
 //    -> 81), 16 S not (584 -> 572; at 5 S 91 -> 93); K = 9 aligned from 4 S (BF16
@@ -165,7 +174,7 @@ DwConfig default_config(int op, const DwArgs& a) {
   const int64_t S = sm_count();
   const int64_t T = a.N * a.C * ((a.W + kTileW - 1) / kTileW) * ((a.H + 63) / 64);
   const bool f32 = a.dtype == 0;
-  const bool aligned = a.vec && a.W % (f32 ? 4 : 8) == 0;
+  const bool aligned = inputs_aligned(a);
   switch (op) {
     case TUNE_FWD:
     case TUNE_BWD_INPUT:
@@ -176,7 +185,7 @@ DwConfig default_config(int op, const DwArgs& a) {
       break;
     case TUNE_BWD_FUSED: {
       const bool pairs = f32 && a.K <= 3 && T >= (a.K == 1 ? 80 : 100) * S;
-      const bool ring = !pairs && a.K <= 3 && aligned && T >= (f32 ? 16 : 4) * S;
+      const bool ring = !pairs && a.K <= 3 && aligned && a.vec && T >= (f32 ? 16 : 4) * S;
       int64_t from = -1;  // two passes from this many tiles per SM on
       if (a.K >= 13)
         from = 2;
