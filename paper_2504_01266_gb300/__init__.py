@@ -51,13 +51,14 @@ def _require_cuda(*ts):
 
 # The current stream of a device as an integer: the handle alone, without the
 # Stream object that torch.cuda.current_stream builds (2.0 us a call on the
-# Grace host against 0.1 us).
-_raw_stream = torch._C._cuda_getCurrentRawStream
+# Grace host against 0.1 us).  A private name: None where torch has none (a build
+# without CUDA), and the Stream object serves.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream(device) -> int:
     index = device.index
-    if index is None:
+    if index is None or _raw_stream is None:
         return torch.cuda.current_stream(device).cuda_stream
     return _raw_stream(index)
 
