@@ -335,6 +335,8 @@ giga_status_t giga_gray_conv2d_fwd(const giga_conv2d_desc_t* desc, const void* x
  *   2 full:   like cached, and the entry points benchmark the candidates the
  *             first time they meet an uncached problem class (not while the
  *             stream is capturing).
+ * A problem class is the op, type, K, border, size (log2 of N*C*H*W) and whether
+ * the planes are aligned (rows and bases on 16-byte boundaries).
  * The cache is kept in memory and, if GIGA_AUTOTUNE_CACHE names a file,
  * loaded from / saved to it as JSON.  A corrupt cache file is ignored.  With
  * GIGA_LOG set (to anything but "0") every tuning decision, including the
@@ -346,11 +348,12 @@ int32_t giga_autotune_get_mode(void);
 giga_status_t giga_autotune_conv2d(const giga_conv2d_desc_t* desc, int32_t ops, const void* x,
                                    const void* w, void* y, const void* dy, void* dx, float* dw,
                                    void* ws, size_t ws_bytes, void* stream);
-/* The configuration id stored for (desc, op), which the entry points will use;
- * 0 if there is none (the built-in rule then decides); -1 on error. */
+/* The configuration id stored for (desc, op) and tensors on 16-byte boundaries,
+ * which the entry points will use; 0 if there is none (the built-in rule then
+ * decides); -1 on error. */
 int32_t giga_autotune_choice(const giga_conv2d_desc_t* desc, int32_t op);
 /* Pin configuration `id` for (desc's problem class, op) in the cache, as if
- * the tuner had chosen it; used in modes 1 and 2.  GIGA_ERR_INVALID_ARG for
+ * the tuner had chosen it for planes of either alignment; used in modes 1 and 2.  GIGA_ERR_INVALID_ARG for
  * an unknown op or an id outside the op's candidates. */
 giga_status_t giga_autotune_set_choice(const giga_conv2d_desc_t* desc, int32_t op, int32_t id);
 giga_status_t giga_autotune_save(const char* path);

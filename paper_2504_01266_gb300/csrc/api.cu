@@ -593,11 +593,19 @@ giga_status_t giga_autotune_conv2d(const giga_conv2d_desc_t* desc, int32_t ops, 
   DwArgs a = make_args(desc);
   a.x = x; a.y = y; a.dy = dy; a.dx = dx; a.w = static_cast<const float*>(w); a.dw = dw;
   a.partials = static_cast<float*>(ws);
-  a.vec = vec_ok(a, x, y, nullptr) && vec_ok(a, dy, dx, nullptr);
-  if ((ops & GIGA_OP_FWD) && (s = tune_dw_op(TUNE_FWD, a, st))) return s;
-  if (fused) return tune_dw_op(TUNE_BWD_FUSED, a, st);
-  if ((ops & GIGA_OP_BWD_INPUT) && (s = tune_dw_op(TUNE_BWD_INPUT, a, st))) return s;
-  if ((ops & GIGA_OP_BWD_FILTER) && (s = tune_dw_op(TUNE_BWD_FILTER, a, st))) return s;
+  // each op with the tensors it takes, as its entry point would: their alignment
+  // is part of the problem class
+  auto tune = [&](int op, const void* in_x, const void* in_dy, const void* out) {
+    DwArgs b = a;
+    b.x = in_x;
+    b.dy = in_dy;
+    b.vec = vec_ok(b, in_x, in_dy, out);
+    return tune_dw_op(op, b, st);
+  };
+  if ((ops & GIGA_OP_FWD) && (s = tune(TUNE_FWD, x, nullptr, y))) return s;
+  if (fused) return tune(TUNE_BWD_FUSED, x, dy, dx);
+  if ((ops & GIGA_OP_BWD_INPUT) && (s = tune(TUNE_BWD_INPUT, nullptr, dy, dx))) return s;
+  if ((ops & GIGA_OP_BWD_FILTER) && (s = tune(TUNE_BWD_FILTER, x, dy, nullptr))) return s;
   return GIGA_OK;
 }
 
@@ -607,7 +615,9 @@ int32_t giga_autotune_choice(const giga_conv2d_desc_t* desc, int32_t op) {
   const int top = tune_op_of(op);
   if (top < 0) return -1;
   if (tune_mode() == 0) return 0;
-  const int id = tune_lookup(top, make_args(desc));
+  DwArgs a = make_args(desc);
+  a.vec = desc->W % 4 == 0;  // as for tensors on 16-byte boundaries
+  const int id = tune_lookup(top, a);
   return id < 0 ? 0 : id;
 }
 
@@ -620,7 +630,7 @@ giga_status_t giga_autotune_set_choice(const giga_conv2d_desc_t* desc, int32_t o
   if (top < 0) return fail(GIGA_ERR_INVALID_ARG, "op must be 1, 2, 4 or 6");
   if (id < 0 || id >= tune_candidates(top))
     return fail(GIGA_ERR_INVALID_ARG, "configuration id " + std::to_string(id) + " out of range");
-  tune_store(top, make_args(desc), id);
+  tune_store(top, make_args(desc), id, true);
   return GIGA_OK;
 }
 

@@ -9,7 +9,9 @@
 //                             without an L2 prefetch of a later tile;
 //   filter gradient (alone or fused): tiles per CTA = automatic, 2, 4, 8, 16
 //                             (fewer partial sums vs. better load balance).
-// Problem class: (op, dtype, K, border, floor(log2(N*C*H*W))).
+// Problem class: (op, dtype, K, border, floor(log2(N*C*H*W)), planes aligned or
+// not -- they run separately compiled kernels).  A choice pinned for a
+// description, or in a cache without the alignment, holds for both.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -207,12 +209,27 @@ DwConfig default_config(int op, const DwArgs& a) {
   return c;
 }
 
-static std::string key_of(int op, const DwArgs& a) {
+static bool planes_aligned(const DwArgs& a) { return a.vec && inputs_aligned(a); }
+
+// Key without the alignment, and with it.
+static std::string pin_key(int op, const DwArgs& a) {
   const double n = (double)a.N * a.C * a.H * a.W;
   const int sc = n > 0 ? (int)std::floor(std::log2(n)) : 0;
   char buf[96];
   std::snprintf(buf, sizeof(buf), "%d:%d:%d:%d:%d", op, a.dtype, a.K, a.border, sc);
   return buf;
+}
+static std::string key_of(int op, const DwArgs& a) {
+  return pin_key(op, a) + (planes_aligned(a) ? ":0" : ":1");
+}
+
+// A choice for a key without the alignment replaces those of both alignments.
+static void put_choice(const std::string& key, int id) {
+  if (std::count(key.begin(), key.end(), ':') == 4) {
+    g_cache.erase(key + ":0");
+    g_cache.erase(key + ":1");
+  }
+  g_cache[key] = id;
 }
 
 // ---- JSON persistence: {"giga_autotune": 1, "entries": {"key": id, ...}}
@@ -252,7 +269,7 @@ static bool load_file(const char* path) {
   ss << f.rdbuf();
   std::map<std::string, int> m;
   if (!parse_cache(ss.str(), m)) return false;  // a corrupt cache is ignored
-  for (auto& kv : m) g_cache[kv.first] = kv.second;
+  for (auto& kv : m) put_choice(kv.first, kv.second);  // in order: a key before its longer ones
   return true;
 }
 
@@ -283,14 +300,15 @@ int tune_lookup(int op, const DwArgs& a) {
   ensure_loaded();
   if (g_cache.empty()) return -1;
   auto it = g_cache.find(key_of(op, a));
+  if (it == g_cache.end()) it = g_cache.find(pin_key(op, a));
   if (it == g_cache.end()) return -1;
   return it->second < tune_candidates(op) ? it->second : -1;
 }
 
-void tune_store(int op, const DwArgs& a, int id) {
+void tune_store(int op, const DwArgs& a, int id, bool pin) {
   std::lock_guard<std::mutex> lk(g_mu);
   ensure_loaded();
-  g_cache[key_of(op, a)] = id;
+  put_choice(pin ? pin_key(op, a) : key_of(op, a), id);
   if (const char* p = std::getenv("GIGA_AUTOTUNE_CACHE")) save_file(p);
 }
 
@@ -346,7 +364,7 @@ giga_status_t tune_dw_op(int op, const DwArgs& a, cudaStream_t st) {
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (status == GIGA_OK) {
-    tune_store(op, a, best);
+    tune_store(op, a, best, false);
     if (tune_log_enabled())
       std::fprintf(stderr,
                    "giga autotune: %s %s K=%d %s N*C*H*W=%lld (class %s) -> candidate %d "

@@ -24,7 +24,8 @@ DwConfig tune_config(int op, int id, const DwArgs& a);
 DwConfig default_config(int op, const DwArgs& a);
 // Cached choice for (op, problem class); -1 if none.
 int tune_lookup(int op, const DwArgs& a);
-void tune_store(int op, const DwArgs& a, int id);
+// pin: for planes of any alignment, else for those of `a`.
+void tune_store(int op, const DwArgs& a, int id, bool pin);
 // Run one depthwise op with candidate `id` (used by the autotuner).
 giga_status_t run_dw_op(int op, const DwArgs& a, const DwConfig& cfg, cudaStream_t st);
 // Benchmark all candidates of `op` on these buffers and store the fastest.
