@@ -352,6 +352,10 @@ giga_status_t giga_autotune_conv2d(const giga_conv2d_desc_t* desc, int32_t ops, 
  * which the entry points will use; 0 if there is none (the built-in rule then
  * decides); -1 on error. */
 int32_t giga_autotune_choice(const giga_conv2d_desc_t* desc, int32_t op);
+/* The configuration id that the entry points use for (desc, op), tensors on
+ * 16-byte boundaries and the present mode: the stored one, else the built-in
+ * rule's (pinning it changes nothing); -1 on error. */
+int32_t giga_autotune_effective_choice(const giga_conv2d_desc_t* desc, int32_t op);
 /* Pin configuration `id` for (desc's problem class, op) in the cache, as if
  * the tuner had chosen it for planes of either alignment; used in modes 1 and 2.  GIGA_ERR_INVALID_ARG for
  * an unknown op or an id outside the op's candidates. */

@@ -609,16 +609,25 @@ giga_status_t giga_autotune_conv2d(const giga_conv2d_desc_t* desc, int32_t ops, 
   return GIGA_OK;
 }
 
-int32_t giga_autotune_choice(const giga_conv2d_desc_t* desc, int32_t op) {
+// The stored choice for (desc, op) and tensors on 16-byte boundaries, else the
+// built-in rule's (rule) or 0; -1 on error.
+static int32_t choice_of(const giga_conv2d_desc_t* desc, int32_t op, bool rule) {
   clear_error();
   if (check_desc(desc) != GIGA_OK || !is_depthwise(desc)) return -1;
   const int top = tune_op_of(op);
   if (top < 0) return -1;
-  if (tune_mode() == 0) return 0;
   DwArgs a = make_args(desc);
-  a.vec = desc->W % 4 == 0;  // as for tensors on 16-byte boundaries
-  const int id = tune_lookup(top, a);
-  return id < 0 ? 0 : id;
+  a.vec = desc->W % 4 == 0;
+  const int id = tune_mode() == 0 ? -1 : tune_lookup(top, a);
+  return id >= 0 ? id : (rule ? default_choice(top, a) : 0);
+}
+
+int32_t giga_autotune_choice(const giga_conv2d_desc_t* desc, int32_t op) {
+  return choice_of(desc, op, false);
+}
+
+int32_t giga_autotune_effective_choice(const giga_conv2d_desc_t* desc, int32_t op) {
+  return choice_of(desc, op, true);
 }
 
 giga_status_t giga_autotune_set_choice(const giga_conv2d_desc_t* desc, int32_t op, int32_t id) {

@@ -144,6 +144,10 @@ static bool inputs_aligned(const DwArgs& a) {
          reinterpret_cast<uintptr_t>(a.dy) % 16 == 0;
 }
 
+// Candidates that the built-in rule takes beside 0 (tune_config).
+constexpr int kTileRows32 = 1, kPrefetch = 4;            // forward, input gradient
+constexpr int kTilePairs = 1, kTwoPasses = 5, kRing = 6;  // both gradients
+
 // Without a stored choice the configuration follows from the filter size, the
 // storage type, the inputs' alignment and the number T of 64 x 128 tiles
 // against the S SMs (S = 152; times in us, candidate 0 -> the choice):
@@ -171,42 +175,34 @@ static bool inputs_aligned(const DwArgs& a) {
 //    67 -> 64, FP32 equal; 4 x 3 x 1024^2 111 -> 103); BF16 K = 7 from 8 S aligned
 //    (75.7 -> 73.3; 16 x 3 x 2048^2 923 -> 807; at 5 S equal), 16 S not (425 ->
 //    402); BF16 K = 5 aligned from 8 S (55 -> 51; at 5 S 34 -> 36).
-DwConfig default_config(int op, const DwArgs& a) {
-  DwConfig c = tune_config(op, 0, a);
+int default_choice(int op, const DwArgs& a) {
   const int64_t S = sm_count();
   const int64_t T = a.N * a.C * ((a.W + kTileW - 1) / kTileW) * ((a.H + 63) / 64);
   const bool f32 = a.dtype == 0;
   const bool aligned = inputs_aligned(a);
-  switch (op) {
-    case TUNE_FWD:
-    case TUNE_BWD_INPUT:
-      if (T <= 2 * S)
-        c.rows_per_thread = 4;
-      else
-        c.prefetch = aligned && (f32 ? a.K == 7 || a.K == 9 : a.K <= 3);
-      break;
-    case TUNE_BWD_FUSED: {
-      const bool pairs = f32 && a.K <= 3 && T >= (a.K == 1 ? 80 : 100) * S;
-      const bool ring = !pairs && a.K <= 3 && aligned && a.vec && T >= (f32 ? 16 : 4) * S;
-      int64_t from = -1;  // two passes from this many tiles per SM on
-      if (a.K >= 13)
-        from = 2;
-      else if (a.K == 11)
-        from = aligned ? 4 : 16;
-      else if (a.K == 9 && aligned)
-        from = 4;
-      else if (a.K == 7 && !f32)
-        from = aligned ? 8 : 16;
-      else if (a.K == 5 && !f32 && aligned)
-        from = 8;
-      const bool split = from >= 0 && T >= from * S;
-      if (ring || split || pairs) c = tune_config(op, split ? 5 : (ring ? 6 : 1), a);
-      break;
-    }
-    default:
-      break;
+  if (op == TUNE_FWD || op == TUNE_BWD_INPUT) {
+    if (T <= 2 * S) return kTileRows32;
+    return aligned && (f32 ? a.K == 7 || a.K == 9 : a.K <= 3) ? kPrefetch : 0;
   }
-  return c;
+  if (op != TUNE_BWD_FUSED) return 0;
+  if (f32 && a.K <= 3 && T >= (a.K == 1 ? 80 : 100) * S) return kTilePairs;
+  if (a.K <= 3 && aligned && a.vec && T >= (f32 ? 16 : 4) * S) return kRing;
+  int64_t from = -1;  // two passes from this many tiles per SM on
+  if (a.K >= 13)
+    from = 2;
+  else if (a.K == 11)
+    from = aligned ? 4 : 16;
+  else if (a.K == 9 && aligned)
+    from = 4;
+  else if (a.K == 7 && !f32)
+    from = aligned ? 8 : 16;
+  else if (a.K == 5 && !f32 && aligned)
+    from = 8;
+  return from >= 0 && T >= from * S ? kTwoPasses : 0;
+}
+
+DwConfig default_config(int op, const DwArgs& a) {
+  return tune_config(op, default_choice(op, a), a);
 }
 
 static bool planes_aligned(const DwArgs& a) { return a.vec && inputs_aligned(a); }

@@ -20,7 +20,8 @@ enum TuneOp { TUNE_FWD = 0, TUNE_BWD_INPUT = 1, TUNE_BWD_FILTER = 2, TUNE_BWD_FU
 int tune_mode();
 int tune_candidates(int op);
 DwConfig tune_config(int op, int id, const DwArgs& a);
-// Configuration of a call for which no choice is stored.
+// Candidate and configuration of a call for which no choice is stored.
+int default_choice(int op, const DwArgs& a);
 DwConfig default_config(int op, const DwArgs& a);
 // Cached choice for (op, problem class); -1 if none.
 int tune_lookup(int op, const DwArgs& a);
