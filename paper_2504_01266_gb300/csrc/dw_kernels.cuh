@@ -1251,14 +1251,15 @@ static_assert(kFilterTileH == kBwdTileH, "both filter-gradient kernels share the
 // warps in 3 groups (up to 168 registers): K = 9 with 8-row blocks 658 -> 638 /
 // 701 -> 664, K = 11 948 -> 935 / 1013 -> 1009, K = 13 1235 -> 1240 / 1488 ->
 // 1379 against 16 warps; 8-row blocks lose at K >= 11 (K = 11 1077, K = 15
-// 1536 -> 1737).
-template <int K>
+// 1536 -> 1737).  WIDE: 16 warps of 4-row blocks, for the BF16 planes that
+// dw_launch_impl.cuh picks (filter_wide).
+template <int K, bool WIDE>
 constexpr int filter_warps() {
-  return K <= 7 ? 8 : 12;
+  return WIDE ? 16 : (K <= 7 ? 8 : 12);
 }
-template <int K>
+template <int K, bool WIDE>
 constexpr int filter_groups() {
-  return K <= 7 ? 1 : 3;
+  return WIDE ? dw_groups<K>() : (K <= 7 ? 1 : 3);
 }
 
 // Accumulators per tap and lane: two where fewer warps leave a lane twice the
@@ -1267,23 +1268,23 @@ constexpr int filter_groups() {
 // error against FP64 was 1.3 times that of 16 warps; the second costs registers
 // that are free but at BF16 K = 7, where two CTAs per SM become one (16 x 3 x
 // 2048^2 411 -> 448 us, W = 2399 227 -> 293).
-template <int K>
+template <int K, bool WIDE>
 constexpr int filter_sets() {
-  return K <= 7 || K == 11 ? 2 : 1;
+  return !WIDE && (K <= 7 || K == 11) ? 2 : 1;
 }
 
-template <int K, typename T, int AL>
+template <int K, typename T, int AL, bool WIDE>
 struct FilterShape {
   using G = Geo<K, sizeof(T), !AL>;  // tiles stay in the storage type (no widening pass)
   static constexpr int DYP = geo_pitch(1, sizeof(T), !AL);  // dy tile pitch (no halo)
-  static constexpr int NW = filter_warps<K>();
+  static constexpr int NW = filter_warps<K, WIDE>();
   static constexpr int NT = NW * 32;
-  static constexpr int GT = filter_groups<K>();
+  static constexpr int GT = filter_groups<K, WIDE>();
   static constexpr int WPG = NW / GT;
   static constexpr int AT = (K + GT - 1) / GT;
   static constexpr int ROWS = kFilterTileH / WPG;  // tile rows per warp
-  static constexpr int DR = K <= 9 ? 8 : 4;        // dy rows per unrolled block
-  static constexpr int SETS = filter_sets<K>();
+  static constexpr int DR = K <= 9 && !WIDE ? 8 : 4;  // dy rows per unrolled block
+  static constexpr int SETS = filter_sets<K, WIDE>();
   static constexpr int X_ROWS = kFilterTileH + 2 * G::R;
   static constexpr int X_BYTES = X_ROWS * G::SP * (int)sizeof(T);
   static constexpr int DY_BYTES = kFilterTileH * DYP * (int)sizeof(T);
@@ -1297,14 +1298,14 @@ struct FilterShape {
   static_assert(SM_BYTES <= 227 * 1024, "shared memory");
 };
 
-template <typename T, int K, int AL>
-__global__ void __launch_bounds__(FilterShape<K, T, AL>::NT, 1)
+template <typename T, int K, int AL, bool WIDE>
+__global__ void __launch_bounds__(FilterShape<K, T, AL, WIDE>::NT, 1)
     dw_filter_kernel(const __grid_constant__ CUtensorMap tmx,
                      const __grid_constant__ CUtensorMap tmdy, const T* __restrict__ x,
                      const T* __restrict__ dy, float* __restrict__ partials, int H, int W,
                      FastDiv ftx, int tiles_per_plane, FastDiv fcpp, int tpc, int num_chunks,
                      int clamp, int odd_rows, int* err) {
-  using S = FilterShape<K, T, AL>;
+  using S = FilterShape<K, T, AL, WIDE>;
   using G = typename S::G;
   extern __shared__ __align__(128) float smem[];
   char* sm = reinterpret_cast<char*>(smem);

@@ -211,13 +211,13 @@ cudaError_t dw_bwd_ring_launch(const DwArgs& a, const DwConfig& cfg, cudaStream_
   }
 }
 
-template <typename T, int K, int AL>
+template <typename T, int K, int AL, bool WIDE>
 static cudaError_t filter_run(const DwArgs& a, const CUtensorMap& tmx, const CUtensorMap& tmdy,
                               const DwConfig& cfg, cudaStream_t st) {
-  using S = FilterShape<K, T, AL>;
+  using S = FilterShape<K, T, AL, WIDE>;
   const size_t smem = (size_t)S::SM_BYTES;
-  auto kern = dw_filter_kernel<T, K, AL>;
-  cudaError_t e = set_smem_once<dw_filter_kernel<T, K, AL>>(smem);
+  auto kern = dw_filter_kernel<T, K, AL, WIDE>;
+  cudaError_t e = set_smem_once<dw_filter_kernel<T, K, AL, WIDE>>(smem);
   if (e != cudaSuccess) return e;
   static int ctas_per_sm[64] = {};
   int dev = 0;
@@ -248,12 +248,31 @@ static cudaError_t filter_run(const DwArgs& a, const CUtensorMap& tmx, const CUt
   return cudaGetLastError();
 }
 
+// BF16 planes that TMA cannot load, where 16 warps beat 8 or 12: staging them
+// takes the warps longer than a small filter does (K = 1; K = 3, 5 with rows to be
+// shifted and few tiles: from about 5 S on, and for planes of one tile, the
+// 16 warps' 4-row blocks cost more than they save), at K = 7 the two accumulators
+// leave 8 warps per SM, and at K = 13 they are a little better.  16 warps against
+// 8 / 12 (us): 3 x 3 x 257 x 251 K = 1 7.6 / 10.1, K = 3 8.3 / 9.9, K = 5 10.4 / 12.2,
+// K = 7 11.8 / 12.8; 8 x 3 x 1024 x 1021 K = 3 1.17 times as long; 4 x 3 x 1801 x
+// 2399 K = 1 0.89, K = 7 0.84, K = 13 0.93 times.
+template <int K>
+static bool filter_wide(const DwArgs& a) {
+  if (K == 1 || K == 7 || K == 13) return true;
+  const int64_t tpp = ((a.W + kTileW - 1) / kTileW) * ((a.H + kFilterTileH - 1) / kFilterTileH);
+  return has_odd_rows(2, a.W, a.x, a.dy) && tpp > 1 &&
+         a.N * a.C * tpp <= 4 * (int64_t)sm_count();
+}
+
 template <typename T, int K>
 static cudaError_t filter_impl(const DwArgs& a, const DwConfig& cfg, cudaStream_t st) {
   CUtensorMap tmx, tmdy;
-  return xdy_maps<T, K>(a, FilterShape<K, T, kAligned>::X_ROWS, kFilterTileH, kTileW, &tmx, &tmdy)
-             ? filter_run<T, K, kAligned>(a, tmx, tmdy, cfg, st)
-             : filter_run<T, K, kAnyPlanes>(a, tmx, tmdy, cfg, st);
+  if (xdy_maps<T, K>(a, FilterShape<K, T, kAligned, false>::X_ROWS, kFilterTileH, kTileW, &tmx,
+                     &tmdy))
+    return filter_run<T, K, kAligned, false>(a, tmx, tmdy, cfg, st);
+  if constexpr (sizeof(T) == 2 && (K <= 7 || K == 13))
+    if (filter_wide<K>(a)) return filter_run<T, K, kAnyPlanes, true>(a, tmx, tmdy, cfg, st);
+  return filter_run<T, K, kAnyPlanes, false>(a, tmx, tmdy, cfg, st);
 }
 
 template <int K>
