@@ -160,25 +160,31 @@ constexpr int kTilePairs = 1, kTwoPasses = 5, kRing = 6;  // both gradients
 //  * both gradients, fused kernel -> the choice:
 //    FP32 K <= 3, very many tiles: the fused kernel with two tiles per CTA, whose
 //    three CTAs per SM keep HBM busier than the ring's one, and whose CTAs work
-//    on nearer tiles than with the usual 8 or 16 each: K = 3 from T = 100 S (ring ->
-//    pairs: 8 x 3 x 2048^2, 81 S, 189 -> 201; 12 x 3 x 2048^2 307 -> 290; 8 x 3 x
-//    4096^2 793 -> 738; unaligned 16 x 3 x 2048 x 2047 598 -> 556), K = 1 from 80 S
-//    (208 -> 181).
-//    K <= 3, aligned planes: the tile ring from T = 16 S (FP32; 8 x 3 x 2048^2
-//    218 -> 189, at T = 10 S 38.8 -> 40.7) or 4 S (BF16; 378 -> 261, at 5 S 25.7
-//    -> 21.2); its one CTA per SM stages unaligned planes with the warps that
-//    compute (160 -> 207), and its four dx warps store rows at any alignment slowly
-//    (BF16 4 x 3 x 1801 x 2400, aligned inputs only: 143 -> 194).
-//    Two passes: K >= 13 from T = 2 S (3 x 1080 x 1920 K = 13: 117 -> 106, 4 x 3
-//    x 1801 x 2400: 997 -> 636; K = 15: 860 -> 803); K = 11 from 4 S aligned (86
-//    -> 81), 16 S not (584 -> 572; at 5 S 91 -> 93); K = 9 aligned from 4 S (BF16
-//    67 -> 64, FP32 equal; 4 x 3 x 1024^2 111 -> 103); BF16 K = 7 from 8 S aligned
-//    (75.7 -> 73.3; 16 x 3 x 2048^2 923 -> 807; at 5 S equal), 16 S not (425 ->
-//    402); BF16 K = 5 aligned from 8 S (55 -> 51; at 5 S 34 -> 36).
+//    on nearer tiles than with the usual 8 or 16 each: K = 3 from T = 100 S (12 x 3 x
+//    2048^2, ring -> pairs 297 -> 289; 8 x 3 x 4096^2 793 -> 738; unaligned 16 x 3 x
+//    2048 x 2047, fused -> pairs 598 -> 556), K = 1 from 80 S (183 -> 179).
+//    K <= 3, aligned planes: the tile ring, FP32 K = 3 from 32 S (4 x 3 x 1801 x 2400
+//    111 -> 104; at 20 S 59.6 -> 60.8) unless a plane is one tile (32 x 128 x 56 x 56
+//    59 -> 75: every chunk one tile, one reduction); BF16 from 4 S (8 x 3 x 1024^2
+//    K = 1 41 -> 31). FP32 K = 1 loses (97 -> 110). Its one CTA per SM stages
+//    unaligned planes with the warps that compute (160 -> 207), and its four dx
+//    warps store rows at any alignment slowly (BF16 4 x 3 x 1801 x 2400, aligned
+//    inputs only: 143 -> 194).
+//    Two passes (planes 4 x 3 x 1801 x 2400 or 2399 unless stated).  FP32: K >= 13 from
+//    4 S (3 x 1080 x 1920 K = 13 102 -> 97; 716 -> 638; K = 15 864 -> 796) but K = 15 on
+//    planes of one tile (8 x 192 x 28 x 28 217 -> 226); K = 11 aligned from 4 S (86 ->
+//    81, 556 -> 476), unaligned from 32 S (600 -> 575; at 20 S 291 -> 300) but planes
+//    of one tile (8 x 512 x 7 x 7 346 -> 366); K = 9 aligned from 4 S (4 x 3 x 1024^2
+//    111 -> 103).  BF16: K = 15, and K = 11, 13 aligned, from 32 S (904 -> 844, 540 ->
+//    512, 721 -> 691; at 20 S equal; K = 11 unaligned 684 -> 708) but planes of one
+//    tile (32 x 128 x 56 x 56 K = 13 433 -> 473); K = 9 aligned from 4 S (67 -> 64);
+//    K = 7 aligned from 8 S (73 -> 67; 16 x 3 x 2048^2 947 -> 837) but planes of one tile
+//    (174 -> 181); K = 5 aligned from 5 S (28.5 -> 26.0).
 int default_choice(int op, const DwArgs& a) {
   const int64_t S = sm_count();
-  const int64_t T = a.N * a.C * ((a.W + kTileW - 1) / kTileW) * ((a.H + 63) / 64);
-  const bool f32 = a.dtype == 0;
+  const int64_t tpp = ((a.W + kTileW - 1) / kTileW) * ((a.H + 63) / 64);
+  const int64_t T = a.N * a.C * tpp;
+  const bool f32 = a.dtype == 0, many = tpp > 1;  // many: a plane is more than one tile
   const bool aligned = inputs_aligned(a);
   if (op == TUNE_FWD || op == TUNE_BWD_INPUT) {
     if (T <= 2 * S) return kTileRows32;
@@ -186,18 +192,19 @@ int default_choice(int op, const DwArgs& a) {
   }
   if (op != TUNE_BWD_FUSED) return 0;
   if (f32 && a.K <= 3 && T >= (a.K == 1 ? 80 : 100) * S) return kTilePairs;
-  if (a.K <= 3 && aligned && a.vec && T >= (f32 ? 16 : 4) * S) return kRing;
+  if (a.K <= 3 && aligned && a.vec && (f32 ? a.K == 3 && many && T >= 32 * S : T >= 4 * S))
+    return kRing;
   int64_t from = -1;  // two passes from this many tiles per SM on
-  if (a.K >= 13)
-    from = 2;
-  else if (a.K == 11)
-    from = aligned ? 4 : 16;
+  if (f32 && (a.K == 13 || (a.K == 15 && many) || (a.K == 11 && aligned)))
+    from = 4;
+  else if (a.K >= 11 && many && (aligned || f32 || a.K == 15))
+    from = 32;
   else if (a.K == 9 && aligned)
     from = 4;
-  else if (a.K == 7 && !f32)
-    from = aligned ? 8 : 16;
-  else if (a.K == 5 && !f32 && aligned)
+  else if (a.K == 7 && !f32 && aligned && many)
     from = 8;
+  else if (a.K == 5 && !f32 && aligned)
+    from = 5;
   return from >= 0 && T >= from * S ? kTwoPasses : 0;
 }
 

@@ -1041,21 +1041,28 @@ __global__ void __launch_bounds__(kThreads, 5) dw_sep_kernel_hi_occ(
 //  * groups of filter rows: as few as keep the accumulators in registers.
 //    FP32 K = 7 with three CTAs of 80 registers takes 2 (771; one group and two
 //    CTAs 877), unaligned, where two CTAs fit better, 1 (1016, against 1113).
-//  * rows per unrolled block of the dx and dw bodies, and whether blocks below
-//    the image are skipped (it costs registers where they are tight: BF16 K = 5
-//    542 -> 579, FP32 K = 7 771 -> 789, K = 9 1224 -> 1295 with 8-row dx
-//    blocks; it gains at odd heights).
+//  * rows per unrolled block of the dx and dw bodies, so that nothing to speak of
+//    spills: 8-row dx blocks cost BF16 K = 11 84 to 316 bytes at K = 13 and FP32 K
+//    = 13 156 (8 x 3 x 1024^2, 8 -> 4 rows: BF16 K = 11 278 -> 264, K = 13, with 8
+//    groups, 500 -> 343, K = 15 491 -> 428; FP32 K = 13 466 -> 389); and whether blocks
+//    below the image are skipped (it costs registers where they are tight: FP32
+//    K = 7 771 -> 789, K = 9 1224 -> 1295 with 8-row dx blocks; it gains at odd
+//    heights).
 //  * CTAs per SM: three where the registers allow, so that more loads are in
-//    flight (K = 3 304, against 368 with two).
+//    flight (K = 3 304, against 368 with two).  BF16 K = 5 spills 100 bytes with
+//    three: two are faster up to some 15 tiles per SM (512^2 9.8 -> 9.0), beyond 5
+//    of which the two passes are taken.
 template <int K, typename T, int AL>
 struct BwdTune {
   static constexpr bool F32 = sizeof(T) == 4;
   static constexpr int GROUPS =
-      K <= 5 ? 1 : (K == 7 ? (F32 && AL ? 2 : 1) : (K == 9 ? 2 : (K <= 13 ? 4 : 8)));
-  static constexpr int DX_ROWS = (K == 7 && F32) || K == 9 ? 4 : 8;
+      K <= 5 ? 1 : (K == 7 ? (F32 && AL ? 2 : 1)
+                           : (K == 9 ? 2 : (K == 11 || (K == 13 && F32) ? 4 : 8)));
+  static constexpr int DX_ROWS =
+      K <= 5 || (F32 ? K == 11 || K == 15 : K == 7) ? 8 : 4;
   static constexpr int DW_ROWS = K <= 3 || (K == 5 && !AL) || (K == 7 && !F32) ? 8 : 4;
   static constexpr bool SKIP = K <= 3 || (K == 5 && F32) || (K == 7 && !AL);
-  static constexpr int MIN_CTAS = K <= 3 || (AL && (K == 5 || (K == 7 && F32))) ? 3 : 2;
+  static constexpr int MIN_CTAS = K <= 3 || (AL && F32 && (K == 5 || K == 7)) ? 3 : 2;
 };
 
 template <int K, typename T, int AL>

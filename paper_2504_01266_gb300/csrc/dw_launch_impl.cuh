@@ -257,8 +257,11 @@ static cudaError_t filter_run(const DwArgs& a, const CUtensorMap& tmx, const CUt
 // K = 7 11.8 / 12.8; 8 x 3 x 1024 x 1021 K = 3 1.17 times as long; 4 x 3 x 1801 x
 // 2399 K = 1 0.89, K = 7 0.84, K = 13 0.93 times.
 template <int K>
+constexpr bool filter_wide_always() {
+  return K == 1 || K == 7 || K == 13;
+}
+template <int K>
 static bool filter_wide(const DwArgs& a) {
-  if (K == 1 || K == 7 || K == 13) return true;
   const int64_t tpp = ((a.W + kTileW - 1) / kTileW) * ((a.H + kFilterTileH - 1) / kFilterTileH);
   return has_odd_rows(2, a.W, a.x, a.dy) && tpp > 1 &&
          a.N * a.C * tpp <= 4 * (int64_t)sm_count();
@@ -270,9 +273,13 @@ static cudaError_t filter_impl(const DwArgs& a, const DwConfig& cfg, cudaStream_
   if (xdy_maps<T, K>(a, FilterShape<K, T, kAligned, false>::X_ROWS, kFilterTileH, kTileW, &tmx,
                      &tmdy))
     return filter_run<T, K, kAligned, false>(a, tmx, tmdy, cfg, st);
-  if constexpr (sizeof(T) == 2 && (K <= 7 || K == 13))
-    if (filter_wide<K>(a)) return filter_run<T, K, kAnyPlanes, true>(a, tmx, tmdy, cfg, st);
-  return filter_run<T, K, kAnyPlanes, false>(a, tmx, tmdy, cfg, st);
+  if constexpr (sizeof(T) == 2 && filter_wide_always<K>()) {
+    return filter_run<T, K, kAnyPlanes, true>(a, tmx, tmdy, cfg, st);
+  } else {
+    if constexpr (sizeof(T) == 2 && (K == 3 || K == 5))
+      if (filter_wide<K>(a)) return filter_run<T, K, kAnyPlanes, true>(a, tmx, tmdy, cfg, st);
+    return filter_run<T, K, kAnyPlanes, false>(a, tmx, tmdy, cfg, st);
+  }
 }
 
 template <int K>

@@ -163,7 +163,9 @@ __device__ __forceinline__ void finish_sums(const FinishArgs& p, double* red) {
   __syncthreads();
   if ((int)threadIdx.x < TB && tap < p.KK) {
     double sum = 0.0;
-    for (int w = 0; w < NT / 32; ++w) sum += red[w * TB + threadIdx.x];
+    // warps beyond the last row have nothing
+    const int warps = min(NT / 32, ((int)min(count, (uint32_t)NT) * TB + 31) / 32);
+    for (int w = 0; w < warps; ++w) sum += red[w * TB + threadIdx.x];
     p.dw[(int64_t)c * p.KK + tap] = (float)sum;
   }
 }
