@@ -99,10 +99,13 @@ static int auto_filter_tiles_per_chunk(const DwArgs& a, int max_tiles = 16) {
 // the terms of a chunk one after the other in FP32, 4 rows of every tile for K <=
 // 7, 8 for K = 11, 16 else.  No more tiles than keep that as short as four warps
 // of a fused kernel with the automatic chunks do: 16 rows for K <= 7, 32 for K = 9
-// and 11, 64 above.
+// and 11, 64 above; half as many for BF16 K <= 7, whose short chains are almost
+// exact, so that the FP32 sums over lanes and warps count (error of dw against
+// FP64, 16 x 8 x 512^2 K = 7: 1.11e-7 with four tiles, 1.02e-7 with two, 0.98e-7
+// the fused kernel with roles; 4 x 3 x 1024^2 67 -> 70 us).
 static int split_tiles_per_chunk(const DwArgs& a) {
-  return auto_filter_tiles_per_chunk(
-      a, std::min(16, (a.K == 9 ? 2 : 4) * auto_tiles_per_cta(a)));
+  const int per = a.K == 9 || (a.K <= 7 && a.dtype != 0) ? 2 : 4;
+  return auto_filter_tiles_per_chunk(a, std::min(16, per * auto_tiles_per_cta(a)));
 }
 
 DwConfig tune_config(int op, int id, const DwArgs& a) {

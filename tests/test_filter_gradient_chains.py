@@ -38,7 +38,7 @@ def test_filter_kernel_rows(giga, dtype, W, K, rows):
 @pytest.mark.parametrize("dtype,K,per_sm,tile", [
     (torch.float32, 3, 16, 1), (torch.float32, 3, 40, 1), (torch.bfloat16, 1, 4, 1),
     (torch.bfloat16, 3, 4, 1),
-    (torch.float32, 9, 4, 2), (torch.float32, 11, 4, 4), (torch.bfloat16, 7, 8, 4),
+    (torch.float32, 9, 4, 2), (torch.float32, 11, 4, 4), (torch.bfloat16, 7, 8, 2),
     (torch.float32, 13, 4, 4)])
 def test_both_gradients_tiles(giga, dtype, K, per_sm, tile):
     """Both gradients from the tile count on where the built-in choice leaves the
