@@ -155,8 +155,10 @@ constexpr int kTilePairs = 1, kTwoPasses = 5, kRing = 6;  // both gradients
 // storage type, the inputs' alignment and the number T of 64 x 128 tiles
 // against the S SMs (S = 152; times in us, candidate 0 -> the choice):
 //  * forward and input gradient, T <= 2 S: 32-row tiles, because 64-row tiles
-//    leave SMs with no CTA or one (512^2 K = 21: 24 -> 15, K = 31: 46 -> 26;
-//    3 x 300 x 401 K = 15: 19 -> 15; 3 x 1080 x 1920, T = 5 S: equal).
+//    leave SMs with no CTA or one (512^2 K = 21: 21.2 -> 12.0, K = 31: 43 -> 24;
+//    2 x 3 x 512^2 K = 15: 19 -> 16; 3 x 1080 x 1920, T = 5 S: equal), but for K >= 25,
+//    whose halo costs them most, where an SM then has twice as many all the same
+//    (3 x 512^2 K = 31: 43 -> 47).
 //    Above: the L2 prefetch where the tile load shows -- aligned FP32 K = 7, 9
 //    (16 x 3 x 2048^2: 380 -> 368, 573 -> 554) and BF16 K <= 3 (197 -> 179);
 //    FP32 K = 3 loses by it (230 -> 253), the others are equal.
@@ -190,7 +192,9 @@ int default_choice(int op, const DwArgs& a) {
   const bool f32 = a.dtype == 0, many = tpp > 1;  // many: a plane is more than one tile
   const bool aligned = inputs_aligned(a);
   if (op == TUNE_FWD || op == TUNE_BWD_INPUT) {
-    if (T <= 2 * S) return kTileRows32;
+    const int64_t T32 = a.N * a.C * ((a.W + kTileW - 1) / kTileW) * ((a.H + 31) / 32);
+    const bool rows32 = a.K < 25 || (T32 + S - 1) / S < 2 * ((T + S - 1) / S);
+    if (T <= 2 * S && rows32) return kTileRows32;
     return aligned && (f32 ? a.K == 7 || a.K == 9 : a.K <= 3) ? kPrefetch : 0;
   }
   if (op != TUNE_BWD_FUSED) return 0;

@@ -25,7 +25,8 @@ def desc(N, side, K, dtype=0, W=None):
 
 
 @pytest.mark.parametrize("args,op,want", [
-    ((1, 64, 7), FWD, 1), ((16, 2048, 7), FWD, 4), ((16, 2048, 5), FWD, 0),
+    ((1, 64, 7), FWD, 1), ((1, 512, 21), FWD, 1), ((1, 512, 31), FWD, 0), ((1, 64, 31), FWD, 1),
+    ((2, 512, 31), FWD, 1), ((16, 2048, 7), FWD, 4), ((16, 2048, 5), FWD, 0),
     ((16, 2048, 3, 1), FWD, 4), ((16, 2048, 3, 1, 2046), FWD, 0),
     ((1, 64, 3), BOTH, 0), ((4, 2048, 3), BOTH, 6), ((64, 2048, 3), BOTH, 1),
     ((4, 2048, 3, 0, 2046), BOTH, 0), ((16, 2048, 15), BOTH, 5), ((16, 2048, 7), BOTH, 0),
