@@ -203,7 +203,7 @@ __device__ __forceinline__ int row_is_odd(const T* row) {
 // image column tx0 - RP + c, for c < kTileW + RP + R.  BF16 rows that start off
 // a 4-byte boundary land one element to the right (shift_odd_rows).  Nothing
 // outside the rows is read.  Issues the copies, no commit.
-template <typename T, int NT>
+template <typename T, int NT, bool SMALL = true>
 __device__ __forceinline__ void stage_any(T* __restrict__ sm, const T* plane, int H, int W,
                                           int ty0, int tx0, int rows, int R, int RP, int pitch,
                                           int odd_rows) {
@@ -213,7 +213,7 @@ __device__ __forceinline__ void stage_any(T* __restrict__ sm, const T* plane, in
   const bool inside = j0 >= 1 && j0 + kTileW <= W;
   const T* row = plane + (int64_t)(ty0 - R + w0) * W;
   T* dst = sm + w0 * pitch;
-  if (ES == 4 && 2 * H < rows) {
+  if (SMALL && ES == 4 && 2 * H < rows) {
     // most rows lie outside the image: one store a lane for those (a loop of its
     // own, because the choice inside the other costs that one registers: 8 x 512
     // planes of 7 x 7, K = 3 34 -> 26 us; inside, W = 2399 K = 3 75 -> 77)
@@ -929,7 +929,10 @@ __device__ __forceinline__ void dw_sep_body(
     }
   } else {
     const T* xp = x + (int64_t)plane * H * W;
-    stage_any<T, kThreads>(staged, xp, H, W, ty0, tx0, S::ROWS, G::R, GS::RP, GS::SP, odd_rows);
+    // without the loop for small images, which costs this kernel registers (4 x 3 x
+    // 1801 x 2399 K = 15 with it 122 -> 124 us)
+    stage_any<T, kThreads, false>(staged, xp, H, W, ty0, tx0, S::ROWS, G::R, GS::RP, GS::SP,
+                                  odd_rows);
     cp_async_wait_all();
     if (odd_rows)
       shift_odd_rows<T, kThreads>(staged, xp, H, W, ty0, S::ROWS, G::R, GS::RP, GS::SP);
