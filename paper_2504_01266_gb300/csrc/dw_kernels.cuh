@@ -312,14 +312,16 @@ __host__ __device__ constexpr int shift_words(int R, int RP) { return (kTileW + 
 // BF16 rows that stage_any left one element to the right (row addresses that
 // are not multiples of 4: every second row when W is odd) move into place.
 // Every thread calls it once its own copies have landed; it begins with a CTA
-// barrier, and another must follow before the tile is read.
+// barrier (sync; a second tile whose copies had landed before the first one's
+// needs none), and another must follow before the tile is read.
 template <typename T, int NT>
 __device__ __forceinline__ void shift_odd_rows(T* __restrict__ sm, const T* plane, int H, int W,
-                                               int ty0, int rows, int R, int RP, int pitch) {
+                                               int ty0, int rows, int R, int RP, int pitch,
+                                               bool sync = true) {
   if constexpr (sizeof(T) == 2) {
     const int lane = threadIdx.x & 31;
     const int words = shift_words(R, RP);  // at most 80
-    cta_barrier();
+    if (sync) cta_barrier();
     for (int sr = threadIdx.x >> 5; sr < rows; sr += NT / 32) {
       const int gi = ty0 - R + sr;
       if (gi < 0 || gi >= H || !row_is_odd(plane + (int64_t)gi * W)) continue;
@@ -1165,7 +1167,7 @@ __global__ void __launch_bounds__(kThreads, BwdTune<K, T, AL>::MIN_CTAS)
       cp_async_wait_all();
       if (odd_rows) {
         shift_odd_rows<T, kThreads>(st_x, xp, H, W, ty0, S::ROWS, G::R, GS::RP, GS::SP);
-        shift_odd_rows<T, kThreads>(st_dy, dyp, H, W, ty0, S::ROWS, G::R, GS::RP, GS::SP);
+        shift_odd_rows<T, kThreads>(st_dy, dyp, H, W, ty0, S::ROWS, G::R, GS::RP, GS::SP, false);
       }
       cta_barrier();
     }
@@ -1432,7 +1434,7 @@ __global__ void __launch_bounds__(FilterShape<K, T, AL, WIDE>::NT, 1)
       int ty0, tx0;
       tile_origin(cs.t, ty0, tx0);
       shift_odd_rows<T, S::NT>(sx, x + off, H, W, ty0, S::X_ROWS, G::R, G::RP, G::SP);
-      shift_odd_rows<T, S::NT>(sdy, dy + off, H, W, ty0, kFilterTileH, 0, 0, S::DYP);
+      shift_odd_rows<T, S::NT>(sdy, dy + off, H, W, ty0, kFilterTileH, 0, 0, S::DYP, false);
     }
     cta_barrier();
     if (AL && *s_abort) break;
@@ -1659,7 +1661,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (!AL && odd_rows) {
       const int64_t off = (int64_t)plane * H * W;
       shift_odd_rows<T, S::NT>(sx, x + off, H, W, ty0, S::ROWS, G::R, G::RP, G::SP);
-      shift_odd_rows<T, S::NT>(sdy, dy + off, H, W, ty0, S::ROWS, G::R, G::RP, G::SP);
+      shift_odd_rows<T, S::NT>(sdy, dy + off, H, W, ty0, S::ROWS, G::R, G::RP, G::SP, false);
     }
     cta_barrier();
     if (AL && *s_abort) break;

@@ -101,7 +101,8 @@ struct RagLayout {
   // space: those are used at a chunk's end, behind barriers
   static constexpr int BUF = RED;
   static constexpr int INTS = RED + kRagWarps * kRowBuf;
-  static constexpr int SM_BYTES = INTS + 16;
+  static constexpr int IMAGE = INTS + 16;         // the current chunk's RagImage
+  static constexpr int SM_BYTES = IMAGE + (int)sizeof(RagImage);
   static_assert(RagShape<9, T>::AT * 9 <= RED_FLOATS && RagShape<11, T>::AT * 11 <= RED_FLOATS &&
                     RagShape<15, T>::AT * 15 <= RED_FLOATS && RED_FLOATS * 4 <= kRowBuf,
                 "reduction rows");
@@ -151,16 +152,18 @@ __device__ __forceinline__ void rag_stage(const RagParams& p, const RagChunk& ch
 // clamp border, folds the edges of dx.  It runs once per chunk, outside the
 // filter sizes' bodies (K known at run time): inlined into each of them the
 // sums cost the tile loops registers (seven K = 11 images 2.82 -> 2.91 ms).
+// `im` is the copy in shared memory that the chunk's start left there: the fence
+// empties L1, and two loads in a row from L2 are felt where a chunk is a small
+// image.
 template <typename T>
-__device__ __forceinline__ void rag_complete(const RagParams& p, int c, double* ps, int* s_flag) {
+__device__ __forceinline__ void rag_complete(const RagParams& p, int channel, const RagImage& im,
+                                             double* ps, int* s_flag) {
   const bool do_dw = p.ops & 4, folds = (p.ops & 2) && p.border == 1;
   if (do_dw || folds) {
-    __threadfence();
+    __threadfence();  // this thread's outputs and partials, before the count
     cta_barrier();
-    const RagChunk ch = p.chunks[c];
-    const RagImage im = p.images[ch.image];
     if (threadIdx.x == 0)
-      *s_flag = atomicAdd(p.counters + 1 + im.ic_base + ch.channel, 1) == im.nch - 1;
+      *s_flag = atomicAdd(p.counters + 1 + im.ic_base + channel, 1) == im.nch - 1;
     cta_barrier();
     if (*s_flag) {
       __threadfence();
@@ -168,8 +171,8 @@ __device__ __forceinline__ void rag_complete(const RagParams& p, int c, double* 
       if (do_dw) {
         // every tap's partials in FP64 by GR threads, each every GR-th chunk,
         // then their sums in order
-        const float* part = p.partials + im.partial_base + (int64_t)ch.channel * im.nch * KK;
-        const int GR = min(kRagThreads / KK, 16);
+        const float* part = p.partials + im.partial_base + (int64_t)channel * im.nch * KK;
+        const int GR = min(min(kRagThreads / KK, 16), im.nch);
         const int k = threadIdx.x % KK, q = threadIdx.x / KK;
         if (q < GR) {
           double s = 0.0;
@@ -181,14 +184,14 @@ __device__ __forceinline__ void rag_complete(const RagParams& p, int c, double* 
         if (threadIdx.x < KK) {
           double s = 0.0;
           for (int g = 0; g < GR; ++g) s += ps[g * KK + threadIdx.x];
-          im.dw[(int64_t)ch.channel * KK + threadIdx.x] = (float)s;
+          im.dw[(int64_t)channel * KK + threadIdx.x] = (float)s;
         }
       }
       if (folds) {
-        const int64_t off = (int64_t)ch.channel * im.H * im.W;
+        const int64_t off = (int64_t)channel * im.H * im.W;
         const int64_t edges = edge_pixels(im.H, im.W);
         for (int64_t e = threadIdx.x; e < edges; e += kRagThreads)
-          fold_edge_pixel<T>(static_cast<const T*>(im.dy) + off, im.w + (int64_t)ch.channel * KK,
+          fold_edge_pixel<T>(static_cast<const T*>(im.dy) + off, im.w + (int64_t)channel * KK,
                              static_cast<T*>(im.dx) + off, im.H, im.W, K, e);
       }
     }
@@ -248,7 +251,7 @@ __device__ __forceinline__ int rag_chunk(const RagParams& p, const RagChunk& ch,
                                        G::R, G::RP, G::SP);
       if (do_dx || do_dw)
         shift_odd_rows<T, kRagThreads>(sdy, static_cast<const T*>(im.dy) + off, H, W, ty0,
-                                       S::ROWS, G::R, G::RP, G::SP);
+                                       S::ROWS, G::R, G::RP, G::SP, !(do_fwd || do_dw));
     }
     cta_barrier();
     if (clamp && (do_fwd || do_dw) &&
@@ -303,7 +306,6 @@ __device__ __forceinline__ int rag_chunk(const RagParams& p, const RagChunk& ch,
       part_c[(int64_t)j * KK + k] = sum;
     }
   }
-  __threadfence();  // before the completion count that follows the caller's next barrier
   return sb;
 }
 
@@ -332,6 +334,8 @@ __global__ void __launch_bounds__(kRagThreads, 1) rag_kernel(RagParams p) {
     const int cn = *s_next;
     const RagChunk ch = p.chunks[c];
     const RagImage im = p.images[ch.image];
+    RagImage* s_im = reinterpret_cast<RagImage*>(sm + L::IMAGE);
+    if (threadIdx.x == 0) *s_im = im;  // read behind rag_chunk's barriers
     switch (im.K) {
       case 1: sb = rag_chunk<T, 1>(p, ch, im, cn, sm, sb, fb); break;
       case 3: sb = rag_chunk<T, 3>(p, ch, im, cn, sm, sb, fb); break;
@@ -342,7 +346,7 @@ __global__ void __launch_bounds__(kRagThreads, 1) rag_kernel(RagParams p) {
       case 13: sb = rag_chunk<T, 13>(p, ch, im, cn, sm, sb, fb); break;
       default: sb = rag_chunk<T, 15>(p, ch, im, cn, sm, sb, fb); break;
     }
-    rag_complete<T>(p, c, reinterpret_cast<double*>(sm + L::RED), s_flag);
+    rag_complete<T>(p, ch.channel, *s_im, reinterpret_cast<double*>(sm + L::RED), s_flag);
     if (cn >= p.n_chunks) break;
     c = cn;
     fb ^= 1;
