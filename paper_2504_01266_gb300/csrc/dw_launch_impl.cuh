@@ -250,7 +250,7 @@ static cudaError_t filter_run(const DwArgs& a, const CUtensorMap& tmx, const CUt
 
 // BF16 planes that TMA cannot load, where 16 warps beat 8 or 12: staging them
 // takes the warps longer than a small filter does (K = 1; K = 3, 5 with rows to be
-// shifted and few tiles: from about 5 S on, and for planes of one tile, the
+// shifted and few tiles: from some 10 S on, and for planes of one tile, the
 // 16 warps' 4-row blocks cost more than they save), at K = 7 the two accumulators
 // leave 8 warps per SM, and at K = 13 they are a little better.  16 warps against
 // 8 / 12 (us): 3 x 3 x 257 x 251 K = 1 7.6 / 10.1, K = 3 8.3 / 9.9, K = 5 10.4 / 12.2,
@@ -264,7 +264,7 @@ template <int K>
 static bool filter_wide(const DwArgs& a) {
   const int64_t tpp = ((a.W + kTileW - 1) / kTileW) * ((a.H + kFilterTileH - 1) / kFilterTileH);
   return has_odd_rows(2, a.W, a.x, a.dy) && tpp > 1 &&
-         a.N * a.C * tpp <= 4 * (int64_t)sm_count();
+         a.N * a.C * tpp <= 6 * (int64_t)sm_count();
 }
 
 template <typename T, int K>

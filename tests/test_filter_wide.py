@@ -23,9 +23,9 @@ def giga():
 @pytest.mark.parametrize("H,W,offset,extra", [(65, 127, 0, 0), (65, 127, 0, 1), (64, 125, 0, 0),
                                               (65, 126, 0, 0), (65, 128, 4, 0), (3, 131, 0, 1)])
 def test_bf16(giga, K, H, W, offset, extra):
-    """Planes of two tiles (one: 64 x 125), in all 4 tiles per SM or just more."""
+    """Planes of two tiles (one: 64 x 125), in all 6 tiles per SM or just more."""
     tpp = -(-H // 64) * -(-W // 128)
-    planes = 4 * torch.cuda.get_device_properties(0).multi_processor_count // tpp + extra
+    planes = 6 * torch.cuda.get_device_properties(0).multi_processor_count // tpp + extra
     border = oracle.CLAMP if K % 4 == 1 else oracle.ZERO
     gen = torch.Generator().manual_seed(K + W)
     x = torch.rand((planes, 1, H, W), generator=gen).bfloat16()
