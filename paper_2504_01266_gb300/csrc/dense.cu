@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1)
 // the last one, so the pair (last slot, slot 0) is adjacent too.  D
 // accumulates in TMEM over all chunks of the CTA (2 x 192 columns); each CTA
 // then writes its FP32 partial sums [tap][c][o] and a second kernel adds the
-// CTAs' partials in FP64 in a fixed order.
+// CTAs' partials, at least as exactly as FP64, in a fixed order.
 constexpr int kWgTileP = 64;                           // pixel positions per chunk (MMA K: 4 x 16)
 constexpr int kWgXPx = kWgTileP + 1;                   // x band: 65 pixels
 constexpr int kWgDyPx = kWgTileP + 2;                  // dy band: 66 pixels
@@ -687,10 +687,39 @@ __global__ void __launch_bounds__(kDenseThreads, 1)
   }
 }
 
-// dw[o][a][b][c] = sum over CTAs (FP64, in a fixed order) of
-// partial[cta][3a + b][c][o].  A block takes one (tap, c): 64 lanes across o read
-// whole lines of a partial, four groups of them take every fourth CTA, and the
-// groups add up.  22 MB of partials come from L2 whatever the image size.
+// A running sum in three floats, at least as good as FP64's.  s is the rounded
+// sum; Knuth's TwoSum gives what each addition to it rounds away exactly; these
+// remainders are summed in e the same way, and what that rounds away in f, the
+// only sum that loses anything.  With u = 2^-24, n terms and S the sum of their
+// magnitudes, the remainders are at most u S each and n u S together, those of
+// e at most n u^2 S each, and f errs by at most n u times n of these, n^3 2^-72 S:
+// for n <= 724 no more than the n 2^-53 S of n FP64 additions (the kernel below
+// has n <= 64).  Where the terms and sums fit 53 bits, so that FP64 is exact, e
+// and f are too.  Thirteen FP32 instructions a term, where FP64 takes a
+// conversion and an addition on a unit of about two lanes a clock and SM.
+// Not for sums that are not finite on the way: see the caller.
+struct ThreeFloatSum {
+  float s = 0.f, e = 0.f, f = 0.f;
+  // sum += x; returns what the addition rounded away
+  static __device__ __forceinline__ float two_sum(float& sum, float x) {
+    const float t = __fadd_rn(sum, x);
+    const float z = __fadd_rn(t, -sum);
+    const float r = __fadd_rn(__fadd_rn(sum, -__fadd_rn(t, -z)), __fadd_rn(x, -z));
+    sum = t;
+    return r;
+  }
+  __device__ __forceinline__ void add(float x) {
+    f = __fadd_rn(f, two_sum(e, two_sum(s, x)));
+  }
+  __device__ __forceinline__ double value() const { return (double)s + ((double)e + (double)f); }
+};
+
+// dw[o][a][b][c] = sum over CTAs, in a fixed order, of partial[cta][3a + b][c][o].
+// A block takes one (tap, c): 64 lanes across o read whole lines of a partial,
+// four groups of them take every fourth CTA in a ThreeFloatSum, and the groups
+// add up in FP64.  22 MB of partials come from L2 whatever the image size; all
+// in FP64 the additions take about 22 us, thus 7 (1 x 64 x 64 pixels, the whole
+// filter gradient: 30.1 -> 15.5 us).
 constexpr int kWgFinGroups = 4;
 __global__ void __launch_bounds__(kDenseC * kWgFinGroups)
     dense_wgrad_finalize_kernel(const float* __restrict__ partials, int ctas,
@@ -699,9 +728,14 @@ __global__ void __launch_bounds__(kDenseC * kWgFinGroups)
   const int o = threadIdx.x % kDenseC, g = threadIdx.x / kDenseC;
   const int tap = blockIdx.x / kDenseC, c = blockIdx.x % kDenseC;
   const float* src = partials + ((int64_t)tap * kDenseC + c) * kDenseC + o;
-  double s = 0.0;
+  ThreeFloatSum sum;
 #pragma unroll 8
-  for (int b = g; b < ctas; b += kWgFinGroups) s += (double)__ldg(src + (int64_t)b * kWgPartialFloats);
+  for (int b = g; b < ctas; b += kWgFinGroups) sum.add(__ldg(src + (int64_t)b * kWgPartialFloats));
+  double s = sum.value();
+  if (!isfinite(s)) {  // infinities, NaN or an overflow on the way
+    s = 0.0;
+    for (int b = g; b < ctas; b += kWgFinGroups) s += (double)__ldg(src + (int64_t)b * kWgPartialFloats);
+  }
   part[g][o] = s;
   __syncthreads();
   if (g == 0) {
