@@ -17,13 +17,14 @@
 //    out-of-image part arrives as zeros: the zero border; under the clamp
 //    border the edge tiles are then fixed in shared memory by clamp_fix);
 //    other inputs are staged by every thread's cp.async copies (stage_any) to
-//    the same layout.  The kernels are compiled once for each: the aligned one
-//    keeps the registers and instructions that the other spends on staging and
-//    on rows that cannot be stored in whole chunks.  Either way the compute
-//    loops never branch on coordinates.  BF16 is widened to FP32 once per staged tile (forward and
-//    fused backward) or when a row enters registers.  The column halo is
-//    rounded up to 16 bytes of elements so every staged row stays 16-byte
-//    aligned (TMA's rule for the x coordinate).
+//    the same layout.  The kernels are compiled for each alignment (kAnyPlanes
+//    ..): the aligned one keeps the registers and instructions that the others
+//    spend on staging and on rows that cannot be stored in whole chunks.  Either
+//    way the compute loops never branch on coordinates.  BF16 is widened to FP32
+//    once per staged tile (forward and fused backward) or when a row enters
+//    registers.  The column halo is rounded up to 16 bytes of elements: a tiled
+//    TMA load has to start on a 16-byte boundary of the row (an x coordinate off
+//    one, which nothing checks beforehand, raises an illegal-instruction error).
 //  * Each lane owns 4 adjacent output columns and PY rows.  The filter is
 //    consumed A rows at a time with those A rows held in registers; every
 //    staged input row is read once per group with 128-bit shared loads and
@@ -43,8 +44,8 @@
 namespace giga {
 
 // Column halo of a K x K filter for elements of ES bytes: r rounded up to 16
-// bytes of elements (4 FP32, 8 BF16), so a staged row starts 16-byte aligned
-// in memory (TMA's rule for the x coordinate) and in shared memory.
+// bytes of elements (4 FP32, 8 BF16), so a staged row starts 16-byte aligned in
+// memory, as a tiled TMA load must, and in shared memory.
 __host__ __device__ constexpr int geo_rp(int K, int ES) {
   return ES == 2 ? ((K - 1) / 2 + 7) / 8 * 8 : ((K - 1) / 2 + 3) / 4 * 4;
 }
@@ -162,17 +163,16 @@ template <> struct Tile<__nv_bfloat16> {
 // one, two or four copies (FP32) and about ten integer instructions; the few
 // columns right of them are copied for all rows together.  What bounds the
 // unaligned passes at small K is the instructions and the load/store slots
-// they take: a lane per 4-element chunk with four 4-byte copies (the former
-// scheme) took about 40 instructions a chunk and touched 16 sectors and a
-// quarter of the banks per copy; 16-byte copies of the row's aligned chunks
-// followed by a shift inside shared memory took about 65 instructions a row.
-// Pixels outside the image arrive as zeros; the clamp border is clamp_fix's.
-// With store_rows, 4 x 3 x 1801 x 2399, zero border, former scheme -> this one
-// (W = 2400, staged by TMA, beside it), us:
-//   FP32 K = 3 forward 112 -> 79 (65), both gradients 204 -> 166 (124),
-//        separable 115 -> 89 (65); K = 7 165 -> 136 (112), 369 -> 304 (243)
-//   BF16 K = 3 forward 135 -> 101 (58), both gradients 293 -> 252 (121),
-//        separable 124 -> 107 (63); K = 7 203 -> 163 (112), 501 -> 447 (274)
+// they take: a lane per 4-element chunk with four 4-byte copies takes about 40
+// instructions a chunk, 16-byte copies of the row's aligned chunks with a shift
+// inside shared memory about 65 a row.  Pixels outside the image arrive as
+// zeros; the clamp border is clamp_fix's.
+// 4 x 3 x 1801 x 2399, zero border, a lane per chunk with scalar stores -> rows by
+// warps with store_rows (W = 2400, staged by TMA, beside it), us:
+//   FP32 K = 3 forward 109 -> 75 (63), both gradients 199 -> 156 (105),
+//        separable 112 -> 88 (62); K = 7 162 -> 131 (103), 363 -> 302 (232)
+//   BF16 K = 3 forward 132 -> 99 (51), both gradients 287 -> 225 (83),
+//        separable 121 -> 102 (59); K = 7 200 -> 160 (108), 497 -> 413 (240)
 
 // `odd_rows` of the general kernels: some BF16 row of one of the planes starts
 // off a 4-byte boundary, so shift_odd_rows has work.
@@ -1037,9 +1037,9 @@ __global__ void __launch_bounds__(kThreads, 5) dw_sep_kernel_hi_occ(
 // split into groups of filter rows and tile rows, then write g (= dx for the
 // zero border) from the dy tile, 8 rows each, so every warp has the same work
 // between a tile's barriers.  (With 4 warps for each gradient the slower role's
-// warps ran alone at a tile's end: 4 x 3 x 1801 x 2400 K = 5 161 -> 150 us, K =
-// 15 1140 -> 860; 4 x 3 x 1801 x 2399 K = 5 227 -> 206, K = 9 442 -> 413, BF16
-// K = 9 672 -> 571.)  A CTA owns `tpc` consecutive 64 x
+// warps ran alone at a tile's end: 4 x 3 x 1801 x 2400 K = 5 161 -> 148 us, K =
+// 15 1140 -> 863; 4 x 3 x 1801 x 2399 K = 5 227 -> 205, K = 9 442 -> 417, BF16
+// K = 9 672 -> 542.)  A CTA owns `tpc` consecutive 64 x
 // 128 tiles of one plane and writes one K*K vector of FP32 partial sums to
 // partials[blockIdx.x].  Aligned planes are staged by two TMA loads per tile
 // (zeros outside the image), others by stage_any; under the clamp border the x
@@ -1242,15 +1242,15 @@ __global__ void __launch_bounds__(kThreads, BwdTune<K, T, AL>::MIN_CTAS)
 // ------------------------------------------------------- filter gradient
 // The filter gradient alone (Eq. 3's adjoint with respect to the filter):
 // dw[c][a][b] = sum over n, i, j of dy[n][c][i][j] * xs[n][c][i + a - r][j + b - r],
-// xs the border-extended input.  One CTA of 8 or 12 warps per SM, persistent over
+// xs the border-extended input.  One CTA of 8, 12 or 16 warps per SM, persistent over
 // chunks of `tpc` consecutive 64 x 128 tiles of one plane (chunk q runs on
 // CTA q mod gridDim.x).  NS shared-memory stages hold {x tile with halo, dy
 // tile}; the copies of the tile NS - 1 items ahead are in flight while the
-// current one is reduced, across chunk boundaries too.  For FP32 rows with a
-// 16-byte stride a stage is filled by two TMA tensor loads issued by one
-// thread (out-of-image reads arrive as zeros: the zero border; under the
-// clamp border the edge tiles then get clamp_fix); otherwise by every
-// thread's cp.async copies with the border applied.  Tap rows are split into GT groups; warp w takes group w / WPG and
+// current one is reduced, across chunk boundaries too.  Planes on 16-byte
+// boundaries, FP32 or BF16, are loaded by two TMA loads per stage that one thread
+// issues, others by stage_any; either way pixels outside the image arrive
+// as zeros (the zero border), and under the clamp border the edge tiles then
+// get clamp_fix.  Tap rows are split into GT groups; warp w takes group w / WPG and
 // tile rows part w mod WPG, so each of the SM's four schedulers (w mod 4)
 // holds one warp of every group.  At the end of a chunk the warps' sums
 // (fixed butterfly order) and then the group's warps (fixed order) give the
@@ -1263,10 +1263,10 @@ static_assert(kFilterTileH == kBwdTileH, "both filter-gradient kernels share the
 // into 8-row dy blocks: 14 x rows per block instead of the 20 that two 4-row
 // blocks take, and that shared-memory traffic was what 16 warps of 4 rows
 // waited for.  16 x 3 x 2048^2, 16 warps -> 8 warps (us), FP32 / BF16: K = 5
-// 281 -> 253 / 300 -> 233, K = 7 458 -> 412 / 488 -> 447.  From K = 9 on, 12
-// warps in 3 groups (up to 168 registers): K = 9 with 8-row blocks 658 -> 638 /
-// 701 -> 664, K = 11 948 -> 935 / 1013 -> 1009, K = 13 1235 -> 1240 / 1488 ->
-// 1379 against 16 warps; 8-row blocks lose at K >= 11 (K = 11 1077, K = 15
+// 297 -> 251 / 306 -> 237, K = 7 457 -> 414 / 484 -> 447.  From K = 9 on, 12
+// warps in 3 groups (up to 168 registers): K = 9 with 8-row blocks 662 -> 639 /
+// 701 -> 666, K = 11 972 -> 932 / 1061 -> 1021, K = 13 1252 -> 1234 / 1426 ->
+// 1389 against 16 warps; 8-row blocks lose at K >= 11 (K = 11 1077, K = 15
 // 1536 -> 1737).  WIDE: 16 warps of 4-row blocks, for the BF16 planes that
 // dw_launch_impl.cuh picks (filter_wide).
 template <int K, bool WIDE>

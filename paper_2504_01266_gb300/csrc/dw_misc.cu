@@ -98,11 +98,11 @@ __global__ void dw_fixup_kernel(const T* __restrict__ dy, const float* __restric
 // has none): the filter gradient's sums, the fold of NT / 2 pixels of the
 // first and last row or column of a plane, and the fold of a plane's corner
 // pixels, which both folds touch.  All are short and bound by latency, so they
-// run beside each other instead of one after the other.  4 x 3 x 1801 x 2399,
-// K = 3: 4.4 (rows) + 6.7 (columns) + 13.8 us (sums, a warp per tap striding
-// over the partials, uncoalesced) as three launches, 6.1 us as one; K = 15,
-// 8 x 3 x 1024^2: 52 -> 12.9 us; BF16 K = 9, 4 x 3 x 1800 x 2400: 60 (the
-// pixel-by-pixel fold 45 of it) -> 10.7 us; 4 x 3 x 257 x 251: 10.5 -> 4.3 us.
+// run beside each other instead of one after the other.  As launches of their
+// own -> one launch with FP64 sums (this one profiled, with cold caches), us:
+// 4 x 3 x 1801 x 2399, K = 3 24.9 (rows 4.4, columns 6.7, sums 13.8) -> 8.4;
+// 8 x 3 x 1024^2, K = 15 52 -> 14.6; BF16 K = 9, 4 x 3 x 1800 x 2400 60 (a fold pixel
+// by pixel 45 of it) -> 12.3; 4 x 3 x 257 x 251, K = 3 10.5 -> 7.6.
 //
 // NT is 512, or 128 (finish_small) where the planes' edges or the partial sums
 // are so few that most of 512 threads would idle.

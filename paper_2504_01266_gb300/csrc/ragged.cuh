@@ -13,10 +13,10 @@
 //    three cost the same per pixel, so every warp has the same work between
 //    the tile's barriers, and a scheduler has four busy warps throughout.
 //    (With fixed roles -- 4 warps forward, 4 input gradient, 4 or 8 filter
-//    gradient -- the warps of the slowest role ran alone at a tile's end, and 4
-//    of the 16 idled for K <= 9.  One 3 x 2001 x 2999 image, that -> this: K = 3
-//    155 -> 109 us, K = 5 184 -> 137, K = 9 301 -> 258, K = 11 380 -> 333, BF16 K = 3
-//    224 -> 129, K = 11 472 -> 397; forward alone K = 11 165 -> 126.)
+//    gradient -- the warps of the slowest role run alone at a tile's end, and 4
+//    of the 16 idle for K <= 9.  One 3 x 2001 x 2999 image, zero border, that ->
+//    this: K = 3 155 -> 109 us, K = 11 380 -> 333, BF16 K = 3 224 -> 129, K = 11 472 ->
+//    397; forward alone, clamp border, K = 3 72 -> 53, K = 11 168 -> 131.)
 //  * each chunk writes one K*K vector of FP32 filter-gradient partials; the
 //    CTA that completes the last chunk of an (image, channel) -- detected with
 //    a per-(image, channel) atomic counter after a memory fence -- sums that

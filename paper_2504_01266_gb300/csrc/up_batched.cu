@@ -109,10 +109,11 @@ __device__ __forceinline__ void up_rag_body(const UpRagParams& p) {
 }
 
 // CTAs per SM that the kernel is compiled for (0: left to the compiler), where
-// one more than the compiler's choice fits without a spill and pays (17 images
-// of 64 to 704 pixels a side, us): K = 5 five CTAs of 48 registers, FP32 54.5 ->
-// 52.1, BF16 62.5 -> 61.8; K = 11 four of 64, FP32 113.6 -> 112.2, BF16 395.8 ->
-// 393.5; K = 13, 15 FP32 as the single-image kernel.  K = 9 takes four by itself.
+// one more than the compiler's own choice fits without a spill and pays (17
+// images of 64 to 704 pixels a side, compiler's choice / stated, us): K = 5 five
+// CTAs of 48 registers, FP32 54.5 / 52.1, BF16 62.5 / 61.8; K = 11 four of 64, FP32
+// 113.6 / 112.2, BF16 395.8 / 393.5; K = 13, 15 FP32 as the single-image kernel.
+// K = 9 takes four by itself.
 template <typename T, int K>
 constexpr int up_rag_min_ctas() {
   return K == 5 ? 5 : (K == 11 || (K > 11 && sizeof(T) == 4) ? 4 : 0);
